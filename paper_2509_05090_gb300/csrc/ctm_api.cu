@@ -79,6 +79,19 @@ std::vector<Shape> step_shapes(const ctm_ctx *c)
             {chi * chi, D2, D2 * D2}, {chi * chi, D2 * D2, D2}, {chi, n, n}};
 }
 
+// Slices of the contraction engine in this context's own precision: n_split, or those of
+// the FP64 contractions that run on the tensor cores; 0: none do.
+static int engine_slices(const ctm_ctx *c) { return c->split_T > 0 ? c->split_T : c->f64_T; }
+
+// CTM_FP64: whether any of the step's contractions gains from the tensor cores
+static int f64_slices(const ctm_ctx *c)
+{
+    if (c->cfg.precision != CTM_FP64) return 0;
+    for (const auto &sh : step_shapes(c))
+        if (split_f64_pays(sh.M, sh.N, sh.K)) return SPLIT_F64_T;
+    return 0;
+}
+
 // Carve the workspace.  With base == nullptr only the size is computed.
 size_t layout(ctm_ctx *c, char *base)
 {
@@ -132,6 +145,7 @@ size_t layout(ctm_ctx *c, char *base)
     need(chi * chi, d * d * D2, D2 * D2);
     c->splitk_elems = sk;
     c->splitk = td((long long)sk + 1);
+    c->splitk_c = td((long long)sk + 1);
     c->qr_sbuf = td((long long)qr_scratch_doubles((int)chi));
     c->qr_rowbuf = td((long long)qr_rowbuf_doubles((int)chi));
     c->qr_wy = td((long long)qr_wy_doubles((int)n, (int)chi));
@@ -194,7 +208,8 @@ size_t layout(ctm_ctx *c, char *base)
         c->sw_e.Apk = (unsigned char *)take(ap);
         c->sw_e.eA = (int *)take(sizeof(int) * (size_t)ecap);
     }
-    if (c->split_T > 0) {
+    const int eng_T = engine_slices(c);
+    if (eng_T > 0) {
         // packed digit slices, exponents and the split-K integer accumulator for the
         // largest operand of the step's contractions
         size_t ap = 0, bp = 0, pp = 0;
@@ -204,7 +219,8 @@ size_t layout(ctm_ctx *c, char *base)
         shapes.push_back({(int)n, (int)n, (int)chi});
         shapes.push_back({(int)(chi * chi), (int)(d * d * D2), (int)(D2 * D2)});
         for (const auto &sh : shapes) {
-            SplitPlan pl = split_plan_caps(sh.M, sh.N, sh.K, c->split_T);
+            if (c->f64_T > 0 && !split_f64_pays(sh.M, sh.N, sh.K)) continue;
+            SplitPlan pl = split_plan_caps(sh.M, sh.N, sh.K, eng_T);
             if (pl.a_pack_bytes > ap) ap = pl.a_pack_bytes;
             if (pl.b_pack_bytes > bp) bp = pl.b_pack_bytes;
             if (pl.partial_bytes > pp) pp = pl.partial_bytes;
@@ -232,7 +248,7 @@ size_t layout(ctm_ctx *c, char *base)
         c->sw_e.eA = (int *)take(sizeof(int) * (size_t)ecap);
         const Shape ash[2] = {{(int)(chi * chi), (int)D2, (int)(D2 * D2)}, {(int)(chi * chi), (int)(D2 * D2), (int)D2}};
         for (int sl = 0; sl < 2; ++sl) {
-            SplitPlan pl = split_plan_caps(ash[sl].M, ash[sl].N, ash[sl].K, c->split_T);
+            SplitPlan pl = split_plan_caps(ash[sl].M, ash[sl].N, ash[sl].K, eng_T);
             c->apk[sl] = (unsigned char *)take(pl.b_pack_bytes);
             c->apk_cap[sl] = pl.b_pack_bytes;
             c->ape[sl] = (int *)take(sizeof(int) * (size_t)ash[sl].N);
@@ -241,7 +257,7 @@ size_t layout(ctm_ctx *c, char *base)
         // A packs kept for a second contraction: T (n x chi) and Q^T (chi x n)
         const Shape csh[2] = {{(int)n, (int)chi, (int)chi}, {(int)chi, (int)chi, (int)n}};
         for (int sl = 0; sl < 2; ++sl) {
-            SplitPlan pl = split_plan_caps(csh[sl].M, csh[sl].N, csh[sl].K, c->split_T);
+            SplitPlan pl = split_plan_caps(csh[sl].M, csh[sl].N, csh[sl].K, eng_T);
             c->ack[sl] = (unsigned char *)take(pl.a_pack_bytes);
             c->ack_cap[sl] = pl.a_pack_bytes;
             c->ace[sl] = (int *)take(sizeof(int) * (size_t)csh[sl].M);
@@ -273,7 +289,8 @@ bool config_ok(const ctm_config *cfg)
     return true;
 }
 
-// The step's contractions: FP64 GEMM, or the split-BF16 tcgen05 engine.
+// The step's contractions: the split-BF16 tcgen05 engine (in FP64 with SPLIT_F64_T slices,
+// for the shapes that gain from it), the TF32 engine, or the FP64 pipe's GEMM.
 cudaError_t run_gemm(ctm_ctx *c, const GemmF64 &g, int hint, int lane)
 {
     cudaEvent_t *ev = nullptr;
@@ -281,11 +298,14 @@ cudaError_t run_gemm(ctm_ctx *c, const GemmF64 &g, int hint, int lane)
         ev = c->prof_ev + c->prof_n;
         c->prof_n += 3;
     }
-    if (c->tf32_T > 0) {
-        const SplitWork &w = lane == 1 ? c->sw_c : (lane == 2 ? c->sw_e : c->sw);
-        return gemm_tf32(g, c->tf32_T, w, lane == 1 ? c->lane2 : c->stream, ev);
-    }
-    if (c->split_T > 0) {
+    cudaStream_t lst = lane == 1 ? c->lane2 : c->stream;
+    const SplitWork &lw = lane == 1 ? c->sw_c : (lane == 2 ? c->sw_e : c->sw);
+    if (c->tf32_T > 0) return gemm_tf32(g, c->tf32_T, lw, lst, ev);
+    const int T = c->split_T > 0 ? c->split_T
+                  : c->f64_T > 0 && split_f64_pays(g.M, g.N, g.K) && split_fits(g.M, g.N, g.K, c->f64_T, lw)
+                      ? c->f64_T
+                      : 0;
+    if (T > 0) {
         SplitOpts o{};
         if (hint == GEMM_REUSE_A) o.reuse_a = 1;
         if (hint == GEMM_B_IS_A_LZ || hint == GEMM_B_IS_A_ZX) {
@@ -305,17 +325,17 @@ cudaError_t run_gemm(ctm_ctx *c, const GemmF64 &g, int hint, int lane)
             o.a_fill = use ? 0 : 1;
             if (!use) fill_slot = slot;
         }
-        const SplitWork &w = lane == 1 ? c->sw_c : (lane == 2 ? c->sw_e : c->sw);
-        cudaError_t e = gemm_split(g, c->split_T, w, lane == 1 ? c->lane2 : c->stream, ev, &o);
+        cudaError_t e = gemm_split(g, T, lw, lst, ev, &o);
         if (fill_slot >= 0) c->ack_valid[fill_slot] = (e == cudaSuccess);
         return e;
     }
     if (ev) {
-        cudaEventRecord(ev[2], c->stream);   // no pre-pass in FP64
-        cudaEventRecord(ev[0], c->stream);
+        cudaEventRecord(ev[2], lst);   // no pre-pass
+        cudaEventRecord(ev[0], lst);
     }
-    cudaError_t e = gemm_f64(g, gemm_f64_pick_split(g.M, g.N, g.K), c->splitk, c->splitk_elems, c->stream);
-    if (ev) cudaEventRecord(ev[1], c->stream);
+    cudaError_t e = gemm_f64(g, gemm_f64_pick_split(g.M, g.N, g.K), lane == 1 ? c->splitk_c : c->splitk,
+                             c->splitk_elems, lst);
+    if (ev) cudaEventRecord(ev[1], lst);
     return e;
 }
 
@@ -361,26 +381,34 @@ int enqueue_projector(ctm_ctx *c, double *Qout)
     const long long n = c->n;
     cudaStream_t st = c->stream;
     c->ack_valid[1] = 0;   // the QR below writes a new Q
-    CK(launch_warm_start((int)n, chi, c->Q, c->C, c->Qs, st));
-    GemmF64 g{(int)n, chi, (int)n, c->M, idx_lin(n), idx_lin(1), c->Qs, idx_lin(chi), idx_lin(1),
-              c->Y, idx_lin(chi), idx_lin(1), 1.0, 0.0};
-    CK(run_gemm(c, g));
+    if (c->q_unit && c->cfg.precision == CTM_FP64) {
+        // M times unit columns is a selection of M's columns: exact to the last bit, which the
+        // slices' row grids are not for elements far below their row's largest
+        CK(launch_select_columns((int)n, chi, c->M, c->C, c->Y, st));
+        c->m_packed = 0;
+    } else {
+        CK(launch_warm_start((int)n, chi, c->Q, c->C, c->Qs, st));
+        GemmF64 g{(int)n, chi, (int)n, c->M, idx_lin(n), idx_lin(1), c->Qs, idx_lin(chi), idx_lin(1),
+                  c->Y, idx_lin(chi), idx_lin(1), 1.0, 0.0};
+        CK(run_gemm(c, g));
+        c->m_packed = 1;
+    }
     QrScratch qs = qr_scratch(c);
     CK(qr_householder((int)n, chi, c->Y, Qout, c->R, qs, st));
     return CTM_OK;
 }
 
 // Fig. 3(a): Cout = sym(Qp^T M Qp) / |.|_F.
-// lane 1 (split mode): on lane2, with the corner lane's work buffers.
+// lane 1: on lane2, with the corner lane's work buffers.
 int enqueue_corner(ctm_ctx *c, const double *Qp, double *Cout, int lane = 0)
 {
     const int chi = c->chi;
     const long long n = c->n;
     cudaStream_t st = lane == 1 ? c->lane2 : c->stream;
-    // the previous split contraction was Y = M Qs (only the QR in between): M is already packed
+    // after Y = M Qs (only the QR in between) M is already packed
     GemmF64 g{(int)n, chi, (int)n, c->M, idx_lin(n), idx_lin(1), Qp, idx_lin(chi), idx_lin(1),
               c->MQ, idx_lin(chi), idx_lin(1), 1.0, 0.0};
-    CK(run_gemm(c, g, GEMM_REUSE_A, lane));
+    CK(run_gemm(c, g, c->m_packed ? GEMM_REUSE_A : GEMM_PLAIN, lane));
     g = GemmF64{chi, chi, (int)n, Qp, idx_lin(1), idx_lin(chi), c->MQ, idx_lin(chi), idx_lin(1),
                 c->Cr, idx_lin(chi), idx_lin(1), 1.0, 0.0};
     CK(run_gemm(c, g, (Qp == c->Qn || Qp == c->Q) ? GEMM_A_FILL_Q : GEMM_PLAIN, lane));
@@ -399,7 +427,7 @@ int enqueue_corner_from_r(ctm_ctx *c, double *Cout)
 }
 
 // Fig. 3(b): T'[i,x,j] = sum Q[(a,y),i] T[a,u,g] a[u,w,z] a[z,x,y] Q[(g,w),j], normalised.
-// lane 2 (split mode): with the edge lane's work buffers, concurrent with a corner
+// lane 2: with the edge lane's work buffers, concurrent with a corner
 // update on lane2; the last contraction waits for it (it uses the corner's pack of Q^T).
 int enqueue_edge(ctm_ctx *c, const double *Qp, double *Tout, int lane = 0)
 {
@@ -452,14 +480,14 @@ int enqueue_step(ctm_ctx *c)
         CK(cudaEventRecord(c->ev_join, c->side));
         c->side_pending = 1;
     }
-    // Split mode after the first step (whose eager contractions time their plans
+    // After the first step (whose eager contractions time their plans
     // one at a time): the corner and edge updates both need only Q, so the corner
     // update runs on lane2 beside the edge update.  This path also writes the new
     // environment in place: C, T and Q are not read after the QR except by their
     // own updates (the warm start and the enlarged corner come before it; the edge
     // update reads T in its first contraction, before its last one writes T'), so
     // no hand-over copies are needed.
-    const bool lanes = (c->split_T > 0 || c->tf32_T > 0) && c->steps_done > 0 && c->cfg.corner_mode == 0;
+    const bool lanes = c->steps_done > 0 && c->cfg.corner_mode == 0;
     if ((rc = enqueue_enlarged_corner(c)) != CTM_OK) return rc;
     if ((rc = enqueue_projector(c, lanes ? c->Q : c->Qn)) != CTM_OK) return rc;
     if (lanes) {
@@ -496,6 +524,7 @@ int enqueue_step(ctm_ctx *c)
     CK(cudaMemcpyAsync(c->C, c->Cn, sizeof(double) * chi * chi, cudaMemcpyDeviceToDevice, st));
     CK(cudaMemcpyAsync(c->T, c->Tn, sizeof(double) * chi * D2 * chi, cudaMemcpyDeviceToDevice, st));
     CK(cudaMemcpyAsync(c->Q, c->Qn, sizeof(double) * n * chi, cudaMemcpyDeviceToDevice, st));
+    c->q_unit = 0;
     if (c->spec_skip) return CTM_OK;
     CK(cudaEventRecord(c->ev_fork, st));
     CK(cudaStreamWaitEvent(c->side, c->ev_fork, 0));
@@ -531,6 +560,8 @@ int enqueue_step_profiled(ctm_ctx *c, cudaEvent_t *ev)
         GemmF64 g{(int)n, (int)chi, (int)n, c->M, idx_lin(n), idx_lin(1), c->Qs, idx_lin(chi), idx_lin(1),
                   c->Y, idx_lin(chi), idx_lin(1), 1.0, 0.0};
         CK(run_gemm(c, g));
+        c->m_packed = 1;
+        c->q_unit = 0;
     }
     CK(cudaEventRecord(ev[2], st));
     {
@@ -846,6 +877,7 @@ size_t ctm_workspace_bytes(const ctm_config *cfg)
     c.n = (long long)c.chi * c.D2;
     c.split_T = (cfg->precision == CTM_SPLIT_BF16) ? cfg->n_split : 0;
     c.tf32_T = tf32_slices(cfg->precision);
+    c.f64_T = f64_slices(&c);
     c.qr_force_slab = qr_force_slab_from_env();
     return layout(&c, nullptr);
 }
@@ -871,7 +903,9 @@ int ctm_init(const ctm_config *cfg, const double *A_dev, void *workspace, size_t
     c->n = (long long)c->chi * c->D2;
     c->split_T = (cfg->precision == CTM_SPLIT_BF16) ? cfg->n_split : 0;
     c->tf32_T = tf32_slices(cfg->precision);
+    c->f64_T = f64_slices(c);
     c->qr_rows_min = 1;
+    c->q_unit = 1;
     c->qr_force_slab = qr_force_slab_from_env();
     c->stream = (cudaStream_t)stream;
     if (!qr_supported((int)c->n, c->chi)) {
@@ -1086,6 +1120,7 @@ int ctm_set_env(ctm_ctx *c, const double *C_dev, const double *T_dev, const doub
     if (join_side(c) != CTM_OK) return CTM_ECUDA;
     const long long chi = c->chi, D2 = c->D2, n = c->n;
     cudaStream_t st = c->stream;
+    c->q_unit = 0;
     CK(cudaMemcpyAsync(c->C, C_dev, sizeof(double) * chi * chi, cudaMemcpyDeviceToDevice, st));
     CK(cudaMemcpyAsync(c->T, T_dev, sizeof(double) * chi * D2 * chi, cudaMemcpyDeviceToDevice, st));
     CK(cudaMemcpyAsync(c->Q, Q_dev, sizeof(double) * n * chi, cudaMemcpyDeviceToDevice, st));

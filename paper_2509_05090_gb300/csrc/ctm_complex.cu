@@ -30,6 +30,7 @@ struct ctm_complex_ctx {
     long long n;
     int split_T;
     int tf32_T;   // 1, 2: TF32 products (CTM_FP32_TF32, CTM_SPLIT_TF32)
+    int f64_T;    // SPLIT_F64_T where CTM_FP64 products run on the tensor cores, else 0
     cudaStream_t stream;
     double U[3][3][2];      // the rotation paired with the leg cycle (energies of the x, y bonds)
     // planes: P_* is the plane stride of each tensor (elements)
@@ -857,10 +858,14 @@ struct ZGemm {
 int real_gemm(ctm_complex_ctx *c, const GemmF64 &g, int reuse_a)
 {
     if (c->tf32_T > 0) return gemm_tf32(g, c->tf32_T, c->sw, c->stream, nullptr) == cudaSuccess ? CTM_OK : CTM_ECUDA;
-    if (c->split_T > 0) {
+    const int T = c->split_T > 0 ? c->split_T
+                  : c->f64_T > 0 && split_f64_pays(g.M, g.N, g.K) && split_fits(g.M, g.N, g.K, c->f64_T, c->sw)
+                      ? c->f64_T
+                      : 0;
+    if (T > 0) {
         SplitOpts o{};
         o.reuse_a = reuse_a;
-        return gemm_split(g, c->split_T, c->sw, c->stream, nullptr, &o) == cudaSuccess ? CTM_OK : CTM_ECUDA;
+        return gemm_split(g, T, c->sw, c->stream, nullptr, &o) == cudaSuccess ? CTM_OK : CTM_ECUDA;
     }
     return gemm_f64(g, gemm_f64_pick_split(g.M, g.N, g.K), c->splitk, c->splitk_elems, c->stream) == cudaSuccess
                ? CTM_OK
@@ -933,6 +938,15 @@ std::vector<std::array<int, 3>> zshapes(const ctm_complex_ctx *c)
     return {{n, chi, 2 * chi},          {n, n, 2 * chi},          {chi * chi, D2, 2 * D2 * D2},
             {chi * chi, D2 * D2, 2 * D2}, {n, chi, 2 * n},          {chi, chi, 2 * n},
             {n, chi, 2 * chi},          {chi, chi, 2 * chi},      {chi * chi, dd * D2, 2 * D2 * D2}};
+}
+
+// CTM_FP64: whether any product gains from the tensor cores
+int zf64_slices(const ctm_complex_ctx *c)
+{
+    if (c->cfg.precision != CTM_FP64) return 0;
+    for (const auto &sh : zshapes(c))
+        if (split_f64_pays(sh[0], sh[1], sh[2])) return SPLIT_F64_T;
+    return 0;
 }
 
 size_t zlayout(ctm_complex_ctx *c, char *base)
@@ -1015,12 +1029,13 @@ size_t zlayout(ctm_complex_ctx *c, char *base)
     c->rho_raw = td(2 * dd * dd);
     c->hrot = td(3 * 2 * dd * dd);
     c->eout = td(4 + 2 * dd * dd);
-    if (c->split_T > 0 || c->tf32_T > 0) {
+    if (c->split_T > 0 || c->tf32_T > 0 || c->f64_T > 0) {
         size_t ap = 0, bp = 0, pp = 0;
         long long ecap = 0;
         for (const auto &sh : zshapes(c)) {
+            if (c->f64_T > 0 && !split_f64_pays(sh[0], sh[1], sh[2])) continue;
             SplitPlan pl = c->tf32_T > 0 ? tf32_plan_caps(sh[0], sh[1], sh[2], c->tf32_T)
-                                         : split_plan_caps(sh[0], sh[1], sh[2], c->split_T);
+                                         : split_plan_caps(sh[0], sh[1], sh[2], c->f64_T > 0 ? c->f64_T : c->split_T);
             if (pl.a_pack_bytes > ap) ap = pl.a_pack_bytes;
             if (pl.b_pack_bytes > bp) bp = pl.b_pack_bytes;
             if (pl.partial_bytes > pp) pp = pl.partial_bytes;
@@ -1359,6 +1374,7 @@ size_t ctm_complex_workspace_bytes(const ctm_config *cfg, int irrep)
     c.n = (long long)c.chi * c.D2;
     c.split_T = cfg->precision == CTM_SPLIT_BF16 ? cfg->n_split : 0;
     c.tf32_T = cfg->precision == CTM_SPLIT_TF32 ? 2 : (cfg->precision == CTM_FP32_TF32 ? 1 : 0);
+    c.f64_T = zf64_slices(&c);
     return zlayout(&c, nullptr);
 }
 
@@ -1382,6 +1398,7 @@ int ctm_complex_init(const ctm_config *cfg, int irrep, const double *A_dev, void
     c->n = (long long)c->chi * c->D2;
     c->split_T = cfg->precision == CTM_SPLIT_BF16 ? cfg->n_split : 0;
     c->tf32_T = cfg->precision == CTM_SPLIT_TF32 ? 2 : (cfg->precision == CTM_FP32_TF32 ? 1 : 0);
+    c->f64_T = zf64_slices(c);
     c->stream = (cudaStream_t)stream;
     if (ws_bytes < zlayout(c, nullptr)) {
         delete c;

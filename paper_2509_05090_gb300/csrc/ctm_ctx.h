@@ -17,7 +17,7 @@ struct ctm_ctx {
     cudaEvent_t ev_in, ev_out;
     cudaStream_t side;        // corner spectrum runs here, overlapped with the edge update
     cudaEvent_t ev_fork, ev_join;
-    // split mode: the corner update (M Q, Q^T (M Q), normalisation) runs on lane2
+    // after the first step: the corner update (M Q, Q^T (M Q), normalisation) runs on lane2
     // while the edge update runs on the step's stream; ev_q = Q is ready,
     // ev_corner = the corner update (and its pack of Q^T) is done
     cudaStream_t lane2;
@@ -25,16 +25,18 @@ struct ctm_ctx {
     // FP64 buffers (device, inside the caller's workspace)
     double *Araw, *A, *a;
     double *C, *Cn, *Cr;
-    double *Cspec;            // split mode: the copy of C' the side-stream spectrum reads
+    double *Cspec;            // the copy of C' the side-stream spectrum reads
     double *T, *Tn;
     double *Q, *Qn, *Qs, *Y, *W, *MQ;
     double *R;
     double *M, *X, *H;
     double *Y1;
     double *s, *s_new, *delta, *spec_work;
-    double *splitk;
+    double *splitk, *splitk_c;   // split-K partials of the FP64 GEMM: the step's stream, the corner lane
     size_t splitk_elems;
     int split_T;              // 0: FP64 contractions; 2..5: split-BF16 slices per operand
+    int f64_T;                // SPLIT_F64_T where the FP64 contractions that gain from it run on the tensor
+                              // cores (CTM_FP64 contexts with such shapes), else 0
     int tf32_T;               // 1, 2: TF32 slices per operand (FP32_TF32, SPLIT_TF32); 0 otherwise
     SplitWork sw;
     SplitWork sw_c;           // corner lane: M's pack read from sw; own B pack, exponents, split-K buffer
@@ -95,6 +97,8 @@ struct ctm_ctx {
     int force_timeout;        // ctm_debug_force_timeout: the QR grid barrier waits for an arrival that never comes
     cudaEvent_t prof_ev[CTM_PROF_EVENTS];   // three per contraction: kernel start, kernel end, pre-pass start
     int steps_done;
+    int q_unit;               // Q is still the initial projector, the first chi columns of I_n
+    int m_packed;             // M's packed slices (of Y = M Qs) are in sw's A buffer
 };
 
 namespace ctmi {

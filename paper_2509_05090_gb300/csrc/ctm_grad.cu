@@ -17,6 +17,10 @@
 #include <math.h>
 #include <string.h>
 
+#include <algorithm>
+#include <array>
+#include <vector>
+
 #include "ctm_ctx.h"
 
 namespace {
@@ -275,8 +279,18 @@ struct GradBufs {
     double *rawb, *scal, *part;
     double *sk;                                       // split-K partials of the adjoint GEMMs
     size_t sk_elems;
+    SplitWork sw;                                     // packs of the adjoint products on the tensor cores
     size_t ck_stride;
 };
+
+// (M, N, K) of the recomputed step's, the energy's and the adjoint's products, as issued below
+std::vector<std::array<long long, 3>> grad_shapes(const ctm_ctx *c)
+{
+    const long long chi = c->chi, D2 = c->D2, n = c->n, dd = (long long)c->d * c->d, c2 = chi * chi, DD = D2 * D2;
+    return {{n, chi, chi}, {n, n, chi},  {c2, D2, DD},      {c2, DD, D2},      {n, chi, n},       {chi, chi, n},
+            {chi, n, n},   {D2, DD, c2}, {DD, D2, c2},      {c2, DD, dd * D2}, {dd * D2, DD, c2}, {DD, dd * D2, c2},
+            {c2, dd * D2, DD}};
+}
 
 size_t grad_layout(const ctm_ctx *c, int k, GradBufs *g, char *base)
 {
@@ -334,6 +348,28 @@ size_t grad_layout(const ctm_ctx *c, int k, GradBufs *g, char *base)
     if (ske < (1LL << 20)) ske = 1LL << 20;
     b.sk = td(ske);
     b.sk_elems = (size_t)ske;
+    size_t ap = 0, bp = 0, pp = 0;
+    long long ecap = 0;
+    for (const auto &s : grad_shapes(c)) {
+        if (!split_f64_pays((int)s[0], (int)s[1], (int)s[2])) continue;
+        const SplitPlan pl = split_plan_caps((int)s[0], (int)s[1], (int)s[2], SPLIT_F64_T);
+        ap = std::max(ap, pl.a_pack_bytes);
+        bp = std::max(bp, pl.b_pack_bytes);
+        pp = std::max(pp, pl.partial_bytes);
+        ecap = std::max(ecap, std::max(s[0], s[1]));
+    }
+    auto bytes = [&](size_t count) { return (unsigned char *)td((long long)((count + 7) / 8)); };
+    b.sw.Apk = bytes(ap);
+    b.sw.Bpk = bytes(bp);
+    b.sw.a_pack_cap = ap;
+    b.sw.b_pack_cap = bp;
+    b.sw.eA = (int *)bytes(sizeof(int) * (size_t)ecap);
+    b.sw.eB = (int *)bytes(sizeof(int) * (size_t)ecap);
+    b.sw.e_cap = (int)ecap;
+    b.sw.partial = bytes(pp);
+    b.sw.partial_cap = pp;
+    b.sw.err = c->err;
+    b.sw.autotune = 1;
     if (g) *g = b;
     return off;
 }
@@ -344,7 +380,8 @@ size_t grad_layout(const ctm_ctx *c, int k, GradBufs *g, char *base)
         if (_e != cudaSuccess) return CTM_ECUDA; \
     } while (0)
 
-// C(m,n) = alpha A(m,k) B(k,n) + beta C(m,n), FP64
+// C(m,n) = alpha A(m,k) B(k,n) + beta C(m,n), FP64: on the tensor cores where the shape gains
+// from it, as in a CTM_FP64 context's step
 struct G64 {
     ctm_ctx *c;
     const GradBufs *b;
@@ -352,6 +389,8 @@ struct G64 {
                            double *C, Idx2 Cm, Idx2 Cn, double alpha = 1.0, double beta = 0.0) const
     {
         GemmF64 g{M, N, K, A, Am, Ak, B, Bk, Bn, C, Cm, Cn, alpha, beta};
+        if (split_f64_pays(M, N, K) && split_fits(M, N, K, SPLIT_F64_T, b->sw))
+            return gemm_split(g, SPLIT_F64_T, b->sw, c->stream, nullptr);
         return gemm_f64(g, gemm_f64_pick_split(M, N, K), b->sk, b->sk_elems, c->stream);
     }
 };

@@ -78,7 +78,15 @@ struct SplitOpts {
 };
 // Largest pack / accumulator sizes over every plan the autotuner may pick.
 SplitPlan split_plan_caps(int M, int N, int K, int T);
-int split_supported_T(int T);
+int split_supported_T(int T);   // the slice counts a caller may choose (n_split)
+// Slices of the FP64 contractions (CTM_FP64 contexts and the adjoint) where they run on the
+// tensor cores: 62-bit operand grids, eight exact levels, one rounding of the result.  alpha
+// and beta may be any; rows and columns with infinities or NaNs take the plain FP64 sum.
+constexpr int SPLIT_F64_T = 8;
+// Whether a CTM_FP64 contraction of this shape runs there (else the FP64 pipe's GEMM), and
+// whether its packs fit the work buffers.
+bool split_f64_pays(int M, int N, int K);
+bool split_fits(int M, int N, int K, int T, const SplitWork &w);
 cudaError_t split_prepare();
 // ev (may be null): three events, recorded around the contraction kernel (ev[0] before,
 // ev[1] after) and before its operand pre-pass (ev[2]).
@@ -165,6 +173,8 @@ cudaError_t launch_c3v_project_normalize(int d, int D, const double *Ain, double
                                          cudaStream_t st);
 cudaError_t launch_double_layer(int d, int D, const double *K, const double *B, double *a, cudaStream_t st);
 cudaError_t launch_init_env(int chi, int D, const double *a, double *C, double *T, double *Q, cudaStream_t st);
+// Y[r][j] = sgn(C_jj) M[r][j], j < chi: M Q S for the initial projector Q = first chi columns of I
+cudaError_t launch_select_columns(int n, int chi, const double *M, const double *C, double *Y, cudaStream_t st);
 cudaError_t launch_warm_start(int n, int chi, const double *Q, const double *C, double *Qs, cudaStream_t st);
 // partials: CORNER_NORM_BLOCKS doubles of scratch
 constexpr int CORNER_NORM_BLOCKS = 64;

@@ -20,6 +20,23 @@
 // 8 (T-1)): the int64 -> FP64 conversion instruction and an exact shift of the
 // exponent field.
 //
+// FP64 slices (T = SPLIT_F64_T = 8).  CTM_FP64 contractions run here too where the shape
+// gains from it: GB300's FP64 pipe does 1.25 TFLOP/s, its BF16 tensor cores 1900, and 36
+// slice products per FP64 product still leave a factor of 40 between them.  The grids have
+// P = 62 bits (a value within 2^-9 of its row's largest keeps all 53), the chunks are 128
+// deep so that all eight levels are exact integers in FP32, the levels go into two int64
+// sums 2^32 apart, and the only rounding after the grids is the result's own.  What is lost
+// is products of elements far below their row's and column's largest: the error is below
+// (K 2^-61 + 2^-53 |C|) in units of (row max) (column max), where the FP64 sum's grows like
+// K 2^-53 sum |a b|.  Measured against 128-bit sums (2-norm over the output): 3e-17 to 6e-17
+// at every shape and for normal, uniform, graded and constant operands, the FP64 GEMM 1e-16
+// to 2e-15.  Rows and columns with infinities or NaNs have no grid; their outputs are the
+// plain FP64 sums.  Against the FP64 pipe's GEMM: 8192 x 8192 x 128 14.07 -> 1.11 ms,
+// 8192 x 128 x 8192 14.28 -> 0.95 ms, 2592 x 2592 x 72 848 -> 146 us, 2592 x 72 x 2592
+// 934 -> 141 us, 900 x 900 x 36 72 -> 34 us; below MNK = 8e6 (512 x 512 x 32: 27 against
+// 28 us, 243 x 243 x 27: 14 against 29) the two packs and three launches cost more than
+// the FP64 GEMM, which keeps those shapes (split_f64_pays).
+//
 // Kernel.  Tile 128 x NT (NT = 64 or 96), K staged 64 at a time; one MMA covers up to
 // 256 / NT slice pairs (N = up to 256), since narrow MMAs run far below the tensor peak.  The slicing
 // pre-pass writes each operand tile in the exact shared-memory image the MMA
@@ -41,21 +58,34 @@ namespace {
 
 constexpr int SP_BM = 128;       // tile rows = TMEM lanes
 constexpr int SP_BK = 64;        // K per packed tile (128-byte rows)
-constexpr int SP_KT_PER_CHUNK = 4;   // 4 x 64 = 256 K per exact chunk
 constexpr int SP_BSLOTS = 2;     // B ring: all T slices of a K tile per slot
+// K tiles per chunk.  T <= 5: 256 K, so that levels 0 .. 3 are exact (the last one is far
+// below the result's accuracy).  FP64 slices (T = 8): 128 K, so that all eight are: a
+// level-t accumulator stays below (t + 1) 2^14 128 <= 2^24 in magnitude.
+__host__ __device__ constexpr int sp_chunk_kt(int T) { return T > 5 ? 2 : 4; }
+// Fraction bits of the top digit: 7, or 6 where the biased word would pass 64 bits (T = 8)
+__host__ __device__ constexpr int sp_top_bits(int T) { return T == 8 ? 6 : 7; }
+// FP64 slices: the level sums do not fit one int64 (2^(12 + 56) K), so levels 0 .. 3 and
+// 4 .. 7 have an accumulator each, 2^32 apart
+__host__ __device__ constexpr bool sp_wide(int T) { return T > 5; }
 // Per tile width: A-slice ring depth (the next K tile's slices in flight while the
 // current one is multiplied, within 227 KB with T = 5 B slices x 2), epilogue warps
 // (four or two per TMEM sub-partition), TMEM columns (T NT <= the allocation) and
 // CTAs per SM.  NT = 48 is the two-CTAs-per-SM shape: 256 TMEM columns and ~109 KB
 // of shared memory each, so one CTA's epilogue overlaps the other's loads and MMAs.
+// T = 8 takes NT = 32 (256 TMEM columns, 97 KB, two CTAs per SM) or NT = 64.
+constexpr int sp_aslots(int nt, int T)
+{
+    return T == 8 ? (nt == 32 ? 2 : 6) : nt == 96 ? 6 : (nt == 64 ? 8 : 3);
+}
 template <int NT>
 struct SpCfg {
-    static constexpr int ASLOTS = NT == 96 ? 6 : (NT == 64 ? 8 : 3);
-    static constexpr int EPI_WARPS = NT == 48 ? 8 : 16;
+    static constexpr bool TWO = NT <= 48;   // two CTAs per SM
+    static constexpr int EPI_WARPS = TWO ? 8 : 16;
     static constexpr int EPI_THREADS = 32 * EPI_WARPS;
     static constexpr int THREADS = 64 + EPI_THREADS;   // producers, MMA issuer, epilogue
-    static constexpr int TMEM_COLS = NT == 48 ? 256 : 512;
-    static constexpr int MIN_BLOCKS = NT == 48 ? 2 : 1;
+    static constexpr int TMEM_COLS = TWO ? 256 : 512;
+    static constexpr int MIN_BLOCKS = TWO ? 2 : 1;
 };
 // The deep-ring variant of the 48-wide tile (plan code SP_DEEP_CODE): one CTA per SM
 // whose A ring takes the shared memory a second CTA would have used, so a K-heavy
@@ -135,15 +165,22 @@ __global__ void split_colexp_kernel(int R, int K, const double *X, long long kst
 // repeatedly taking the balanced low byte and shifting.
 template <int T>
 struct SplitDigits {
-    static constexpr int P = 7 + 8 * (T - 1);
-    static constexpr unsigned long long B = 128ULL * (((1ULL << (8 * T)) - 1) / 255);
+    static constexpr int P = sp_top_bits(T) + 8 * (T - 1);
+    static constexpr int PRE = P > 52 ? P - 52 : 0;   // grids finer than the mantissa: it is shifted up first
+    static constexpr unsigned long long B = 0x8080808080808080ULL >> (64 - 8 * T);
 };
 
 // Right shift, less one guard bit, that puts a value of biased exponent field ex
 // on the grid of a row with exponent E: x = mant 2^(ex - 1075), so
 // F = round(x 2^(P - E)) = ((mant >> sh) + 1) >> 1 with sh = rs - ex,
-// rs = E + 1074 - P (rounding half up on the magnitude).
-__device__ __forceinline__ int grid_shift(int E, int P) { return E + 1074 - P; }
+// rs = E + 1074 - P (rounding half up on the magnitude).  For P > 52 the mantissa is
+// shifted up by PRE = P - 52 bits first and rs is larger by as much (sh >= 0 for every
+// value of the row, and PRE + 53 <= 63 bits).
+template <int T>
+__device__ __forceinline__ int grid_shift(int E)
+{
+    return E + 1074 - SplitDigits<T>::P + SplitDigits<T>::PRE;
+}
 
 // G = F + B of one value from its IEEE fields, integer operations only.  Zero
 // and subnormal values (far below any row grid) give F = 0, as do values more
@@ -155,7 +192,7 @@ __device__ __forceinline__ unsigned long long biased_fixed(double x, int rs)
     const unsigned long long b = (unsigned long long)__double_as_longlong(x);
     const int ex = (int)(b >> 52) & 0x7FF;
     const int sh = rs - ex;
-    const unsigned long long mant = (b & 0xFFFFFFFFFFFFFULL) | (1ULL << 52);
+    const unsigned long long mant = ((b & 0xFFFFFFFFFFFFFULL) | (1ULL << 52)) << SplitDigits<T>::PRE;
     unsigned long long F = ((mant >> (sh & 63)) + 1) >> 1;
     if (ex == 0 || (unsigned)sh > 63u) F = 0;
     const unsigned long long m = (unsigned long long)((long long)b >> 63);   // all ones if negative
@@ -179,7 +216,9 @@ template <int T>
 __device__ __forceinline__ float slice_digit(unsigned long long G, int t)
 {
     if (t == 0) return __uint_as_float(0x4B000000u + (uint32_t)(G >> (8 * (T - 1)))) - 8388736.0f;
-    return __uint_as_float(__byte_perm((uint32_t)G, 0x4B000000u, 0x7650u | (unsigned)(T - 1 - t))) - 8388736.0f;
+    const int byte = T - 1 - t;
+    const uint32_t w = byte < 4 ? (uint32_t)G : (uint32_t)(G >> 32);
+    return __uint_as_float(__byte_perm(w, 0x4B000000u, 0x7650u | (unsigned)(byte & 3))) - 8388736.0f;
 }
 
 // Slices of 8 consecutive-K values: slice t's 16-byte chunk goes to base + t * slice_bytes.
@@ -196,15 +235,15 @@ __device__ __forceinline__ void write_digit_chunks(const unsigned long long *G, 
     }
 }
 
-// Pack T digit slices of X (R x K via maps) into [T][rowTiles][kTiles][rowsT x 64] swizzled tiles.
+// Pack T digit slices of X (R x K via maps) into [rowTiles][kTiles][T][rowsT x 64] swizzled tiles (a
+// tile's slices adjacent, so that all T of a B tile move in one copy).
 // One thread per (row, 8-wide K chunk): it writes one 16-byte chunk per slice.
 template <int T>
 __global__ void split_pack_kernel(int R, int K, int rowsT, int rowTiles, int kTiles, const double *X, Idx2 rmap,
                                   Idx2 kmap, const int *e, unsigned char *out)
 {
     const long long units = (long long)rowTiles * rowsT * kTiles * 8;
-    const long long tile_bytes = (long long)rowsT * SP_BK * 2;
-    const long long slice_bytes = tile_bytes * rowTiles * kTiles;
+    const long long slice_bytes = (long long)rowsT * SP_BK * 2, tile_bytes = slice_bytes * T;
     for (long long u = blockIdx.x * (long long)blockDim.x + threadIdx.x; u < units;
          u += (long long)gridDim.x * blockDim.x) {
         const int c8 = (int)(u % (kTiles * 8));
@@ -212,7 +251,7 @@ __global__ void split_pack_kernel(int R, int K, int rowsT, int rowTiles, int kTi
         const int k0 = c8 * 8;
         unsigned long long G[8];
         if (r < R) {
-            const int rs = grid_shift(exp_of_word(e[r]), SplitDigits<T>::P);
+            const int rs = grid_shift<T>(exp_of_word(e[r]));
             const long long ro = off2(rmap, r);
 #pragma unroll
             for (int q = 0; q < 8; ++q) {
@@ -235,13 +274,12 @@ __global__ void split_pack_kernel(int R, int K, int rowsT, int rowTiles, int kTi
 // tile count are written as zero digits.
 template <int T>
 __global__ void __launch_bounds__(256) split_rowpack_kernel(int R, int K, int rowsT, int rowsTotal, int kTiles,
-                                                            const double *X, Idx2 rmap, int *e, unsigned char *out,
-                                                            long long slice_bytes)
+                                                            const double *X, Idx2 rmap, int *e, unsigned char *out)
 {
     const int r = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int lane = threadIdx.x & 31;
     if (r >= rowsTotal) return;
-    const long long tile_bytes = (long long)rowsT * SP_BK * 2;
+    const long long slice_bytes = (long long)rowsT * SP_BK * 2, tile_bytes = slice_bytes * T;
     unsigned char *row_base = out + (long long)(r / rowsT) * kTiles * tile_bytes;
     unsigned long long G[8];
     if (r < R) {
@@ -258,7 +296,7 @@ __global__ void __launch_bounds__(256) split_rowpack_kernel(int R, int K, int ro
         unsigned m = max(max(m0, m1), max(m2, m3));
         for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
         if (lane == 0) e[r] = (int)m;
-        const int rs = grid_shift(exp_of_word((int)m), SplitDigits<T>::P);
+        const int rs = grid_shift<T>(exp_of_word((int)m));
         for (int c8 = lane; c8 < kTiles * 8; c8 += 32) {
             const int k0 = c8 * 8;
 #pragma unroll
@@ -288,7 +326,7 @@ __global__ void __launch_bounds__(256) split_rowpack_kernel(int R, int K, int ro
 template <int NV, int T>
 __global__ void __launch_bounds__(512, 1) split_rowpack_reg_kernel(int R, int K, int rowsT, int rowsTotal, int kTiles,
                                                                 int WPR, const double *X, Idx2 rmap, int *e,
-                                                                unsigned char *out, long long slice_bytes)
+                                                                unsigned char *out)
 {
     __shared__ unsigned s_m[16];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -313,8 +351,8 @@ __global__ void __launch_bounds__(512, 1) split_rowpack_reg_kernel(int R, int K,
     m = 0;
     for (int i = 0; i < WPR; ++i) m = max(m, s_m[g * WPR + i]);
     if (live && w == 0 && lane == 0) e[r] = (int)m;
-    const int rs = grid_shift(exp_of_word((int)m), SplitDigits<T>::P);
-    const long long tile_bytes = (long long)rowsT * SP_BK * 2;
+    const int rs = grid_shift<T>(exp_of_word((int)m));
+    const long long slice_bytes = (long long)rowsT * SP_BK * 2, tile_bytes = slice_bytes * T;
     unsigned char *row_base = out + (long long)(r / rowsT) * kTiles * tile_bytes + sw128_off(r % rowsT, 2 * lane);
 #pragma unroll
     for (int j = 0; j < NV; ++j) {
@@ -336,14 +374,14 @@ __global__ void __launch_bounds__(512, 1) split_rowpack_reg_kernel(int R, int K,
 template <int T>
 __global__ void __launch_bounds__(256) split_pack_t_kernel(int R, int K, int rowsT, int rowsTotal, int kTiles,
                                                            const double *X, long long kstride, const int *e,
-                                                           unsigned char *out, long long slice_bytes)
+                                                           unsigned char *out)
 {
     __shared__ unsigned long long Gs[32][SP_BK + 1];
     const int r0 = blockIdx.x * 32, kt = blockIdx.y;
     {
         const int r = threadIdx.x & 31, kg = threadIdx.x >> 5;
         const int gr = r0 + r;
-        const int rs = grid_shift(gr < R ? exp_of_word(e[gr]) : 0, SplitDigits<T>::P);
+        const int rs = grid_shift<T>(gr < R ? exp_of_word(e[gr]) : 0);
 #pragma unroll
         for (int q = 0; q < 8; ++q) {
             const int kl = kg * 8 + q, k = kt * SP_BK + kl;
@@ -358,7 +396,8 @@ __global__ void __launch_bounds__(256) split_pack_t_kernel(int R, int K, int row
 #pragma unroll
     for (int q = 0; q < 8; ++q) G[q] = Gs[r][c8 * 8 + q];
     const long long tile = (long long)(gr / rowsT) * kTiles + kt;
-    write_digit_chunks<T>(G, out + tile * ((long long)rowsT * SP_BK * 2) + sw128_off(gr % rowsT, c8 * 8), slice_bytes);
+    const long long slice_bytes = (long long)rowsT * SP_BK * 2;
+    write_digit_chunks<T>(G, out + tile * (slice_bytes * T) + sw128_off(gr % rowsT, c8 * 8), slice_bytes);
 }
 
 // ---------------------------------------------------------------- PTX wrappers
@@ -449,6 +488,33 @@ __device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t *r)
 }
 __device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 
+// acc_hi 2^32 + acc_lo (the FP64 slices' level sums, in units of the last level) as the nearest
+// double: the sum's leading 63 bits (all of them unless it is longer) in one int64 and one
+// conversion -- GB300's FP64 pipe also runs the conversions, so a second one and an FMA would
+// cost as much again per element.
+__device__ __forceinline__ double wide_to_double(long long hi, long long lo)
+{
+    hi += lo >> 32;                                          // carry: lo keeps 32 unsigned bits
+    const unsigned l = (unsigned)lo;
+    const unsigned long long mag = (unsigned long long)(hi ^ (hi >> 63));
+    int s = __clzll((long long)mag) - 1;                     // free bits above hi's value
+    s = s > 32 ? 32 : s;
+    const long long S = (hi << s) | (long long)(s == 0 ? 0u : (l >> (32 - s)));
+    const double d = __ll2double_rn(S);
+    const int w = __double2hiint(d);
+    return S == 0 ? 0.0 : __hiloint2double(w + ((32 - s) << 20), __double2loint(d));
+}
+
+// d 2^scale on the exponent field, flushed to zero below the normal range, infinite above it
+__device__ __forceinline__ double scale_exponent(double d, int scale)
+{
+    const int hi = __double2hiint(d), lo = __double2loint(d);
+    const int be = ((hi >> 20) & 0x7FF) + scale;
+    if (((hi & 0x7FFFFFFF) | lo) == 0 || be <= 0) return 0.0;
+    if (be >= 2047) return __hiloint2double((hi & (int)0x80000000) | 0x7FF00000, 0);
+    return __hiloint2double((hi & ~0x7FF00000) | (be << 20), lo);
+}
+
 // int64 -> nearest double (round half to even, the conversion instruction) times
 // 2^scale, the scaling done exactly on the exponent field; results below the
 // normal range flush to zero and above it go to infinity.
@@ -471,19 +537,53 @@ struct SplitArgs {
     const int *eA, *eB;
     double *C;
     Idx2 Cm, Cn;
-    unsigned long long *partial;     // ksplit > 1: M x N int64 accumulator
+    unsigned long long *partial;     // ksplit > 1: M x N int64 accumulator (FP64 slices: two of them)
     int *err;
+    // FP64 slices (T = 8) only: C = alpha A B + beta C, and the operands, for rows and
+    // columns that hold an infinity or a NaN
+    double alpha, beta;
+    const double *A, *B;
+    Idx2 Am, Ak, Bk, Bn;
 };
 
+// A row (column) of FP64 slices whose exponent word is an infinity's or a NaN's has no grid.
+// Its scale is marked, and every output it touches is the plain FP64 sum instead.
+constexpr int SP_NONFINITE = 1 << 28;
+template <int T>
+__device__ __forceinline__ int operand_scale(int word)
+{
+    if (sp_wide(T) && word >= 0x7FF00000) return SP_NONFINITE;
+    return exp_of_word(word);
+}
+__device__ __noinline__ double plain_dot(const SplitArgs &a, int m, int n)
+{
+    const double *x = a.A + off2(a.Am, m), *y = a.B + off2(a.Bn, n);
+    double s = 0.0;
+    for (int k = 0; k < a.K; ++k) s = fma(x[off2(a.Ak, k)], y[off2(a.Bk, k)], s);
+    return s;
+}
+// The output element of an unscaled FP64-slice sum d: scale, alpha and beta applied.
+__device__ __forceinline__ void store_wide(const SplitArgs &a, double d, int scale, int m, int n, long long off)
+{
+    double v = scale > SP_NONFINITE / 2 ? plain_dot(a, m, n) : scale_exponent(d, scale);
+    if (a.alpha != 1.0) v *= a.alpha;
+    if (a.beta != 0.0) v = fma(a.beta, a.C[off], v);
+    a.C[off] = v;
+}
+
 template <int NT, int T, bool DEEP = false>
-__global__ void __launch_bounds__(SpCfg<NT>::THREADS, DEEP ? 1 : SpCfg<NT>::MIN_BLOCKS) gemm_split_kernel(SplitArgs a)
+__global__ void __launch_bounds__(SpCfg<NT>::THREADS, DEEP ? 1 : SpCfg<NT>::MIN_BLOCKS)
+gemm_split_kernel(SplitArgs a)
 {
     constexpr int A_TILE = SP_BM * SP_BK * 2;   // 16 KB
     constexpr int B_TILE = NT * SP_BK * 2;
     constexpr int QW = NT / (SpCfg<NT>::EPI_WARPS / 4);   // columns per epilogue warp
-    constexpr int SP_ASLOTS = DEEP ? SpDeep<T>::A : SpCfg<NT>::ASLOTS;
+    constexpr int SP_ASLOTS = DEEP ? SpDeep<T>::A : sp_aslots(NT, T);
     constexpr int SP_EPI_WARPS = SpCfg<NT>::EPI_WARPS;
     constexpr int SP_EPI_THREADS = SpCfg<NT>::EPI_THREADS;
+    constexpr int SP_KT_PER_CHUNK = sp_chunk_kt(T);
+    constexpr bool WIDE = sp_wide(T);
+    constexpr int UNIT = 2 * sp_top_bits(T) + 8 * (T - 1);   // the sums' unit is 2^(E_A + E_B - UNIT)
     constexpr int TMEM_COLS = SpCfg<NT>::TMEM_COLS;
     extern __shared__ unsigned char smem_raw[];
     __shared__ uint64_t bars[SP_ASLOTS * 2 + SP_BSLOTS * 2 + 3];
@@ -548,11 +648,8 @@ __global__ void __launch_bounds__(SpCfg<NT>::THREADS, DEEP ? 1 : SpCfg<NT>::MIN_
                     const int sb = b % SP_BSLOTS;
                     if (!mbar_wait(B_empty(sb), ((b / SP_BSLOTS) & 1) ^ 1, abort_flag)) break;
                     mbar_expect_tx(B_full(sb), (uint32_t)(T * B_TILE));
-                    for (int j = 0; j < T; ++j) {
-                        const unsigned char *src =
-                            a.Bpk + j * a.b_slice_bytes + ((long long)nt * a.kTiles + kt) * B_TILE;
-                        bulk_g2s(smem_u32(Bsm + (sb * T + j) * B_TILE), src, B_TILE, B_full(sb));
-                    }
+                    bulk_g2s(smem_u32(Bsm + sb * T * B_TILE),
+                             a.Bpk + ((long long)nt * a.kTiles + kt) * (T * B_TILE), T * B_TILE, B_full(sb));
                 }
             }
         } else if (lane == 1) {
@@ -564,8 +661,7 @@ __global__ void __launch_bounds__(SpCfg<NT>::THREADS, DEEP ? 1 : SpCfg<NT>::MIN_
                         const int sa = u % SP_ASLOTS;
                         if (!mbar_wait(A_empty(sa), ((u / SP_ASLOTS) & 1) ^ 1, abort_flag)) break;
                         mbar_expect_tx(A_full(sa), (uint32_t)A_TILE);
-                        const unsigned char *src =
-                            a.Apk + i * a.a_slice_bytes + ((long long)mt * a.kTiles + kt) * A_TILE;
+                        const unsigned char *src = a.Apk + (((long long)mt * a.kTiles + kt) * T + i) * A_TILE;
                         bulk_g2s(smem_u32(Asm + sa * A_TILE), src, A_TILE, A_full(sa));
                     }
                 }
@@ -640,9 +736,11 @@ __global__ void __launch_bounds__(SpCfg<NT>::THREADS, DEEP ? 1 : SpCfg<NT>::MIN_
         const int sub = warp & 3;              // TMEM sub-partition this warp may read
         const int part = (warp - 2) >> 2;      // which slice of the NT columns
         const uint32_t lane_base = (uint32_t)(32 * sub) << 16;
-        long long acc[QW];
+        long long acc[QW], acl[WIDE ? QW : 1];   // acl: levels 4 .. 7 of the FP64 slices
 #pragma unroll
         for (int q = 0; q < QW; ++q) acc[q] = 0;
+#pragma unroll
+        for (int q = 0; q < (WIDE ? QW : 1); ++q) acl[q] = 0;
         int chunk = 0;
         for (int c = c_beg; c < c_end; ++c, ++chunk) {
             // one lane polls, the warp follows it, so tcgen05.ld below runs converged
@@ -654,15 +752,21 @@ __global__ void __launch_bounds__(SpCfg<NT>::THREADS, DEEP ? 1 : SpCfg<NT>::MIN_
             // one level at a time: all its column groups in flight, then one wait.
             // A level holds an integer below 2^31 in magnitude (exact for t <= 3),
             // so a 32-bit conversion suffices.
+#pragma unroll
             for (int t = 0; t < T; ++t) {
-                const int sh = 8 * (T - 1 - t);
+                const int sh = WIDE ? 8 * (3 - (t & 3)) : 8 * (T - 1 - t);
                 uint32_t r[QW];
 #pragma unroll
                 for (int g = 0; g < QW / 8; ++g)
                     tmem_ld8(tmem + lane_base + (uint32_t)(t * NT + part * QW + 8 * g), r + 8 * g);
                 tmem_wait_ld();
 #pragma unroll
-                for (int q = 0; q < QW; ++q) acc[q] += (long long)__float2int_rn(__uint_as_float(r[q])) << sh;
+                for (int q = 0; q < QW; ++q) {
+                    const int v = __float2int_rn(__uint_as_float(r[q]));
+                    if (WIDE && t >= 4) acl[WIDE ? q : 0] += (long long)v * (1 << sh);
+                    else if (WIDE) acc[q] += (long long)v * (1 << sh);
+                    else acc[q] += (long long)v << sh;
+                }
             }
             tc_fence_before();
             __syncwarp();
@@ -675,7 +779,8 @@ __global__ void __launch_bounds__(SpCfg<NT>::THREADS, DEEP ? 1 : SpCfg<NT>::MIN_
         // out with the lanes running along whichever output index is contiguous.
         constexpr int PITCH = NT + 1;
         long long *stage = reinterpret_cast<long long *>(sm);
-        long long *row_off = stage + SP_BM * PITCH;
+        long long *stage_lo = stage + SP_BM * PITCH;   // FP64 slices with split-K: the second accumulator
+        long long *row_off = stage + (WIDE ? 2 : 1) * SP_BM * PITCH;
         long long *col_off = row_off + SP_BM;
         int *row_sc = reinterpret_cast<int *>(col_off + NT);   // exponent scales of the output
         int *col_sc = row_sc + SP_BM;
@@ -693,17 +798,23 @@ __global__ void __launch_bounds__(SpCfg<NT>::THREADS, DEEP ? 1 : SpCfg<NT>::MIN_
             if (m < a.M) {
                 if (part == 0) {
                     row_off[r] = fin ? off2(a.Cm, m) : (long long)m * a.N;
-                    row_sc[r] = fin ? exp_of_word(__ldg(a.eA + m)) - 14 - 8 * (T - 1) : 0;
+                    row_sc[r] = fin ? operand_scale<T>(__ldg(a.eA + m)) - UNIT : 0;
                 }
 #pragma unroll
                 for (int q = 0; q < QW; ++q) {
                     const int c = part * QW + q;
-                    if (n0 + c < a.N) stage[r * PITCH + c] = acc[q];
+                    if (n0 + c >= a.N) continue;
+                    if (WIDE && fin) {
+                        stage[r * PITCH + c] = __double_as_longlong(wide_to_double(acc[q], acl[WIDE ? q : 0]));
+                    } else {
+                        stage[r * PITCH + c] = acc[q];
+                        if (WIDE) stage_lo[r * PITCH + c] = acl[WIDE ? q : 0];
+                    }
                 }
             }
             for (int c = et; c < cols; c += SP_EPI_THREADS) {
                 col_off[c] = fin ? off2(a.Cn, n0 + c) : (long long)(n0 + c);
-                col_sc[c] = fin ? exp_of_word(__ldg(a.eB + n0 + c)) : 0;
+                col_sc[c] = fin ? operand_scale<T>(__ldg(a.eB + n0 + c)) : 0;
             }
         }
         asm volatile("bar.sync 1, %0;" ::"n"(SP_EPI_THREADS) : "memory");
@@ -740,8 +851,17 @@ __global__ void __launch_bounds__(SpCfg<NT>::THREADS, DEEP ? 1 : SpCfg<NT>::MIN_
 #pragma unroll
                         for (int j = 0; j < NCH; ++j) {
                             if (lane + 32 * j >= cols) continue;
-                            if (fin) a.C[ro[w] + co[j]] = scaled_int_to_double(v[w][j], rsc[w] + cs[j]);
-                            else atomicAdd(&a.partial[ro[w] + co[j]], (unsigned long long)v[w][j]);
+                            if (WIDE && fin) {
+                                store_wide(a, __longlong_as_double(v[w][j]), rsc[w] + cs[j],
+                                           m0 + rb + w * SP_EPI_WARPS, n0 + lane + 32 * j, ro[w] + co[j]);
+                            } else if (fin) {
+                                a.C[ro[w] + co[j]] = scaled_int_to_double(v[w][j], rsc[w] + cs[j]);
+                            } else {
+                                atomicAdd(&a.partial[ro[w] + co[j]], (unsigned long long)v[w][j]);
+                                if (WIDE)
+                                    atomicAdd(&a.partial[(long long)a.M * a.N + ro[w] + co[j]],
+                                              (unsigned long long)stage_lo[(rb + w * SP_EPI_WARPS) * PITCH + lane + 32 * j]);
+                            }
                         }
                     }
                 }
@@ -772,7 +892,14 @@ __global__ void __launch_bounds__(SpCfg<NT>::THREADS, DEEP ? 1 : SpCfg<NT>::MIN_
                         if (cb + w * SP_EPI_WARPS >= cols) break;
 #pragma unroll
                         for (int j = 0; j < NRC; ++j)
-                            if (lane + 32 * j < rows) a.C[ro[j] + co[w]] = scaled_int_to_double(v[w][j], rsc[j] + cs[w]);
+                        {
+                            if (lane + 32 * j >= rows) continue;
+                            if (WIDE)
+                                store_wide(a, __longlong_as_double(v[w][j]), rsc[j] + cs[w], m0 + lane + 32 * j,
+                                           n0 + cb + w * SP_EPI_WARPS, ro[j] + co[w]);
+                            else
+                                a.C[ro[j] + co[w]] = scaled_int_to_double(v[w][j], rsc[j] + cs[w]);
+                        }
                     }
                 }
             }
@@ -803,8 +930,22 @@ __global__ void split_finalize_kernel(int M, int N, int T, const unsigned long l
     }
 }
 
+// FP64 slices with split-K: the two integer sums to the output maps
+__global__ void split_finalize_wide_kernel(SplitArgs a)
+{
+    const long long total = (long long)a.M * a.N;
+    constexpr int UNIT = 2 * sp_top_bits(8) + 56;
+    for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < total;
+         t += (long long)gridDim.x * blockDim.x) {
+        const int m = (int)(t / a.N), n = (int)(t - (long long)m * a.N);
+        store_wide(a, wide_to_double((long long)a.partial[t], (long long)a.partial[total + t]),
+                   operand_scale<8>(a.eA[m]) + operand_scale<8>(a.eB[n]) - UNIT, m, n, off2(a.Cm, m) + off2(a.Cn, n));
+    }
+}
+
 int pick_nt(int N, int T)
 {
+    if (T == 8) return N <= 32 ? 32 : 64;
     if (T * 96 > 512) return 64;
     long long w64 = (long long)((N + 63) / 64) * 64, w96 = (long long)((N + 95) / 96) * 96;
     return (w96 <= w64) ? 96 : 64;
@@ -816,9 +957,10 @@ template <int NT, bool DEEP = false>
 size_t split_smem_bytes(int T)
 {
     const int aslots = DEEP ? (T == 2 ? SpDeep<2>::A : T == 3 ? SpDeep<3>::A : T == 4 ? SpDeep<4>::A : SpDeep<5>::A)
-                            : SpCfg<NT>::ASLOTS;
+                            : sp_aslots(NT, T);
     size_t b = 1024 + (size_t)aslots * SP_BM * SP_BK * 2 + (size_t)SP_BSLOTS * T * NT * SP_BK * 2;
-    const size_t out_stage = 1024 + (size_t)SP_BM * (NT + 1) * 8 + (size_t)(SP_BM + NT) * 12;   // epilogue reuse
+    const size_t out_stage =
+        1024 + (size_t)SP_BM * (NT + 1) * (sp_wide(T) ? 16 : 8) + (size_t)(SP_BM + NT) * 12;   // epilogue reuse
     if (b < out_stage) b = out_stage;
     if ((DEEP || SpCfg<NT>::MIN_BLOCKS == 1) && b < 120 * 1024) b = 120 * 1024;
     return b;
@@ -828,16 +970,29 @@ size_t split_smem_bytes(int T)
 
 int split_supported_T(int T) { return T >= 2 && T <= 5; }
 
+static bool engine_T(int T) { return split_supported_T(T) || T == SPLIT_F64_T; }
+static bool nt_ok(int nt, int T)
+{
+    if (T == SPLIT_F64_T) return nt == 32 || nt == 64;
+    return nt == 64 || (nt == 96 && T * 96 <= 512) || (nt == 48 && T * 48 <= 256);
+}
+
+// FP64 slices split K only where 128 x 64 tiles leave SMs idle: the large outputs fill the
+// GPU without it, and their two accumulators would take 16 bytes of workspace per element.
+static bool wide_split_k(int M, int N)
+{
+    return (long long)((M + SP_BM - 1) / SP_BM) * ((N + 63) / 64) < 2LL * device_sm_count();
+}
+
 SplitPlan split_plan(int M, int N, int K, int T, int nt_override, int ks_override)
 {
     SplitPlan p{};
+    const int SP_KT_PER_CHUNK = sp_chunk_kt(T);
     if (nt_override == SP_DEEP_CODE && T * 48 <= 256) {
         p.deep = 1;
         nt_override = 48;
     }
-    p.NT = (nt_override == 64 || (nt_override == 96 && T * 96 <= 512) || (nt_override == 48 && T * 48 <= 256))
-               ? nt_override
-               : pick_nt(N, T);
+    p.NT = nt_ok(nt_override, T) ? nt_override : pick_nt(N, T);
     p.mTiles = (M + SP_BM - 1) / SP_BM;
     p.nTiles = (N + p.NT - 1) / p.NT;
     p.kTiles = (K + SP_BK - 1) / SP_BK;
@@ -851,25 +1006,38 @@ SplitPlan split_plan(int M, int N, int K, int T, int nt_override, int ks_overrid
         ks = (int)((sms + tiles - 1) / tiles);
     }
     if (ks > chunks) ks = chunks;
-    if (ks < 1) ks = 1;
+    if (ks < 1 || (sp_wide(T) && !wide_split_k(M, N))) ks = 1;
     p.chunks_per_split = (chunks + ks - 1) / ks;
     p.ksplit = (chunks + p.chunks_per_split - 1) / p.chunks_per_split;
     p.a_pack_bytes = (size_t)T * p.mTiles * p.kTiles * SP_BM * SP_BK * 2;
     p.b_pack_bytes = (size_t)T * p.nTiles * p.kTiles * p.NT * SP_BK * 2;
-    p.partial_bytes = p.ksplit > 1 ? (size_t)M * N * 8 : 0;
+    p.partial_bytes = p.ksplit > 1 ? (size_t)M * N * (sp_wide(T) ? 16 : 8) : 0;
     return p;
 }
 
 SplitPlan split_plan_caps(int M, int N, int K, int T)
 {
     SplitPlan c = split_plan(M, N, K, T);
-    for (int nt : {48, 64, 96}) {
+    for (int nt : {32, 48, 64, 96}) {
+        if (!nt_ok(nt, T)) continue;
         SplitPlan p = split_plan(M, N, K, T, nt, 0);
         if (p.b_pack_bytes > c.b_pack_bytes) c.b_pack_bytes = p.b_pack_bytes;
     }
     const int kTiles = (K + SP_BK - 1) / SP_BK;
-    if (kTiles > SP_KT_PER_CHUNK) c.partial_bytes = (size_t)M * N * 8;   // any split-K candidate
+    if (kTiles > sp_chunk_kt(T) && (!sp_wide(T) || wide_split_k(M, N)))
+        c.partial_bytes = (size_t)M * N * (sp_wide(T) ? 16 : 8);   // any split-K candidate
     return c;
+}
+
+// Both sides measured on either side of this line: MNK = 8.4e6 27 (FP64 pipe) against 28 us and
+// 51 against 38; 4.2e6 31 against 37 and 16 against 27; 2.5e7 86 against 43.
+bool split_f64_pays(int M, int N, int K) { return (double)M * N * K >= 8e6; }
+
+bool split_fits(int M, int N, int K, int T, const SplitWork &w)
+{
+    const SplitPlan p = split_plan_caps(M, N, K, T);
+    return p.a_pack_bytes <= w.a_pack_cap && p.b_pack_bytes <= w.b_pack_cap && p.partial_bytes <= w.partial_cap &&
+           M <= w.e_cap && N <= w.e_cap;
 }
 
 template <int NT, int T, bool DEEP = false>
@@ -898,6 +1066,8 @@ cudaError_t split_prepare()
     if (e == cudaSuccess) e = split_attr<48, 3, true>();
     if (e == cudaSuccess) e = split_attr<48, 4, true>();
     if (e == cudaSuccess) e = split_attr<48, 5, true>();
+    if (e == cudaSuccess) e = split_attr<32, 8>();
+    if (e == cudaSuccess) e = split_attr<64, 8>();
     return e;
 }
 
@@ -927,7 +1097,7 @@ __device__ __forceinline__ unsigned ld_cluster_u32(const void *local, unsigned r
 template <int T, int KCMAX>
 __global__ void __launch_bounds__(256, 1) split_pack_tc_kernel(int R, int K, int rowsT, int rowsTotal, int kTiles,
                                                                int KC, const double *X, long long kstride, int *e,
-                                                               unsigned char *out, long long slice_bytes)
+                                                               unsigned char *out)
 {
     __shared__ unsigned long long Gs[32][SP_BK + 1];
     __shared__ unsigned s_part[8][32];
@@ -964,7 +1134,7 @@ __global__ void __launch_bounds__(256, 1) split_pack_tc_kernel(int R, int K, int
     }
     cluster_arrive();   // this CTA's remote reads are done; waited for before exit
     __syncthreads();
-    const int rs = grid_shift(exp_of_word((int)s_row[lane]), SplitDigits<T>::P);
+    const int rs = grid_shift<T>(exp_of_word((int)s_row[lane]));
     const int rw = threadIdx.x >> 3, c8 = threadIdx.x & 7;
     const int grw = r0 + rw;
 #pragma unroll
@@ -979,8 +1149,8 @@ __global__ void __launch_bounds__(256, 1) split_pack_tc_kernel(int R, int K, int
 #pragma unroll
                 for (int q = 0; q < 8; ++q) G[q] = Gs[rw][c8 * 8 + q];
                 const long long tile = (long long)(grw / rowsT) * kTiles + kt;
-                write_digit_chunks<T>(G, out + tile * ((long long)rowsT * SP_BK * 2) + sw128_off(grw % rowsT, c8 * 8),
-                                      slice_bytes);
+                const long long slice_bytes = (long long)rowsT * SP_BK * 2;
+                write_digit_chunks<T>(G, out + tile * (slice_bytes * T) + sw128_off(grw % rowsT, c8 * 8), slice_bytes);
             }
             __syncthreads();
         }
@@ -990,7 +1160,7 @@ __global__ void __launch_bounds__(256, 1) split_pack_tc_kernel(int R, int K, int
 
 template <int T, int KCMAX>
 static cudaError_t launch_pack_tc(int R, int K, int rowsT, int rowsTotal, int kTiles, int CS, int KC, const double *X,
-                                  long long kstride, int *e, unsigned char *pk, long long slice_bytes, cudaStream_t st)
+                                  long long kstride, int *e, unsigned char *pk, cudaStream_t st)
 {
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3(CS, (rowsTotal + 31) / 32, 1);
@@ -1005,14 +1175,13 @@ static cudaError_t launch_pack_tc(int R, int K, int rowsT, int rowsTotal, int kT
     cfg.attrs = at;
     cfg.numAttrs = 1;
     return cudaLaunchKernelEx(&cfg, split_pack_tc_kernel<T, KCMAX>, R, K, rowsT, rowsTotal, kTiles, KC, X, kstride, e,
-                              pk, slice_bytes);
+                              pk);
 }
 
 template <int T>
 static cudaError_t split_prepass_t(int R, int K, const double *X, Idx2 rmap, Idx2 kmap, int rowsT, int rowTiles,
                                    int kTiles, int *e, unsigned char *pk, cudaStream_t st)
 {
-    const long long slice_bytes = (long long)rowTiles * kTiles * rowsT * SP_BK * 2;
     const int KC = (kTiles + 7) / 8;
     int CS = 1;
     while (CS * KC < kTiles) CS *= 2;   // <= 8 for kTiles <= 64
@@ -1025,9 +1194,9 @@ static cudaError_t split_prepass_t(int R, int K, const double *X, Idx2 rmap, Idx
         (long long)(rowTiles * rowsT + 31) / 32 * CS <= device_sm_count()) {
         CTM_COUNT_LAUNCH(1);
         cudaError_t e1 = KC <= 2 ? launch_pack_tc<T, 2>(R, K, rowsT, rowTiles * rowsT, kTiles, CS, KC, X, kmap.s2, e, pk,
-                                                        slice_bytes, st)
+                                                        st)
                                  : launch_pack_tc<T, 8>(R, K, rowsT, rowTiles * rowsT, kTiles, CS, KC, X, kmap.s2, e, pk,
-                                                        slice_bytes, st);
+                                                        st);
         return e1 != cudaSuccess ? e1 : cudaGetLastError();
     }
     if (rmap.s1 == 0 && rmap.s2 == 1 && kmap.s1 == 0 && kmap.s2 != 1) {
@@ -1037,7 +1206,7 @@ static cudaError_t split_prepass_t(int R, int K, const double *X, Idx2 rmap, Idx
         split_colexp_kernel<<<dim3((R + 127) / 128, (K + SP_COLEXP_K - 1) / SP_COLEXP_K), 128, 0, st>>>(R, K, X,
                                                                                                        kmap.s2, e);
         split_pack_t_kernel<T><<<dim3((rowTiles * rowsT + 31) / 32, kTiles), 256, 0, st>>>(
-            R, K, rowsT, rowTiles * rowsT, kTiles, X, kmap.s2, e, pk, slice_bytes);
+            R, K, rowsT, rowTiles * rowsT, kTiles, X, kmap.s2, e, pk);
         return cudaGetLastError();
     }
     if (kmap.s1 == 0 && kmap.s2 == 1) {
@@ -1051,8 +1220,7 @@ static cudaError_t split_prepass_t(int R, int K, const double *X, Idx2 rmap, Idx
             const int rpb = wpr >= 8 ? 1 : 8 / wpr;         // rows per block
             const int blocks = (rows + rpb - 1) / rpb, threads = 32 * wpr * rpb;
 #define CTM_ROWPACK(NVV)                                                                                              \
-    split_rowpack_reg_kernel<NVV, T><<<blocks, threads, 0, st>>>(R, K, rowsT, rows, kTiles, wpr, X, rmap, e, pk,       \
-                                                                 slice_bytes)
+    split_rowpack_reg_kernel<NVV, T><<<blocks, threads, 0, st>>>(R, K, rowsT, rows, kTiles, wpr, X, rmap, e, pk)
             if (nv == 1) CTM_ROWPACK(1);
             else if (nv == 2) CTM_ROWPACK(2);
             else if (nv == 4) CTM_ROWPACK(4);
@@ -1060,8 +1228,7 @@ static cudaError_t split_prepass_t(int R, int K, const double *X, Idx2 rmap, Idx
 #undef CTM_ROWPACK
             return cudaGetLastError();
         }
-        split_rowpack_kernel<T><<<(rows + 7) / 8, 256, 0, st>>>(R, K, rowsT, rows, kTiles, X, rmap, e, pk,
-                                                                slice_bytes);
+        split_rowpack_kernel<T><<<(rows + 7) / 8, 256, 0, st>>>(R, K, rowsT, rows, kTiles, X, rmap, e, pk);
         return cudaGetLastError();
     }
     CTM_COUNT_LAUNCH(2);
@@ -1082,6 +1249,7 @@ static cudaError_t split_prepass(int R, int K, const double *X, Idx2 rmap, Idx2 
     case 3: return split_prepass_t<3>(R, K, X, rmap, kmap, rowsT, rowTiles, kTiles, e, pk, st);
     case 4: return split_prepass_t<4>(R, K, X, rmap, kmap, rowsT, rowTiles, kTiles, e, pk, st);
     case 5: return split_prepass_t<5>(R, K, X, rmap, kmap, rowsT, rowTiles, kTiles, e, pk, st);
+    case 8: return split_prepass_t<8>(R, K, X, rmap, kmap, rowsT, rowTiles, kTiles, e, pk, st);
     default: return cudaErrorInvalidValue;
     }
 }
@@ -1142,7 +1310,15 @@ static cudaError_t gemm_split_run(const GemmF64 &g, int T, SplitWork w, cudaStre
                 g.Cm,
                 g.Cn,
                 (unsigned long long *)w.partial,
-                w.err};
+                w.err,
+                g.alpha,
+                g.beta,
+                g.A,
+                g.B,
+                g.Am,
+                g.Ak,
+                g.Bk,
+                g.Bn};
     dim3 grid(p.nTiles, p.mTiles, p.ksplit);
     CTM_COUNT_LAUNCH(1);
     if (ev) cudaEventRecord(ev[0], st);
@@ -1164,6 +1340,10 @@ static cudaError_t gemm_split_run(const GemmF64 &g, int T, SplitWork w, cudaStre
     CTM_SPLIT_LAUNCH(48, 4)
     CTM_SPLIT_LAUNCH(48, 5)
 #undef CTM_SPLIT_LAUNCH
+    if (T == 8 && p.NT == 32)
+        gemm_split_kernel<32, 8><<<grid, SpCfg<32>::THREADS, split_smem_bytes<32>(8), st>>>(a);
+    if (T == 8 && p.NT == 64)
+        gemm_split_kernel<64, 8><<<grid, SpCfg<64>::THREADS, split_smem_bytes<64>(8), st>>>(a);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     if (ev) cudaEventRecord(ev[1], st);
     if (p.ksplit > 1) {
@@ -1171,8 +1351,10 @@ static cudaError_t gemm_split_run(const GemmF64 &g, int T, SplitWork w, cudaStre
         long long blocks = (total + 255) / 256, cap = 16LL * device_sm_count();
         if (blocks > cap) blocks = cap;
         CTM_COUNT_LAUNCH(1);
-        split_finalize_kernel<<<(int)blocks, 256, 0, st>>>(g.M, g.N, T, (const unsigned long long *)w.partial,
-                                                              w.eA, w.eB, g.C, g.Cm, g.Cn);
+        if (sp_wide(T)) split_finalize_wide_kernel<<<(int)blocks, 256, 0, st>>>(a);
+        else
+            split_finalize_kernel<<<(int)blocks, 256, 0, st>>>(g.M, g.N, T, (const unsigned long long *)w.partial,
+                                                                  w.eA, w.eB, g.C, g.Cm, g.Cn);
         e = cudaGetLastError();
     }
     return e;
@@ -1197,7 +1379,7 @@ cudaError_t gemm_split(const GemmF64 &g, int T, SplitWork w, cudaStream_t st, cu
                        const SplitOpts *opt)
 {
     if (g.M <= 0 || g.N <= 0) return cudaSuccess;
-    if (!split_supported_T(T) || g.alpha != 1.0 || g.beta != 0.0) return cudaErrorInvalidValue;
+    if (!engine_T(T) || (!sp_wide(T) && (g.alpha != 1.0 || g.beta != 0.0))) return cudaErrorInvalidValue;
     const auto key = std::make_tuple(g.M, g.N, g.K, T);
     {
         std::lock_guard<std::mutex> lk(g_tune_mu);
@@ -1217,13 +1399,15 @@ cudaError_t gemm_split(const GemmF64 &g, int T, SplitWork w, cudaStream_t st, cu
     }
     cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
     cudaStreamIsCapturing(st, &cs);
-    if (!w.autotune || cs != cudaStreamCaptureStatusNone)
+    // (an accumulating product cannot be repeated: it takes the default plan until a plain
+    // product of its shape has been timed)
+    if (!w.autotune || cs != cudaStreamCaptureStatusNone || g.beta != 0.0)
         return gemm_split_run(g, T, w, st, ev, split_plan(g.M, g.N, g.K, T), opt);
     SplitPlan base = split_plan(g.M, g.N, g.K, T);
-    const int chunks = (base.kTiles + SP_KT_PER_CHUNK - 1) / SP_KT_PER_CHUNK;
+    const int chunks = (base.kTiles + sp_chunk_kt(T) - 1) / sp_chunk_kt(T);
     std::vector<std::pair<int, int>> cands;
-    for (int nt : {48, 64, 96, SP_DEEP_CODE}) {
-        if ((nt == 96 && T * 96 > 512) || ((nt == 48 || nt == SP_DEEP_CODE) && T * 48 > 256)) continue;
+    for (int nt : {32, 48, 64, 96, SP_DEEP_CODE}) {
+        if (!nt_ok(nt == SP_DEEP_CODE ? 48 : nt, T)) continue;
         // the deep ring pays off only for long K streams: at K of a few thousand it can win
         // alone yet slow the step, whose concurrent corner update and corner spectrum
         // then find every SM held by one 226 KB CTA (measured 1053 against ~1130 steps/s
@@ -1233,7 +1417,7 @@ cudaError_t gemm_split(const GemmF64 &g, int T, SplitWork w, cudaStream_t st, cu
         const int ntw = nt == SP_DEEP_CODE ? 48 : nt;   // tile width of the candidate
         const int one_wave = (int)(device_sm_count() / ((long long)base.mTiles * ((g.N + ntw - 1) / ntw)));
         for (int ks : {base.ksplit, 1, 2 * base.ksplit, base.ksplit / 2, one_wave}) {
-            if (ks < 1 || ks > chunks) continue;
+            if (ks < 1 || ks > chunks || (ks > 1 && sp_wide(T) && !wide_split_k(g.M, g.N))) continue;
             std::pair<int, int> c{nt, ks};
             bool dup = false;
             for (auto &o : cands) dup |= (o == c);

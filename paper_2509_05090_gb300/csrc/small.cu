@@ -125,6 +125,17 @@ __global__ void warm_start_kernel(long long n, int chi, const double *Q, const d
     }
 }
 
+// Y = M Q S where Q is the first chi columns of I_n (M n x n row-major).
+__global__ void select_columns_kernel(long long n, int chi, const double *M, const double *C, double *Y)
+{
+    for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < n * chi;
+         t += (long long)gridDim.x * blockDim.x) {
+        const int j = (int)(t % chi);
+        const double v = M[(t / chi) * n + j];
+        Y[t] = (C[(size_t)j * chi + j] < 0.0) ? -v : v;
+    }
+}
+
 // a5 tail: C' = (Cr + Cr^T)/2, then unit Frobenius norm, over several blocks (the FP64 work of one SM would
 // bind): partial sums of squares, then every block derives the factor from the
 // partials with one warp and scales its share.
@@ -696,6 +707,13 @@ cudaError_t launch_warm_start(int n, int chi, const double *Q, const double *C, 
 {
     CTM_COUNT_LAUNCH(1);
     warm_start_kernel<<<grid_for((long long)n * chi), 256, 0, st>>>(n, chi, Q, C, Qs);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_select_columns(int n, int chi, const double *M, const double *C, double *Y, cudaStream_t st)
+{
+    CTM_COUNT_LAUNCH(1);
+    select_columns_kernel<<<grid_for((long long)n * chi), 256, 0, st>>>(n, chi, M, C, Y);
     return cudaGetLastError();
 }
 
