@@ -22,6 +22,7 @@
 #include <vector>
 
 #include "ctm_internal.h"
+#include "fp64_chain.h"
 
 struct ctm_complex_ctx {
     ctm_config cfg;
@@ -596,140 +597,201 @@ __global__ void zc_herm_normalize_kernel(int chi, const double *Cr, long long PC
     }
 }
 
-// Sum over the CTA of one value per thread (blockDim a multiple of 32, <= 1024).
-__device__ double zblock_sum(double v, double *red)
-{
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-    const int w = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    __syncthreads();
-    if ((threadIdx.x & 31) == 0) red[w] = v;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double s = 0.0;
-        for (int i = 0; i < nw; ++i) s += red[i];
-        red[32] = s;
-    }
-    __syncthreads();
-    return red[32];
-}
-
 // The corner spectrum, step one: Householder reduction of the Hermitian corner (Re in plane
 // 0, Im in plane 3 of its five planes) to tridiagonal form in one CTA's shared memory.  For
 // column k with x the part below the diagonal, x_0 = |x_0| e^{i theta}: alpha =
 // -e^{i theta} |x|, v = x - alpha e_0, beta = 2 / |v|^2 = 1 / (|x| (|x| + |x_0|)); with
-// p = beta A v, K = (beta/2) Re(v^H p) and w = p - K v the update is
-// A <- A - v w^H - w v^H.  The result is a Hermitian tridiagonal matrix whose eigenvalues
-// are those of the real symmetric one with off-diagonal |e_i|: work receives its diagonal
-// and |e_i|^2, which the bisection of the real spectrum takes as they are.
-constexpr int ZTRI_THREADS = 256;
-size_t ztridiag_smem_bytes(int chi) { return sizeof(double) * ((size_t)2 * chi * (chi | 1) + 4 * (size_t)chi); }
+// p = beta A v and K = (beta/2) Re(v^H p) the update is
+// A <- A - v p^H - g v^H, g = p - 2 K v.  The result is a Hermitian tridiagonal matrix whose
+// eigenvalues are those of the real symmetric one with off-diagonal |e_i|: work receives its
+// diagonal and |e_i|^2, which the bisection of the real spectrum takes as they are.
+//
+// The schedule is the real kernel's (small.cu: tridiag_kernel): lower triangle only, one
+// reduction and three barriers per column -- Re(v^H p) = beta (x^H A x - 2 Re(conj(alpha) y_0)
+// + |alpha|^2 A_00) with y = A x -- and a scalar warp that finishes the next column and its
+// alpha and beta while the others update and multiply.  Bound by FP64 issue (four
+// multiply-adds per element of the mat-vec, eight per element of the triangle).
+// chi = 72: 952 -> 587 us alone.
+constexpr int ZTRI_WARPS = 9;   // eight workers (four lanes per row, eight per row pair), one scalar warp
+__host__ __device__ inline int ztri_pitch(int chi) { return chi + ((20 - chi % 16) % 16); }   // = 4 mod 16
+size_t ztridiag_smem_bytes(int chi)
+{
+    return sizeof(double) * ((size_t)2 * chi * ztri_pitch(chi) + 10 * (size_t)chi);
+}
 size_t ztridiag_launch_bytes(int chi)
 {
     const size_t need = ztridiag_smem_bytes(chi), alone = 220 * 1024;
     return need > alone ? need : alone;
 }
 
-__global__ void __launch_bounds__(ZTRI_THREADS) zc_tridiag_kernel(int chi, const double *C, long long PC, double *work)
+__global__ void __launch_bounds__(32 * ZTRI_WARPS) zc_tridiag_kernel(int chi, const double *C, long long PC,
+                                                                      double *work)
 {
     extern __shared__ double sm[];
-    __shared__ double red[33];
-    __shared__ double sh_beta, sh_ar, sh_ai;
-    const int ld = chi | 1;
-    double *Ar = sm, *Ai = Ar + (size_t)chi * ld;
-    double *vr = Ai + (size_t)chi * ld, *vi = vr + chi, *pr = vi + chi, *pim = pr + chi;
-    const int tid = threadIdx.x;
+    __shared__ double sh_ar, sh_ai, sh_n2, sh_beta, sh_K;
+    const int ld = ztri_pitch(chi);
+    double *Ar = sm, *Ai = Ar + (size_t)chi * ld;          // lower triangles
+    double *xrb = Ai + (size_t)chi * ld, *xib = xrb + 2 * chi;   // 2 x chi each: the column, by parity
+    double *yr = xib + 2 * chi, *yi = yr + chi, *pr = yi + chi, *pi = pr + chi, *vr = pi + chi, *vi = vr + chi;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int nthr = blockDim.x, nwork = nthr - 32;
     const double *Ci = C + 3 * PC;
-    for (int t = tid; t < chi * chi; t += blockDim.x) {
+    for (int t = tid; t < chi * chi; t += nthr) {
         const int i = t / chi, j = t % chi;
+        if (j > i) continue;
         Ar[i * ld + j] = 0.5 * (C[t] + C[j * chi + i]);
-        Ai[i * ld + j] = 0.5 * (Ci[t] - Ci[j * chi + i]);
+        Ai[i * ld + j] = 0.5 * (Ci[t] - Ci[j * chi + i]);   // zero on the diagonal, and kept so
     }
     __syncthreads();
+    auto sync_all = [] { asm volatile("bar.sync 0;" ::: "memory"); };
+    auto sync_next = [&] { asm volatile("bar.sync 1, %0;" ::"r"(nthr) : "memory"); };
+    auto arrive_next = [&] {
+        __threadfence_block();
+        asm volatile("bar.arrive 1, %0;" ::"r"(nthr) : "memory");
+    };
+    if (tid >= nwork) {
+        // ------------------------------------------------ scalar warp
+        for (int i = lane; i + 1 < chi; i += 32) {
+            xrb[i] = Ar[(i + 1) * ld];
+            xib[i] = Ai[(i + 1) * ld];
+        }
+        if (lane == 0) work[0] = Ar[0];
+        __syncwarp();
+        arrive_next();
+        for (int kc = 0; kc + 1 < chi; ++kc) {
+            const double *xr = xrb + (kc & 1) * chi, *xi = xib + (kc & 1) * chi;
+            const int b0 = kc + 1, m = chi - b0;
+            double s1 = 0.0;
+            for (int i = 1 + lane; i < m; i += 32) s1 = fma(xr[i], xr[i], fma(xi[i], xi[i], s1));
+            s1 = warp_sum(s1);
+            const double x0r = xr[0], x0i = xi[0], t = fma(x0r, x0r, x0i * x0i);
+            double ar = x0r, ai = x0i, n2 = t, beta = 0.0;   // already reduced: no reflector
+            if (s1 != 0.0) {
+                double a0 = 0.0, cr = 1.0, ci = 0.0;
+                if (t != 0.0) {
+                    const HouseholderScalars h0 = householder_scalars(t, 0.0);   // |x_0|, 1 / |x_0|^2
+                    a0 = h0.nrm;
+                    cr = x0r * (a0 * h0.beta);
+                    ci = x0i * (a0 * h0.beta);
+                }
+                n2 = s1 + t;
+                const HouseholderScalars h = householder_scalars(n2, a0);
+                ar = -cr * h.nrm;
+                ai = -ci * h.nrm;
+                beta = h.beta;
+            }
+            if (lane == 0) {
+                sh_ar = ar;
+                sh_ai = ai;
+                sh_n2 = n2;
+                sh_beta = beta;
+                work[chi + kc] = n2;
+            }
+            if (kc + 2 >= chi) break;
+            sync_all();   // A
+            sync_all();   // B
+            const double K2 = 2.0 * sh_K, p0r = pr[0], p0i = pi[0], v0r = vr[0], v0i = vi[0];
+            double *nr = xrb + ((kc + 1) & 1) * chi, *ni = xib + ((kc + 1) & 1) * chi;
+            for (int i = lane; i < m; i += 32) {
+                const double a = vr[i], b = vi[i], gr = fma(-K2, a, pr[i]), gi = fma(-K2, b, pi[i]);
+                const double re = fma(-gi, v0i, fma(-gr, v0r, fma(-b, p0i, fma(-a, p0r, Ar[(b0 + i) * ld + b0]))));
+                const double im = fma(gr, v0i, fma(-gi, v0r, fma(a, p0i, fma(-b, p0r, Ai[(b0 + i) * ld + b0]))));
+                if (i == 0) work[b0] = re;
+                else {
+                    nr[i - 1] = re;
+                    ni[i - 1] = im;
+                }
+            }
+            __syncwarp();
+            arrive_next();
+        }
+        if (lane == 0) work[2 * chi - 1] = 0.0;
+        return;
+    }
+    sync_next();
     for (int kc = 0; kc + 2 < chi; ++kc) {
+        const double *xr = xrb + (kc & 1) * chi, *xi = xib + (kc & 1) * chi;
         const int b0 = kc + 1, m = chi - b0;
-        double part = 0.0;
-        for (int i = tid; i < m; i += blockDim.x) {
-            const double xr = Ar[(b0 + i) * ld + kc], xi = Ai[(b0 + i) * ld + kc];
-            vr[i] = xr;
-            vi[i] = xi;
-            if (i > 0) part += xr * xr + xi * xi;
-        }
-        const double tail = zblock_sum(part, red);   // its barriers also publish v
-        if (tail == 0.0) continue;                   // already tridiagonal in this column
-        const double x0r = vr[0], x0i = vi[0];
-        if (tid == (int)blockDim.x - 1) {
-            const double a0 = sqrt(x0r * x0r + x0i * x0i);
-            const double nrm = sqrt(tail + a0 * a0);
-            const double cr = a0 > 0.0 ? x0r / a0 : 1.0, ci = a0 > 0.0 ? x0i / a0 : 0.0;
-            sh_ar = -cr * nrm;
-            sh_ai = -ci * nrm;
-            sh_beta = 1.0 / (nrm * (nrm + a0));
-        }
-        // y = A x over the trailing block (v still holds x)
-        for (int i = tid; i < m; i += blockDim.x) {
-            const double *rr = Ar + (b0 + i) * ld + b0, *ri = Ai + (b0 + i) * ld + b0;
-            double sr0 = 0.0, si0 = 0.0, sr1 = 0.0, si1 = 0.0;
-            int j = 0;
-            for (; j + 1 < m; j += 2) {
-                sr0 = fma(rr[j], vr[j], fma(-ri[j], vi[j], sr0));
-                si0 = fma(rr[j], vi[j], fma(ri[j], vr[j], si0));
-                sr1 = fma(rr[j + 1], vr[j + 1], fma(-ri[j + 1], vi[j + 1], sr1));
-                si1 = fma(rr[j + 1], vi[j + 1], fma(ri[j + 1], vr[j + 1], si1));
+        double *Br = Ar + b0 * ld + b0, *Bi = Ai + b0 * ld + b0;
+        {
+            const int c = tid & 3;
+            for (int i0 = 0; i0 < m; i0 += nwork / 4) {
+                const int i = i0 + (tid >> 2);
+                double r0 = 0.0, r1 = 0.0, q0 = 0.0, q1 = 0.0;
+                if (i < m) {
+                    int j = c;
+                    for (; j <= i; j += 4) {   // A_ij x_j
+                        const double a = Br[i * ld + j], b = Bi[i * ld + j], xa = xr[j], xb = xi[j];
+                        r0 = fma(a, xa, r0);
+                        r1 = fma(-b, xb, r1);
+                        q0 = fma(a, xb, q0);
+                        q1 = fma(b, xa, q1);
+                    }
+                    for (; j < m; j += 4) {    // conj(A_ji) x_j
+                        const double a = Br[j * ld + i], b = Bi[j * ld + i], xa = xr[j], xb = xi[j];
+                        r0 = fma(a, xa, r0);
+                        r1 = fma(b, xb, r1);
+                        q0 = fma(a, xb, q0);
+                        q1 = fma(-b, xa, q1);
+                    }
+                }
+                r0 += r1;
+                q0 += q1;
+                r0 += __shfl_xor_sync(0xffffffffu, r0, 1);
+                q0 += __shfl_xor_sync(0xffffffffu, q0, 1);
+                r0 += __shfl_xor_sync(0xffffffffu, r0, 2);
+                q0 += __shfl_xor_sync(0xffffffffu, q0, 2);
+                if (i < m && c == 0) {
+                    yr[i] = r0;
+                    yi[i] = q0;
+                }
             }
-            if (j < m) {
-                sr0 = fma(rr[j], vr[j], fma(-ri[j], vi[j], sr0));
-                si0 = fma(rr[j], vi[j], fma(ri[j], vr[j], si0));
+        }
+        sync_all();   // A
+        {
+            const double ar = sh_ar, ai = sh_ai, beta = sh_beta;
+            if (warp == 0) {
+                double s2 = 0.0;   // x^H A x, real
+                for (int i = lane; i < m; i += 32) s2 = fma(xr[i], yr[i], fma(xi[i], yi[i], s2));
+                const double q = fma(sh_n2, Br[0], -2.0 * fma(ar, yr[0], ai * yi[0])), hb = 0.5 * beta * beta;
+                s2 = warp_sum(s2);
+                if (lane == 0) sh_K = hb * (s2 + q);
+            } else {
+                for (int i = tid - 32; i < m; i += nwork - 32) {
+                    const double er = Br[i * ld], ei = Bi[i * ld];
+                    pr[i] = beta * fma(ai, ei, fma(-ar, er, yr[i]));
+                    pi[i] = beta * fma(-ai, er, fma(-ar, ei, yi[i]));
+                    vr[i] = i == 0 ? xr[0] - ar : xr[i];
+                    vi[i] = i == 0 ? xi[0] - ai : xi[i];
+                }
             }
-            pr[i] = sr0 + sr1;
-            pim[i] = si0 + si1;
         }
-        __syncthreads();
-        const double beta = sh_beta, ar = sh_ar, ai = sh_ai;
-        // p = beta (A x - alpha A e_0), then v_0 = x_0 - alpha
-        for (int i = tid; i < m; i += blockDim.x) {
-            const double er = Ar[(b0 + i) * ld + b0], ei = Ai[(b0 + i) * ld + b0];
-            pr[i] = beta * (pr[i] - (ar * er - ai * ei));
-            pim[i] = beta * (pim[i] - (ar * ei + ai * er));
+        sync_all();   // B
+        {
+            // rows 1 .. m-1, columns 1 .. row: rows a and mm-1-a make one list of mm+1 elements
+            const double K2 = 2.0 * sh_K;
+            const int mm = m - 1, c = tid & 7;
+            double *Sr = Br + ld + 1, *Si = Bi + ld + 1;
+            for (int a = tid >> 3; a < (mm + 1) / 2; a += nwork / 8) {
+                const int r2 = mm - 1 - a, len = r2 == a ? a + 1 : mm + 1;
+                for (int half = 0; half < 2; ++half) {
+                    const int row = half ? r2 : a, first = half ? a + 1 : 0, last = half ? len : a + 1;
+                    const double ur = vr[row + 1], ui = vi[row + 1];
+                    const double gr = fma(-K2, ur, pr[row + 1]), gi = fma(-K2, ui, pi[row + 1]);
+                    // this lane's elements of the list: e = c, c + 8, ...
+                    for (int e = first + ((c - first) & 7); e < last; e += 8) {
+                        const int j = e - first;
+                        const double a0 = pr[j + 1], a1 = pi[j + 1], b0r = vr[j + 1], b0i = vi[j + 1];
+                        double *tr = Sr + row * ld + j, *ti = Si + row * ld + j;
+                        *tr = fma(-gi, b0i, fma(-gr, b0r, fma(-ui, a1, fma(-ur, a0, *tr))));
+                        if (j != row) *ti = fma(gr, b0i, fma(-gi, b0r, fma(ur, a1, fma(-ui, a0, *ti))));
+                    }
+                }
+            }
         }
-        if (tid == 0) {
-            vr[0] = x0r - ar;
-            vi[0] = x0i - ai;
-        }
-        __syncthreads();
-        double pv = 0.0;   // Re(v^H p)
-        for (int i = tid; i < m; i += blockDim.x) pv += vr[i] * pr[i] + vi[i] * pim[i];
-        pv = zblock_sum(pv, red);
-        const double Kf = 0.5 * beta * pv;
-        for (int i = tid; i < m; i += blockDim.x) {   // p <- w
-            pr[i] -= Kf * vr[i];
-            pim[i] -= Kf * vi[i];
-        }
-        __syncthreads();
-        for (int t = tid; t < m * m; t += blockDim.x) {
-            const int i = t / m, j = t % m;
-            // v_i conj(w_j) + w_i conj(v_j)
-            const double re = vr[i] * pr[j] + vi[i] * pim[j] + pr[i] * vr[j] + pim[i] * vi[j];
-            const double im = vi[i] * pr[j] - vr[i] * pim[j] + pim[i] * vr[j] - pr[i] * vi[j];
-            Ar[(b0 + i) * ld + b0 + j] -= re;
-            Ai[(b0 + i) * ld + b0 + j] -= im;
-        }
-        if (tid == 0) {
-            Ar[b0 * ld + kc] = ar;
-            Ai[b0 * ld + kc] = ai;
-            Ar[kc * ld + b0] = ar;
-            Ai[kc * ld + b0] = -ai;
-        }
-        __syncthreads();
+        sync_next();   // C
     }
-    for (int i = tid; i < chi; i += blockDim.x) {
-        work[i] = Ar[i * ld + i];
-        double e2 = 0.0;
-        if (i + 1 < chi) {
-            const double er = Ar[(i + 1) * ld + i], ei = Ai[(i + 1) * ld + i];
-            e2 = er * er + ei * ei;
-        }
-        work[chi + i] = e2;
-    }
+    if (tid == 0 && chi >= 2) work[chi - 1] = Ar[(chi - 1) * ld + chi - 1];
 }
 
 // raw[pA][pB] = sum_{ab, z} Y1o[ab][pB][z] G2[ab][pA][z] (complex, no conjugation)
@@ -1224,7 +1286,7 @@ int zspectrum(ctm_complex_ctx *c, const double *Cin, cudaStream_t st, double *ds
         CTM_COUNT_LAUNCH(1);
         // all but a few KB of the SM's shared memory: the step's CTAs stay off its SM (as for
         // the real corner spectrum)
-        zc_tridiag_kernel<<<1, ZTRI_THREADS, ztridiag_launch_bytes(chi), st>>>(chi, Cin, c->PC, c->spec_work);
+        zc_tridiag_kernel<<<1, 32 * ZTRI_WARPS, ztridiag_launch_bytes(chi), st>>>(chi, Cin, c->PC, c->spec_work);
         ZK(cudaGetLastError());
         ZK(launch_spectrum_from_tridiag(chi, c->spec_work, c->s_new, c->s, c->delta, st));
     }

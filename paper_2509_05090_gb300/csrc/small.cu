@@ -11,6 +11,7 @@
 #include <mutex>
 
 #include "ctm_internal.h"
+#include "fp64_chain.h"
 
 namespace {
 
@@ -206,7 +207,6 @@ __global__ void scale_by_partials_kernel(long long count, double *x, const doubl
 //     changes of p_i = (d_i - x) p_{i-1} - e_{i-1}^2 p_{i-2}, kept in range by
 //     exact power-of-two rescaling -- no division on the dependent chain;
 // (3) one CTA: |lambda| sorted descending by rank, unit 2-norm, delta.
-constexpr int SPEC_WARPS = 1;   // one eigenvalue per CTA: the chi Sturm chains spread over chi SMs
 constexpr int TRI_THREADS = 256;
 constexpr size_t SPEC_SM_ALONE_BYTES = 220 * 1024;   // within the 224 KB opt-in of spectrum_prepare
 constexpr int TRI_FULL_MAX = 160;   // the full corner in shared memory up to here, its lower triangle beyond
@@ -221,81 +221,180 @@ constexpr int TRI_CLUSTER_MIN = 97;
 // d, e^2 (2 chi) and the eigenvalues (chi)
 __host__ __device__ inline size_t tri_global_off(int chi) { return (size_t)3 * chi + 8; }
 
-__global__ void __launch_bounds__(TRI_THREADS) tridiag_kernel(int chi, const double *C, double *work)
+// One CTA, chi <= TRI_FULL_MAX.  Bound by FP64 issue (one warp instruction per 64 cycles and
+// sub-partition: m^2 multiply-adds for the mat-vec and as many for the update, lower
+// triangle only) and by the serial chain per column, which is kept to one reduction and one
+// pair of Householder scalars:
+//   y = A x (x: the column below the diagonal), s2 = x^T y;  with v = x - alpha e_0 and
+//   p = beta A v = beta (y - alpha A e_0) the inner product p^T v is
+//   beta (s2 - 2 alpha y_0 + alpha^2 A_00), so nothing waits for a second reduction;
+//   with K = beta/2 p^T v and g = p - 2 K v the update is A_ij -= v_i p_j + g_i v_j.
+// Per column three barriers: A (y is complete, and the scalar warp's alpha and beta), B (p, v
+// and K), C (the next x).  The last warp works one column ahead: after B it updates the next
+// column itself (the workers leave it out), hands it over at C without waiting, and forms
+// |x|^2, alpha and beta while the others update and multiply.  A column already reduced has
+// beta = 0, alpha = x_0 and an update of zero.  chi = 72: 391 -> 211 us alone.
+constexpr int TRI_WARPS = 9;   // eight workers, two per sub-partition (four lanes per row, eight per row pair), one scalar warp
+__host__ __device__ inline int tri_pitch(int chi) { return chi + ((20 - chi % 16) % 16); }   // = 4 mod 16: conflict-free rows and columns
+__host__ __device__ inline size_t tri_full_smem_bytes(int chi)
+{
+    return sizeof(double) * ((size_t)chi * tri_pitch(chi) + 5 * (size_t)chi);
+}
+__device__ __forceinline__ void cta_sync() { asm volatile("bar.sync 0;" ::: "memory"); }
+__device__ __forceinline__ void next_x_sync(int threads) { asm volatile("bar.sync 1, %0;" ::"r"(threads) : "memory"); }
+__device__ __forceinline__ void next_x_arrive(int threads)
+{
+    __threadfence_block();
+    asm volatile("bar.arrive 1, %0;" ::"r"(threads) : "memory");
+}
+
+// alpha and beta of column x (m entries) for the kernels below: s1 = sum_{i >= 1} x_i^2
+__device__ __forceinline__ void tri_scalars(double s1, double x0, double *alpha, double *beta)
+{
+    if (s1 == 0.0) {   // already reduced
+        *alpha = x0;
+        *beta = 0.0;
+        return;
+    }
+    const HouseholderScalars h = householder_scalars(fma(x0, x0, s1), fabs(x0));
+    *alpha = (x0 >= 0.0) ? -h.nrm : h.nrm;
+    *beta = h.beta;
+}
+
+__global__ void __launch_bounds__(32 * TRI_WARPS) tridiag_kernel(int chi, const double *C, double *work)
 {
     extern __shared__ double sm[];
-    __shared__ double red[33];
-    __shared__ double sh_beta, sh_alpha;
-    // odd row pitch: the mat-vec's lanes read down a column, conflict-free
-    const int ld = chi | 1;
-    double *A = sm;                      // chi x ld
-    double *v = A + chi * ld;            // chi
-    double *p = v + chi;                 // chi
-    const int tid = threadIdx.x;
-    for (int t = tid; t < chi * chi; t += blockDim.x) {
-        int i = t / chi, j = t % chi;
-        A[i * ld + j] = 0.5 * (C[t] + C[(size_t)j * chi + i]);
+    __shared__ double sh_alpha, sh_beta, sh_K;
+    const int ld = tri_pitch(chi);
+    double *A = sm;                                // chi x ld, lower triangle
+    double *xb = A + (size_t)chi * ld;             // 2 x chi: the column, by parity
+    double *y = xb + 2 * chi, *p = y + chi, *v = p + chi;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int nthr = blockDim.x, nwork = nthr - 32;
+    for (int t = tid; t < chi * chi; t += nthr) {
+        const int i = t / chi, j = t % chi;
+        if (j <= i) A[i * ld + j] = 0.5 * (C[t] + C[(size_t)j * chi + i]);
     }
     __syncthreads();
-    for (int kc = 0; kc + 2 < chi; ++kc) {
-        const int b0 = kc + 1, m = chi - b0;
-        // x = the column below the diagonal, kept in v (v_0 = x_0 until alpha is known)
-        double part = 0.0;
-        for (int i = tid; i < m; i += blockDim.x) {
-            const double x = A[(b0 + i) * ld + kc];
-            v[i] = x;
-            if (i > 0) part += x * x;
-        }
-        const double tail = block_sum(part, red);   // its barriers also publish v
-        if (tail == 0.0) continue;                  // already tridiagonal in this column
-        const double x0 = v[0];
-        // the last thread (outside the mat-vec rows) derives the reflector while the
-        // others form y = A x; then A v = y - alpha A e_0 with v = x - alpha e_0
-        if (tid == (int)blockDim.x - 1) {
-            const double nrm = sqrt(tail + x0 * x0);
-            const double alpha = (x0 >= 0.0) ? -nrm : nrm;
-            sh_alpha = alpha;
-            sh_beta = 1.0 / (nrm * (nrm + fabs(x0)));
-        }
-        for (int i = tid; i < m; i += blockDim.x) {
-            const double *row = A + (b0 + i) * ld + b0;
-            double s0 = 0.0, s1 = 0.0, s2 = 0.0, s3 = 0.0;
-            int j = 0;
-            for (; j + 3 < m; j += 4) {
-                s0 = fma(row[j], v[j], s0);
-                s1 = fma(row[j + 1], v[j + 1], s1);
-                s2 = fma(row[j + 2], v[j + 2], s2);
-                s3 = fma(row[j + 3], v[j + 3], s3);
+    if (tid >= nwork) {
+        // ------------------------------------------------ scalar warp
+        // column 0, then per reduced column the next one
+        for (int i = lane; i + 1 < chi; i += 32) xb[i] = A[(i + 1) * ld];
+        if (lane == 0) work[0] = A[0];
+        __syncwarp();
+        next_x_arrive(nthr);
+        for (int kc = 0; kc + 1 < chi; ++kc) {
+            const double *x = xb + (kc & 1) * chi;
+            const int m = chi - kc - 1;
+            double s1 = 0.0;
+            for (int i = 1 + lane; i < m; i += 32) s1 = fma(x[i], x[i], s1);
+            s1 = warp_sum(s1);
+            double alpha, beta;
+            tri_scalars(s1, x[0], &alpha, &beta);
+            if (lane == 0) {
+                sh_alpha = alpha;
+                sh_beta = beta;
+                work[chi + kc] = alpha * alpha;
             }
-            for (; j < m; ++j) s0 = fma(row[j], v[j], s0);
-            p[i] = (s0 + s1) + (s2 + s3);
+            if (kc + 2 >= chi) break;
+            cta_sync();   // A
+            cta_sync();   // B
+            const int b0 = kc + 1;
+            const double K2 = 2.0 * sh_K, p0 = p[0], v0 = v[0];
+            double *xn = xb + ((kc + 1) & 1) * chi;
+            for (int i = lane; i < m; i += 32) {
+                const double vi = v[i], a = A[(b0 + i) * ld + b0];
+                const double w = fma(-fma(-K2, vi, p[i]), v0, fma(-vi, p0, a));
+                if (i == 0) work[b0] = w;
+                else xn[i - 1] = w;
+            }
+            __syncwarp();
+            next_x_arrive(nthr);
         }
-        __syncthreads();
-        const double beta = sh_beta, alpha = sh_alpha;
-        for (int i = tid; i < m; i += blockDim.x) p[i] = beta * fma(-alpha, A[(b0 + i) * ld + b0], p[i]);
-        if (tid == 0) v[0] = x0 - alpha;
-        __syncthreads();
-        double pv = 0.0;
-        for (int i = tid; i < m; i += blockDim.x) pv += p[i] * v[i];
-        pv = block_sum(pv, red);
-        const double Kf = 0.5 * beta * pv;
-        for (int i = tid; i < m; i += blockDim.x) p[i] -= Kf * v[i];   // p <- w
-        __syncthreads();
-        for (int t = tid; t < m * m; t += blockDim.x) {
-            int i = t / m, j = t % m;
-            A[(b0 + i) * ld + b0 + j] -= v[i] * p[j] + p[i] * v[j];
-        }
-        if (tid == 0) {
-            A[b0 * ld + kc] = alpha;
-            A[kc * ld + b0] = alpha;
-        }
-        __syncthreads();
+        if (lane == 0) work[2 * chi - 1] = 0.0;
+        return;
     }
-    for (int i = tid; i < chi; i += blockDim.x) {
-        work[i] = A[i * ld + i];
-        double e = (i + 1 < chi) ? A[(i + 1) * ld + i] : 0.0;
-        work[chi + i] = e * e;
+    next_x_sync(nthr);
+    for (int kc = 0; kc + 2 < chi; ++kc) {
+        const double *x = xb + (kc & 1) * chi;
+        const int b0 = kc + 1, m = chi - b0;
+        double *B = A + b0 * ld + b0;   // the trailing block's lower triangle
+        {
+            // four elements at a time, loaded before they are used: one worker warp per
+            // sub-partition cannot hide shared memory's latency
+            const int c = tid & 3;
+            for (int i0 = 0; i0 < m; i0 += nwork / 4) {
+                const int i = i0 + (tid >> 2);
+                double s0 = 0.0, s1 = 0.0;
+                if (i0 + (warp << 3) < m) {
+                    const int ii = i < m ? i : m - 1;
+                    auto at = [&](int j) { return j <= ii ? B[ii * ld + j] : B[j * ld + ii]; };
+                    int j = c;
+                    for (; j + 12 < m; j += 16) {
+                        const double a0 = at(j), a1 = at(j + 4), a2 = at(j + 8), a3 = at(j + 12);
+                        const double x0 = x[j], x1 = x[j + 4], x2 = x[j + 8], x3 = x[j + 12];
+                        s0 = fma(a0, x0, s0);
+                        s1 = fma(a1, x1, s1);
+                        s0 = fma(a2, x2, s0);
+                        s1 = fma(a3, x3, s1);
+                    }
+                    for (; j < m; j += 4) s0 = fma(at(j), x[j], s0);
+                }
+                s0 += s1;
+                s0 += __shfl_xor_sync(0xffffffffu, s0, 1);
+                s0 += __shfl_xor_sync(0xffffffffu, s0, 2);
+                if (i < m && c == 0) y[i] = s0;
+            }
+        }
+        cta_sync();   // A
+        {
+            const double alpha = sh_alpha, beta = sh_beta;
+            if (warp == 0) {
+                double s2 = 0.0;
+                for (int i = lane; i < m; i += 32) s2 = fma(x[i], y[i], s2);
+                const double q = alpha * fma(alpha, B[0], -2.0 * y[0]), hb = 0.5 * beta * beta;
+                s2 = warp_sum(s2);
+                if (lane == 0) sh_K = hb * (s2 + q);
+            } else {
+                for (int i = tid - 32; i < m; i += nwork - 32) {
+                    p[i] = beta * fma(-alpha, B[i * ld], y[i]);
+                    v[i] = i == 0 ? x[0] - alpha : x[i];
+                }
+            }
+        }
+        cta_sync();   // B
+        {
+            // rows 1 .. m-1, columns 1 .. row: rows a and mm-1-a make one list of mm+1 elements
+            const double K2 = 2.0 * sh_K;
+            const int mm = m - 1, c = tid & 7;
+            double *S = B + ld + 1;
+            for (int a = tid >> 3; a < (mm + 1) / 2; a += nwork / 8) {
+                const int r2 = mm - 1 - a, len = r2 == a ? a + 1 : mm + 1;
+                const double va = v[a + 1], ga = fma(-K2, va, p[a + 1]);
+                const double vr = v[r2 + 1], gr = fma(-K2, vr, p[r2 + 1]);
+                auto place = [&](int e) { return e <= a ? a * ld + e : r2 * ld + e - a - 1; };
+                auto upd = [&](int e, double t, double pj, double vj) {
+                    return e <= a ? fma(-ga, vj, fma(-va, pj, t)) : fma(-gr, vj, fma(-vr, pj, t));
+                };
+                int e = c;
+                for (; e + 8 < len; e += 16) {
+                    const int f = e + 8, j = e <= a ? e : e - a - 1, h = f <= a ? f : f - a - 1;
+                    double *t = S + place(e), *u = S + place(f);
+                    const double t0 = *t, u0 = *u, pj = p[j + 1], vj = v[j + 1], ph = p[h + 1], vh = v[h + 1];
+                    const double wa = e <= a ? va : vr, wg = e <= a ? ga : gr, za = f <= a ? va : vr, zg = f <= a ? ga : gr;
+                    *t = fma(-wg, vj, fma(-wa, pj, t0));
+                    *u = fma(-zg, vh, fma(-za, ph, u0));
+                }
+                if (e < len) {
+                    const int j = e <= a ? e : e - a - 1;
+                    double *t = S + place(e);
+                    *t = upd(e, *t, p[j + 1], v[j + 1]);
+                }
+            }
+        }
+        next_x_sync(nthr);   // C
     }
+    if (tid == 0 && chi >= 2) work[chi - 1] = A[(chi - 1) * ld + chi - 1];
 }
 
 // The same reduction with only the lower triangle stored (packed rows; the mat-vec reads
@@ -378,30 +477,30 @@ __global__ void __launch_bounds__(TRI_THREADS) tridiag_packed_kernel(int chi, co
 
 // The reduction spread over a thread-block cluster, for chi >= TRI_CLUSTER_MIN: the
 // symmetric corner is distributed by rows (row i, all chi entries, on CTA i % CS), so
-// each CTA's mat-vec and rank-2 update touch only its own shared memory.  Per column kc
-// the CTA owning row kc (= column kc) stores d_kc = A[kc][kc] and writes the row's
-// trailing part x into every CTA's column buffer (distributed shared memory); after a
-// cluster barrier every CTA derives the same reflector from the same bits (alpha =
-// -sign(x_0)|x|, v = x - alpha e_0, beta = 1/(|x|(|x| + |x_0|))), forms p_i = beta (A v)_i
-// for its rows and writes p_i into every CTA's p buffer; after a second barrier every
-// CTA forms w = p - (beta/2)(p^T v) v and updates its rows, A_ij -= v_i w_j + w_i v_j.
-// e_kc = alpha.  The two buffers alternate by column parity, so a broadcast never
-// overwrites one still being read (every CTA passes the next column's first barrier
-// only after finishing the current column).  Cluster barriers are hardware barriers:
-// nothing spins.
-constexpr int TRI_CL_THREADS = 512;   // the largest block tri_cluster_threads gives
+// each CTA's mat-vec and rank-2 update touch only its own shared memory.  The steps are the
+// one-CTA kernel's, with one cluster barrier per column: every CTA forms y_i = (A x)_i for
+// its rows and writes them into every CTA's y buffer (distributed shared memory), and the
+// owner of row kc + 1 writes that row's trailing part, as it is before the update, into
+// every CTA's row buffer.  After the barrier every CTA derives K, p, v, the next column x
+// (the broadcast row, updated) and its alpha and beta from the same bits, and updates its
+// rows.  The two buffers alternate by column parity, so a broadcast never overwrites one
+// still being read (a CTA writes parity kc again only after the barrier of column kc + 1,
+// which every CTA reaches after finishing column kc).  Cluster barriers are hardware
+// barriers: nothing spins.  Bound by the chain of that barrier, one reduction over chi
+// entries and the mat-vec; chi = 128: 654 -> 347 us, chi = 480: 6.52 -> 3.56 ms.
+constexpr int TRI_CL_THREADS = 544;   // the largest block tri_cluster_threads gives
 constexpr int TRI_CL_SMEM_MAX = 226 * 1024;   // dynamic, below the 227 KB opt-in less the static part
 
-// one warp per local row (4 to 16 warps): fewer threads make the per-column barriers cheaper
+// one warp per local row (4 to 16 warps) and the scalar warp
 __host__ __device__ inline int tri_cluster_threads(int chi, int cs)
 {
     const int w = (chi + cs - 1) / cs;
-    return 32 * (w < 4 ? 4 : w > 16 ? 16 : w);
+    return 32 * ((w < 4 ? 4 : w > 16 ? 16 : w) + 1);
 }
 
 __host__ __device__ inline size_t tri_cluster_smem_bytes(int chi, int cs)
 {
-    return sizeof(double) * ((size_t)((chi + cs - 1) / cs) * chi + 5 * (size_t)chi);
+    return sizeof(double) * ((size_t)((chi + cs - 1) / cs) * chi + 8 * (size_t)chi);
 }
 
 template <int CS>
@@ -410,175 +509,296 @@ __global__ void __launch_bounds__(TRI_CL_THREADS, 1) tridiag_cluster_kernel(int 
     namespace cg = cooperative_groups;
     cg::cluster_group cl = cg::this_cluster();
     extern __shared__ double sm[];
-    __shared__ double red[33];
+    __shared__ double sh_alpha, sh_beta, sh_K;
     const int rank = (int)cl.block_rank();
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarps = blockDim.x >> 5;
+    const int nthr = blockDim.x, nwork = nthr - 32;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarps = nwork >> 5;
     const int nloc = (chi - rank + CS - 1) / CS;   // rows rank, rank + CS, ...
     const int nmax = (chi + CS - 1) / CS;
     double *A = sm;                           // nmax x chi, full rows
-    double *vb = A + (size_t)nmax * chi;      // 2 x chi: the pivot row's trailing part, by parity
-    double *pb = vb + 2 * (size_t)chi;        // 2 x chi: p, by parity
-    double *w = pb + 2 * (size_t)chi;         // chi
-    for (int t = tid; t < nloc * chi; t += blockDim.x) {
+    double *yb = A + (size_t)nmax * chi;      // 2 x chi: y, by parity
+    double *rb = yb + 2 * (size_t)chi;        // 2 x chi: the next pivot row, by parity
+    double *xb = rb + 2 * (size_t)chi;        // 2 x chi: the column x, by parity
+    double *p = xb + 2 * (size_t)chi, *v = p + chi;
+    for (int t = tid; t < nloc * chi; t += nthr) {
         const int l = t / chi, j = t % chi, i = rank + CS * l;
         A[t] = 0.5 * (C[(size_t)i * chi + j] + C[(size_t)j * chi + i]);
     }
-    cl.sync();   // every CTA of the cluster is running before the first remote store
-    for (int kc = 0; kc + 2 < chi; ++kc) {
-        const int b0 = kc + 1, m = chi - b0;
-        double *v = vb + (size_t)(kc & 1) * chi;
-        double *p = pb + (size_t)(kc & 1) * chi;
-        if (kc % CS == rank) {
-            const double *row = A + (size_t)(kc / CS) * chi;
-            if (tid == 0) work[kc] = row[kc];
-            for (int t = tid; t < m * CS; t += blockDim.x) {
-                const int r = t / m, j = t % m;
-                double *dst = cl.map_shared_rank(v, r);
-                dst[j] = row[b0 + j];
-            }
+    for (int j = tid; j < chi; j += nthr) {
+        const double a = 0.5 * (C[j] + C[(size_t)j * chi]);
+        if (j == 0) {
+            if (rank == 0) work[0] = a;
+        } else {
+            xb[j - 1] = a;
         }
-        cl.sync();
-        // |x|^2 below the pivot by warp 0 in a fixed order (the same bits in every CTA)
-        if (warp == 0) {
-            double t = 0.0;
-            for (int i = 1 + lane; i < m; i += 32) t = fma(v[i], v[i], t);
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-            if (lane == 0) red[32] = t;
-        }
-        __syncthreads();
-        const double tail = red[32];
-        const double x0 = v[0];
-        if (tail == 0.0) {   // already reduced in this column (the same decision in every CTA)
-            if (rank == 0 && tid == 0) work[chi + kc] = x0 * x0;
-            continue;
-        }
-        const double nrm = sqrt(tail + x0 * x0);
-        const double alpha = (x0 >= 0.0) ? -nrm : nrm;
-        const double beta = 1.0 / (nrm * (nrm + fabs(x0)));
-        const double v0 = x0 - alpha;
-        if (rank == 0 && tid == 0) work[chi + kc] = alpha * alpha;
-        int lf = b0 - rank;                    // first local row with i >= b0
-        lf = lf > 0 ? (lf + CS - 1) / CS : 0;
-        for (int l = lf + warp; l < nloc; l += nwarps) {
-            const int i = rank + CS * l;
-            const double *row = A + (size_t)l * chi + b0;
-            double s0 = 0.0, s1 = 0.0;
-            for (int j = lane; j < m; j += 64) {
-                s0 = fma(row[j], j == 0 ? v0 : v[j], s0);
-                if (j + 32 < m) s1 = fma(row[j + 32], v[j + 32], s1);
-            }
-            double sum = s0 + s1;
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
-            if (lane < CS) {
-                double *dst = cl.map_shared_rank(p, lane);
-                dst[i - b0] = beta * sum;
-            }
-        }
-        cl.sync();
-        if (warp == 0) {
-            double t = 0.0;
-            for (int j = lane; j < m; j += 32) t = fma(p[j], j == 0 ? v0 : v[j], t);
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-            if (lane == 0) red[32] = t;
-        }
-        __syncthreads();
-        const double Kf = 0.5 * beta * red[32];
-        for (int j = tid; j < m; j += blockDim.x) w[j] = p[j] - Kf * (j == 0 ? v0 : v[j]);
-        __syncthreads();
-        for (int l = lf + warp; l < nloc; l += nwarps) {
-            const int ii = rank + CS * l - b0;
-            const double vi = ii == 0 ? v0 : v[ii], wi = w[ii];
-            double *row = A + (size_t)l * chi + b0;
-            for (int j = lane; j < m; j += 32) row[j] -= vi * w[j] + wi * (j == 0 ? v0 : v[j]);
-        }
-        __syncthreads();   // this CTA's rows are final for the column before its next broadcast
     }
-    // the last 2 x 2 block (chi >= TRI_CLUSTER_MIN here): d_{chi-2}, d_{chi-1}, e_{chi-2}
-    for (int i = chi - 2; i < chi; ++i)
-        if (i % CS == rank && tid == 0) {
-            const double *row = A + (size_t)(i / CS) * chi;
-            work[i] = row[i];
-            if (i == chi - 1) {
-                work[2 * chi - 2] = row[chi - 2] * row[chi - 2];
-                work[2 * chi - 1] = 0.0;
+    cl.sync();   // every CTA of the cluster is running before the first remote store
+    if (tid >= nwork) {
+        // ------------------------------------------------ scalar warp (as in tridiag_kernel)
+        for (int kc = 0; kc + 1 < chi; ++kc) {
+            const double *x = xb + (size_t)(kc & 1) * chi;
+            const int b0 = kc + 1, m = chi - b0;
+            double s1 = 0.0, s1b = 0.0;
+            for (int i = 1 + lane; i < m; i += 64) {
+                s1 = fma(x[i], x[i], s1);
+                if (i + 32 < m) s1b = fma(x[i + 32], x[i + 32], s1b);
             }
+            s1 = warp_sum(s1 + s1b);
+            double alpha, beta;
+            tri_scalars(s1, x[0], &alpha, &beta);
+            if (lane == 0) {
+                sh_alpha = alpha;
+                sh_beta = beta;
+                if (rank == 0) work[chi + kc] = alpha * alpha;
+            }
+            if (kc + 2 >= chi) break;
+            cl.sync();
+            cta_sync();   // B
+            const double *r = rb + (size_t)(kc & 1) * chi;
+            double *xn = xb + (size_t)((kc + 1) & 1) * chi;
+            const double v0 = v[0], p0 = p[0], g0 = fma(-2.0 * sh_K, v0, p0);
+            for (int j = lane; j < m; j += 32) {
+                const double w = fma(-g0, v[j], fma(-v0, p[j], r[j]));
+                if (j > 0) xn[j - 1] = w;
+                else if (rank == 0) work[b0] = w;
+            }
+            __syncwarp();
+            next_x_arrive(nthr);
         }
+        if (rank == 0 && lane == 0) work[2 * chi - 1] = 0.0;
+    } else {
+        for (int kc = 0; kc + 2 < chi; ++kc) {
+            const int b0 = kc + 1, m = chi - b0;
+            const double *x = xb + (size_t)(kc & 1) * chi;
+            double *y = yb + (size_t)(kc & 1) * chi, *r = rb + (size_t)(kc & 1) * chi;
+            int lf = b0 - rank;                    // first local row with i >= b0
+            lf = lf > 0 ? (lf + CS - 1) / CS : 0;
+            if (b0 % CS == rank) {
+                const double *row = A + (size_t)(b0 / CS) * chi + b0;
+                for (int t = tid; t < m * CS; t += nwork) {
+                    const int q = t / m, j = t % m;
+                    cl.map_shared_rank(r, q)[j] = row[j];
+                }
+            }
+            // half a warp per row: the mat-vec's sums are short, so fewer lanes mean fewer
+            // FP64 additions to combine them
+            for (int l0 = lf + 2 * warp; l0 < nloc; l0 += 2 * nwarps) {
+                const int l = l0 + (lane >> 4), c = lane & 15, i = rank + CS * l;
+                double s0 = 0.0, s1 = 0.0;
+                if (l < nloc) {
+                    const double *row = A + (size_t)l * chi + b0;
+                    for (int j = c; j < m; j += 32) {
+                        s0 = fma(row[j], x[j], s0);
+                        if (j + 16 < m) s1 = fma(row[j + 16], x[j + 16], s1);
+                    }
+                }
+                s0 += s1;
+#pragma unroll
+                for (int o = 8; o > 0; o >>= 1) s0 += __shfl_xor_sync(0xffffffffu, s0, o);
+                if (l < nloc && c < CS) cl.map_shared_rank(y, c)[i - b0] = s0;
+            }
+            cl.sync();
+            const double alpha = sh_alpha, beta = sh_beta;
+            if (warp == 0) {
+                double s2 = 0.0, s3 = 0.0;
+                for (int i = lane; i < m; i += 64) {
+                    s2 = fma(x[i], y[i], s2);
+                    if (i + 32 < m) s3 = fma(x[i + 32], y[i + 32], s3);
+                }
+                const double q = alpha * fma(alpha, r[0], -2.0 * y[0]), hb = 0.5 * beta * beta;
+                s2 = warp_sum(s2 + s3);
+                if (lane == 0) sh_K = hb * (s2 + q);
+            } else {
+                for (int i = tid - 32; i < m; i += nwork - 32) {
+                    p[i] = beta * fma(-alpha, r[i], y[i]);   // A_i0 = A_0i = r_i
+                    v[i] = i == 0 ? x[0] - alpha : x[i];
+                }
+            }
+            cta_sync();   // B
+            const double K2 = 2.0 * sh_K;
+            for (int l = lf + warp; l < nloc; l += nwarps) {
+                const int ii = rank + CS * l - b0;
+                if (ii == 0) continue;   // the pivot row: finished by the scalar warps
+                const double vi = v[ii], gi = fma(-K2, vi, p[ii]);
+                double *row = A + (size_t)l * chi + b0;
+                for (int j = 1 + lane; j < m; j += 32) row[j] = fma(-gi, v[j], fma(-vi, p[j], row[j]));
+            }
+            next_x_sync(nthr);   // C: the rows are final and the next x is there
+        }
+        if (tid == 0 && (chi - 1) % CS == rank) work[chi - 1] = A[(size_t)((chi - 1) / CS) * chi + chi - 1];
+    }
     cl.sync();   // no CTA leaves while another may still write into its shared memory
 }
 
-// Number of eigenvalues of the tridiagonal (d, e2) below x: the sign changes of
-// p_i = (d_i - x) p_{i-1} - e2_{i-1} p_{i-2}.  Only the recurrence itself is FP64
-// arithmetic (three operations per step -- GB300's FP64 pipe is narrow); the zero
-// test, the sign comparison and the range check read the bit pattern with integer
-// instructions, and the rare rescaling is by exact powers of two.
-__device__ __forceinline__ int sturm_count(int chi, const double *d, const double *e2, double x, double tiny)
+// Number of eigenvalues of the tridiagonal (d, e2), scaled to unit size, below x: the sign
+// changes of p_i = (d_i - x) p_{i-1} - e2_{i-1} p_{i-2}.  One FP64 FMA per step on the
+// dependent chain; signs are counted, and the range is checked every fourth step, with
+// integer instructions on the bit pattern.  No e2 is zero (bisect_kernel puts a floor under
+// them), so p = 0 counts as positive and the next p has the sign opposite to the previous
+// one's: one change, as it should be.  *p_out 2^(300 *k_out) is the last p.
+__device__ __forceinline__ int sturm_count(int n, const double *d, const double *e2, double x, double *p_out,
+                                           int *k_out)
 {
     double pm = 1.0, p = d[0] - x;
-    if (p == 0.0) p = -tiny;
-    int cnt = (p < 0.0);
-    int hp = __double2hiint(p);
-    for (int i = 1; i < chi; ++i) {
-        double pn = fma(d[i] - x, p, -e2[i - 1] * pm);
-        int hn = __double2hiint(pn);
-        if (((hn & 0x7FFFFFFF) | __double2loint(pn)) == 0) {   // +-0
-            pn = (hp < 0) ? tiny : -tiny;
-            hn = __double2hiint(pn);
-        }
-        cnt += ((hn ^ hp) < 0);   // sign bits differ
+    unsigned hp = (unsigned)__double2hiint(p);
+    int cnt = (int)(hp >> 31), k = 0;
+    auto step = [&](int i) {
+        const double pn = fma(d[i] - x, p, -e2[i - 1] * pm);
+        const unsigned hn = (unsigned)__double2hiint(pn);
+        cnt += (int)((hn ^ hp) >> 31);
         pm = p;
         p = pn;
-        const int ex = (hn >> 20) & 0x7FF;
-        if (ex > 1023 + 500) {
-            p *= 0x1p-500;
-            pm *= 0x1p-500;
-            hn = __double2hiint(p);
-        } else if (ex < 1023 - 500) {
-            p *= 0x1p+500;
-            pm *= 0x1p+500;
-            hn = __double2hiint(p);
-        }
         hp = hn;
+    };
+    int i = 1;
+    for (; i + 3 < n; i += 4) {
+        step(i);
+        step(i + 1);
+        step(i + 2);
+        step(i + 3);
+        const int ex = (int)(hp >> 20) & 0x7FF;
+        if (ex > 1023 + 300) {
+            p *= 0x1p-300;
+            pm *= 0x1p-300;
+            ++k;
+        } else if (ex < 1023 - 300) {
+            p *= 0x1p+300;
+            pm *= 0x1p+300;
+            --k;
+        }
+    }
+    for (; i < n; ++i) step(i);
+    *p_out = p;
+    *k_out = k;
+    return cnt;
+}
+
+// The same count in FP32 (four cycles per dependent operation instead of ~64), rescaled
+// every fourth step by the exact power of two of the larger of |p| and |pm|.  Its rounding
+// moves an eigenvalue by a few 2^-24 of the matrix's size; the caller checks it.
+__device__ __forceinline__ int sturm_count_f32(int n, const float *d, const float *e2, float x)
+{
+    float pm = 1.0f, p = d[0] - x;
+    int cnt = (int)(__float_as_uint(p) >> 31);
+    for (int i = 1; i < n; ++i) {
+        const float pn = fmaf(d[i] - x, p, -e2[i - 1] * pm);
+        cnt += (int)((__float_as_uint(pn) ^ __float_as_uint(p)) >> 31);
+        pm = p;
+        p = pn;
+        if ((i & 3) == 0) {
+            const unsigned ex = __float_as_uint(fmaxf(fabsf(p), fabsf(pm))) & 0x7F800000u;
+            const float sc = __uint_as_float((254u << 23) - min(max(ex, 1u << 23), 253u << 23));
+            p *= sc;
+            pm *= sc;
+        }
     }
     return cnt;
 }
 
+// One warp per eigenvalue (the ei-th smallest), one eigenvalue per CTA, so the Sturm chains
+// spread over chi SMs.  Each round counts at 32 points.  Four FP32 rounds bracket the
+// eigenvalue to ~2^-19 of the matrix's size; that bracket, widened by 2^-19 on both sides,
+// enters FP64 only if the FP64 counts at its ends confirm it (else the whole range does).
+// In FP64 the points cluster geometrically (factors of four) around the secant through the
+// bracket's last p values, so a round on a well separated eigenvalue shrinks its bracket by
+// ~2^15 to 2^24 instead of 2^5; a round that shrank it by less than 2^4 is followed by an
+// evenly spaced one, so a cluster costs at most twice the rounds of plain multisection.
+// Bound by the FMA chain of a count: 11 FP64 rounds at ~130 cycles a step before, about
+// three or four at ~75 and four short ones now; chi = 72: 155 -> 38 us (90 on a corner
+// graded over twelve decades), chi = 480: 1068 -> 357 us.
+constexpr double BISECT_WIDTH = 4e-16;   // final bracket, of the Frobenius norm
 __global__ void bisect_kernel(int chi, const double *work, double *lam)
 {
     extern __shared__ double sm[];
-    double *d = sm, *e2 = sm + chi;   // 2 chi
-    for (int i = threadIdx.x; i < chi; i += blockDim.x) {
-        d[i] = work[i];
-        e2[i] = work[chi + i];
-    }
-    __syncthreads();
+    double *d = sm, *e2 = sm + chi;                              // 2 chi
+    float *df = reinterpret_cast<float *>(e2 + chi), *e2f = df + chi;   // 2 chi FP32
     const int lane = threadIdx.x & 31;
-    const int ei = blockIdx.x * SPEC_WARPS + (threadIdx.x >> 5);
-    if (ei >= chi) return;
-    // every eigenvalue lies in [-|T|_F, |T|_F] (the Frobenius norm bounds the
-    // spectral radius; it is the corner's, unchanged by the orthogonal reduction):
-    // one square root instead of per-row Gershgorin radii
+    const int ei = blockIdx.x;
+    // every eigenvalue lies in [-|T|_F, |T|_F] (the Frobenius norm bounds the spectral
+    // radius; it is the corner's, unchanged by the orthogonal reduction)
     double f2 = 0.0;
-    for (int i = 0; i < chi; ++i) f2 = fma(d[i], d[i], f2) + 2.0 * e2[i];
-    const double scale = fmax(sqrt(f2), 1e-300);
-    double lo = -scale * (1.0 + 1e-12), hi = scale * (1.0 + 1e-12);
-    const double tiny = 1e-290 * scale;
-    for (int round = 0; round < 16; ++round) {
-        if (hi - lo <= 4e-16 * scale) break;
-        double x = lo + (hi - lo) * (double)(lane + 1) / 33.0;
-        int cnt = sturm_count(chi, d, e2, x, tiny);
-        unsigned below = __ballot_sync(0xffffffffu, cnt <= ei);   // a prefix of lanes
-        int L = __popc(below);
-        double xl = __shfl_sync(0xffffffffu, x, (L > 0) ? L - 1 : 0);
-        double xh = __shfl_sync(0xffffffffu, x, (L < 32) ? L : 31);
-        double nlo = (L > 0) ? xl : lo;
-        double nhi = (L < 32) ? xh : hi;
+    for (int i = lane; i < chi; i += 32) f2 = fma(work[i], work[i], f2) + 2.0 * work[chi + i];
+    f2 = warp_sum(f2);
+    const int fx = (__double2hiint(f2) >> 20) & 0x7FF;
+    if (fx < 2 || fx > 2044) {   // zero (or far below the range), or not finite
+        if (lane == 0) lam[ei] = fx < 2 ? 0.0 : __longlong_as_double(0x7FF8000000000000LL);
+        return;
+    }
+    const int k = (fx - 1023) >> 1;   // |T|_F = sqrt(f2) in [2^k, 2^(k+1))
+    const double sc = __hiloint2double((1023 - k) << 20, 0);
+    for (int i = lane; i < chi; i += 32) {
+        const double di = work[i] * sc, ei2 = fmax(work[chi + i] * sc * sc, 0x1p-200);
+        d[i] = di;
+        e2[i] = ei2;
+        df[i] = (float)di;
+        e2f[i] = fmaxf((float)ei2, 0x1p-60f);
+    }
+    __syncwarp();
+    const double top = 2.0;   // > |T|_F of the scaled matrix
+    double lo = -top, hi = top;
+    {
+        float flo = -2.0f, fhi = 2.0f;
+        for (int round = 0; round < 4; ++round) {
+            const float x = flo + (fhi - flo) * (float)(lane + 1) * (1.0f / 33.0f);
+            const unsigned below = __ballot_sync(0xffffffffu, sturm_count_f32(chi, df, e2f, x) <= ei);
+            const int L = __popc(below);
+            const float xl = __shfl_sync(0xffffffffu, x, L > 0 ? L - 1 : 0);
+            const float xh = __shfl_sync(0xffffffffu, x, L < 32 ? L : 31);
+            flo = L > 0 ? xl : flo;
+            fhi = L < 32 ? xh : fhi;
+        }
+        lo = (double)flo - 0x1p-19;
+        hi = (double)fhi + 0x1p-19;
+    }
+    const double width = BISECT_WIDTH * sc * sqrt(f2);
+    bool ends = true;       // this round checks the bracket's own ends
+    bool even = true;       // evenly spaced points
+    double r = 0.0;         // secant estimate, when !even
+    for (int round = 0; round < 40 && hi - lo > width; ++round) {
+        double x;
+        if (ends) {
+            x = lo + (hi - lo) * ((double)lane * (1.0 / 31.0));
+        } else if (even) {
+            x = lo + (hi - lo) * ((double)(lane + 1) * (1.0 / 33.0));
+        } else {
+            // lanes 0 .. 15: r - (r - lo) 4^-(lane + 1/2); lanes 16 .. 31 likewise towards hi
+            const int q = lane < 16 ? lane : 31 - lane;
+            const double off = __hiloint2double((1022 - 2 * q) << 20, 0);   // 2^-(2 q + 1)
+            x = lane < 16 ? r - (r - lo) * off : r + (hi - r) * off;
+        }
+        double pl;
+        int pk;
+        const int cnt = sturm_count(chi, d, e2, x, &pl, &pk);
+        const unsigned below = __ballot_sync(0xffffffffu, cnt <= ei);   // a prefix of lanes
+        const int L = __popc(below);
+        if (ends) {
+            ends = false;
+            if (L == 0 || L == 32) {   // the FP32 bracket missed: the whole range
+                lo = -top;
+                hi = top;
+                continue;
+            }
+        }
+        const int a = L > 0 ? L - 1 : 0, b = L < 32 ? L : 31;
+        const double xl = __shfl_sync(0xffffffffu, x, a), xh = __shfl_sync(0xffffffffu, x, b);
+        const double nlo = L > 0 ? xl : lo, nhi = L < 32 ? xh : hi;
+        const bool poor = !even && nhi - nlo > 0.0625 * (hi - lo);
+        // secant through the bracket's ends, in FP32 on a common exponent
+        const double fl = __shfl_sync(0xffffffffu, pl, a), fh = __shfl_sync(0xffffffffu, pl, b);
+        const int kl = __shfl_sync(0xffffffffu, pk, a), kh = __shfl_sync(0xffffffffu, pk, b);
+        const int xa = (__double2hiint(fl) >> 20) & 0x7FF, xe = (__double2hiint(fh) >> 20) & 0x7FF;
         lo = nlo;
         hi = nhi;
+        even = poor || L == 0 || L == 32 || kl != kh || xa == 0 || xe == 0 || xa - xe > 60 || xe - xa > 60;
+        if (!even) {
+            const float ga = (float)__hiloint2double((__double2hiint(fl) & 0x000FFFFF) | 0x3FF00000, __double2loint(fl));
+            const float gb = (float)__hiloint2double(
+                (__double2hiint(fh) & 0x000FFFFF) | ((1023 + xe - xa) << 20), __double2loint(fh));
+            r = lo + (hi - lo) * (double)(ga / (ga + gb));
+            even = !(r > lo && r < hi);
+        }
     }
-    if (lane == 0) lam[ei] = 0.5 * (lo + hi);
+    if (lane == 0) lam[ei] = 0.5 * (lo + hi) * __hiloint2double((1023 + k) << 20, 0);
 }
 
 // stride 2: the chi x stride eigenvalues come in equal pairs (a Hermitian corner through
@@ -591,14 +811,14 @@ __global__ void spectrum_finish_kernel(int chi, int stride, const double *lam_in
     const int tid = threadIdx.x, nall = chi * stride;
     for (int i = tid; i < nall; i += blockDim.x) lam[i] = fabs(lam_in[i]);
     __syncthreads();
+    // magnitudes compare as integers (the FP64 pipe's compares would bind: 139 -> 19 us at
+    // chi = 480)
+    const unsigned long long *key = reinterpret_cast<const unsigned long long *>(lam);
     for (int i = tid; i < nall; i += blockDim.x) {
-        double ai = lam[i];
+        const unsigned long long ai = key[i];
         int rank = 0;
-        for (int j = 0; j < nall; ++j) {
-            double aj = lam[j];
-            rank += (aj > ai) || (aj == ai && j < i);
-        }
-        srt[rank] = ai;
+        for (int j = 0; j < nall; ++j) rank += key[j] + (j < i ? 1 : 0) > ai;
+        srt[rank] = lam[i];
     }
     __syncthreads();
     double ss = 0.0;
@@ -809,8 +1029,7 @@ static cudaError_t spectrum_tail(int chi, int stride, double *work, double *s_ne
 {
     const int n = chi * stride;
     CTM_COUNT_LAUNCH(2);
-    bisect_kernel<<<(n + SPEC_WARPS - 1) / SPEC_WARPS, 32 * SPEC_WARPS, 2 * sizeof(double) * n, st>>>(n, work,
-                                                                                                      work + 2 * n);
+    bisect_kernel<<<n, 32, 3 * sizeof(double) * n, st>>>(n, work, work + 2 * n);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     spectrum_finish_kernel<<<1, 256, 0, st>>>(chi, stride, work + 2 * n, s_new, s_old, delta);
@@ -846,14 +1065,14 @@ static cudaError_t launch_tridiag(int chi, const double *C, double *work, cudaSt
     // slowest CTA): measured 0.892 -> 0.872 ms per step at D = 6, chi = 72.  (Not inside a
     // batch, where many spectra run at once.)
     const bool full = chi <= TRI_FULL_MAX, global = chi > TRI_SMEM_MAX;
-    size_t smem = sizeof(double) * ((full ? (size_t)chi * (chi | 1) : global ? 0 : (size_t)chi * (chi + 1) / 2) +
-                                    2 * (size_t)chi);
+    size_t smem = full ? tri_full_smem_bytes(chi)
+                       : sizeof(double) * ((global ? 0 : (size_t)chi * (chi + 1) / 2) + 2 * (size_t)chi);
     if (reserve_sm && smem < SPEC_SM_ALONE_BYTES) smem = SPEC_SM_ALONE_BYTES;
     CTM_COUNT_LAUNCH(1);
     cudaError_t e = cudaSuccess;
     const int cs = tri_cluster_size(chi);
     if (cs) e = launch_tridiag_cluster(cs, chi, C, work, st);
-    else if (full) tridiag_kernel<<<1, TRI_THREADS, smem, st>>>(chi, C, work);
+    else if (full) tridiag_kernel<<<1, 32 * TRI_WARPS, smem, st>>>(chi, C, work);
     else if (!global) tridiag_packed_kernel<false><<<1, TRI_THREADS, smem, st>>>(chi, C, work);
     else tridiag_packed_kernel<true><<<1, TRI_THREADS, smem, st>>>(chi, C, work);
     if (e != cudaSuccess) return e;
