@@ -29,11 +29,20 @@
 // reflectors v_j as the columns of V and S = V^T V, the triangular factor
 // satisfies T^{-1} = striu(S) + diag(S)/2 (the "UT" form of the product of
 // reflectors), so Q = E - V W with W = T V_top^T.  Every CTA adds its rows' share
-// of S with FP64 atomics; after a grid barrier ceil(k/8) CTAs solve eight columns
+// of S with FP64 atomics; after a grid barrier ceil(k/4) CTAs solve four columns
 // of W each (blocked back-substitution with inverted 8 x 8 diagonal blocks); after
 // a second barrier every CTA forms its rows of Q and applies the gauge (columns
 // with R_jj < 0 negated, and the rows of R with them).  The grid size is tuned
 // once per shape by timing a few rows-per-CTA choices.
+//
+// What bounds it: FP64 instructions, one per warp, 64 cycles and sub-partition, whether or not
+// the next depends on it and whether or not its lanes are predicated off (measured).  So the
+// panel's chain runs in one warp on the QB x QB blocks alone, with the other columns and the
+// rows following it reflector by reflector in other sub-partitions; lanes per column are picked
+// from that cost; partial sums are combined by halving; nothing FP64 sits under a predicate.
+// n x k: 512 x 32 119 -> 66 us, 2592 x 72 307 -> 214 (panels 23k -> 13k cycles each, update and
+// Gram passes 17k -> 8k), 8192 x 128 1027 -> 833, 5184 x 144 987 -> 802, 12000 x 240
+// 2350 -> 1960.
 //
 // The grid barrier is one monotonic counter in global memory; its spin is
 // bounded (about a second) and on expiry sets an error flag that the host
@@ -43,8 +52,10 @@
 // returns.
 #include <cooperative_groups.h>
 #include <cstdlib>
+#include <type_traits>
 
 #include "ctm_internal.h"
+#include "fp64_chain.h"
 
 namespace {
 
@@ -120,7 +131,7 @@ struct QrArgs {
 
 // W = U^{-1} V_top^T with U = striu(S) + diag(S)/2 (unit diagonal where tau = 0).
 // The k right-hand sides are independent: CTA b of the QR grid solves columns
-// [8b, 8b + 8) after the grid barrier that completes S.
+// [4b, 4b + 4) after the grid barrier that completes S.
 // Rows are blocked by QR_WB = 8 from the bottom; every CTA first inverts the
 // diagonal 8 x 8 blocks of U (all blocks at once, one thread per block column),
 // then per row block sums the already solved rows below it (independent dot
@@ -129,8 +140,8 @@ struct QrArgs {
 // block.  U (packed upper triangle), the block inverses and the CTA's W columns
 // live in shared memory.
 constexpr int QR_WB = 8;      // row block (and diagonal inverse) size
-constexpr int QR_WC = 8;      // right-hand-side columns per CTA
-constexpr int QR_WL = 4;      // lanes per dot product in the block update
+constexpr int QR_WC = 4;      // right-hand-side columns per CTA
+constexpr int QR_WL = 8;      // lanes per dot product in the block update
 
 __device__ __forceinline__ int up_off(int k, int i, int j) { return i * k - (i * (i - 1)) / 2 + (j - i); }
 
@@ -249,7 +260,43 @@ __device__ void wy_solve_cta(int k, int cblk, const double *S, const double *V, 
     }
 }
 
-constexpr int QR_QROWS = 8;   // rows per thread and pass in the Q formation
+// RP rows per thread and pass of the Q formation, W from L2 four rows at a time
+template <int RP>
+__device__ void q_rows(const QrArgs &a, const double *alps, const double *Ys, int ld, int r0, int nr)
+{
+    const int k = a.k, grp = blockDim.x / k, col = threadIdx.x % k, g = threadIdx.x / k;
+    if (g >= grp) return;
+    const double sgn = alps[col] < 0.0 ? -1.0 : 1.0;
+    for (int rb = g * RP; rb < nr; rb += grp * RP) {
+        const double *rows[RP];
+        double acc[RP];
+#pragma unroll
+        for (int q = 0; q < RP; ++q) {
+            acc[q] = 0.0;
+            rows[q] = Ys + (size_t)min(rb + q, nr - 1) * ld;
+        }
+        int j = 0;
+        for (; j + 3 < k; j += 4) {
+            double w[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) w[u] = __ldcg(a.W + (size_t)(j + u) * k + col);
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+#pragma unroll
+                for (int q = 0; q < RP; ++q) acc[q] = fma(rows[q][j + u], w[u], acc[q]);
+        }
+        for (; j < k; ++j) {
+            const double w = __ldcg(a.W + (size_t)j * k + col);
+#pragma unroll
+            for (int q = 0; q < RP; ++q) acc[q] = fma(rows[q][j], w, acc[q]);
+        }
+#pragma unroll
+        for (int q = 0; q < RP; ++q) {
+            const int rg = r0 + rb + q;
+            if (rb + q < nr) a.Q[(size_t)rg * k + col] = sgn * ((rg == col ? 1.0 : 0.0) - acc[q]);
+        }
+    }
+}
 
 // GY: the CTA's row block lives in a global slab (L2) instead of shared memory, for
 // blocks too tall for it (large k or n); the algorithm and the access order are the same.
@@ -257,7 +304,10 @@ template <bool GY>
 __global__ void __launch_bounds__(QR_THREADS, 1) qr_kernel(QrArgs a)
 {
     extern __shared__ double sm[];
-    __shared__ int stop_sh[2];
+    __shared__ double pan_sc[QB][3];    // a panel's reflectors: tau, v_0, alpha
+    __shared__ double pan_pc[QB + 1][QB];   // [i][ip]: entry of v_i in the panel's row ip > i (row QB: unused)
+    __shared__ double pan_rr[QB + 1][QB];   // [i][q]: R[j0 + i][j0 + q], q > i (row QB: unused)
+    __shared__ int pan_stop;            // the panel ends before this reflector
     const int k = a.k;
     const int ld = k | 1;   // odd row pitch: a warp reading one column of 16 rows hits 16 distinct bank pairs
     const int c = blockIdx.x;
@@ -269,11 +319,9 @@ __global__ void __launch_bounds__(QR_THREADS, 1) qr_kernel(QrArgs a)
     double *taus = GY ? sm : Ys + (size_t)a.rows_per * ld;          // k
     double *v0s = taus + k;                         // k
     double *alps = v0s + k;                         // k
-    double *g0 = alps + k;                          // QB: squared norms at the panel start
-    double *Gs = g0 + QB;                           // QB x k: panel Gram rows, downdated
-    double *Ps = Gs + QB * k;                       // QB x k: panel rows, updated
+    double *Gs = alps + k;                          // QB x k: panel Gram rows
+    double *Ps = Gs + QB * k;                       // QB x k: panel rows
     double *cfs = Ps + QB * k;                      // QB x k: tau_j v_j^T a_kk
-    double *Rj = cfs + QB * k;                      // k: current row of R
     // (after the factorisation the region from Gs on holds the triangular solve's buffers)
     const bool det = a.gpart != nullptr;
     // atomics: three rotating accumulators; deterministic: this CTA's slot of panel parity blk
@@ -284,6 +332,115 @@ __global__ void __launch_bounds__(QR_THREADS, 1) qr_kernel(QrArgs a)
 
     for (int t = tid; t < nr * k; t += blockDim.x) Ys[(t / k) * ld + t % k] = a.Y[(size_t)r0 * k + t];
     __syncthreads();
+
+    // The sweep of gram_pass below over the columns kk >= j1: P lanes per column share its rows
+    // from local row rs on, two at a time (two independent chains keep the FP64 pipe busy).
+    auto sweep = [&](int j0, int nb, int j1, int nn, int rs, int P, double *acc, double *pub, auto full) {
+        constexpr bool FULL = decltype(full)::value;
+        const int ncols = k - j1, nrow = max(0, nr - rs);
+        const int lg = 31 - __clz(P);
+        auto row_of = [&](int r) { return Ys + (size_t)r * ld; };
+        for (int base = 0; base < ncols * P; base += blockDim.x) {
+            const int t = base + tid;
+            const int kk = j1 + (t >> lg), part = t & (P - 1);
+            double g[QB];
+#pragma unroll
+            for (int i = 0; i < QB; ++i) g[i] = 0.0;
+            if (t < ncols * P) {
+                const bool upd = (FULL || nb > 0) && kk >= j1 + nn;
+                double cf[QB];
+#pragma unroll
+                for (int i = 0; i < QB; ++i) cf[i] = (upd && (FULL || i < nb)) ? cfs[i * k + kk] : 0.0;
+                int r = rs + part;
+                // pairs of rows; the columns of the next panel are updated already (cf = 0)
+                for (; r + P < nr; r += 2 * P) {
+                    double *ra = row_of(r), *rb = row_of(r + P);
+                    double x = ra[kk], y = rb[kk];
+                    if (upd) {
+                        double v[QB], w[QB];
+#pragma unroll
+                        for (int i = 0; i < QB; ++i)
+                            if (FULL || i < nb) {
+                                v[i] = ra[j0 + i];
+                                w[i] = rb[j0 + i];
+                            }
+#pragma unroll
+                        for (int i = 0; i < QB; ++i)
+                            if (FULL || i < nb) {
+                                x = fma(-v[i], cf[i], x);
+                                y = fma(-w[i], cf[i], y);
+                            }
+                        ra[kk] = x;
+                        rb[kk] = y;
+                    }
+#pragma unroll
+                    for (int i = 0; i < QB; ++i)
+                        if (FULL || i < nn) g[i] = fma(ra[j1 + i], x, g[i]);
+#pragma unroll
+                    for (int i = 0; i < QB; ++i)
+                        if (FULL || i < nn) g[i] = fma(rb[j1 + i], y, g[i]);
+                    const int rg = r0 + r;
+                    if (rg < j1 + nn) pub[(rg - j1) * k + kk] = x;
+                    if (rg + P < j1 + nn) pub[(rg + P - j1) * k + kk] = y;
+                }
+                if (r < nr) {
+                    double *ra = row_of(r);
+                    double x = ra[kk];
+                    if (upd) {
+#pragma unroll
+                        for (int i = 0; i < QB; ++i)
+                            if (FULL || i < nb) x = fma(-ra[j0 + i], cf[i], x);
+                        ra[kk] = x;
+                    }
+#pragma unroll
+                    for (int i = 0; i < QB; ++i)
+                        if (FULL || i < nn) g[i] = fma(ra[j1 + i], x, g[i]);
+                    if (r0 + r < j1 + nn) pub[(r0 + r - j1) * k + kk] = x;
+                }
+            }
+            // Combine the P lanes of a column by halving: at each of the first three levels a lane
+            // keeps half of its sums and hands over the other half, 4 + 2 + 1 additions instead of
+            // 8 per level; the sums then sit on different lanes and so do their atomics.
+            int i0 = 0;
+            if (P >= 2) {
+                const bool up = part & 1;
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const double o = __shfl_xor_sync(0xffffffffu, up ? g[i] : g[i + 4], 1);
+                    g[i] = (up ? g[i + 4] : g[i]) + o;
+                }
+                i0 = up ? 4 : 0;
+            }
+            if (P >= 4) {
+                const bool up = part & 2;
+#pragma unroll
+                for (int i = 0; i < 2; ++i) {
+                    const double o = __shfl_xor_sync(0xffffffffu, up ? g[i] : g[i + 2], 2);
+                    g[i] = (up ? g[i + 2] : g[i]) + o;
+                }
+                i0 += up ? 2 : 0;
+            }
+            if (P >= 8) {
+                const bool up = part & 4;
+                const double o = __shfl_xor_sync(0xffffffffu, up ? g[0] : g[1], 4);
+                g[0] = (up ? g[1] : g[0]) + o;
+                i0 += up ? 1 : 0;
+            }
+            if (P >= 16) g[0] += __shfl_xor_sync(0xffffffffu, g[0], 8);
+            if (P >= 32) g[0] += __shfl_xor_sync(0xffffffffu, g[0], 16);
+            const int held = P >= 8 ? 1 : QB >> lg;
+#pragma unroll
+            for (int i = 0; i < QB; ++i) {
+                if (i >= held) break;
+                const int ii = i0 + i;
+                if (t >= ncols * P || (part >> 3) != 0 || ii >= nn) continue;
+                // deterministic: every entry of the panel's rows in this CTA's slot, zero where the
+                // CTA has no rows below the panel
+                if (det) acc[ii * k + kk] = (nrow > 0 && j1 + ii <= kk) ? g[i] : 0.0;
+                else if (nrow > 0 && j1 + ii <= kk) atomicAdd(&acc[ii * k + kk], g[i]);
+            }
+        }
+    };
 
     // Apply the reflectors of the panel at j0 (width nb, coefficients cfs, vectors
     // in the panel columns) to this CTA's rows >= j1 and form the partial Gram
@@ -298,73 +455,42 @@ __global__ void __launch_bounds__(QR_THREADS, 1) qr_kernel(QrArgs a)
         if (nb > 0) {
             for (int t = tid; t < nrow * nn; t += blockDim.x) {
                 const int r = rs + t / nn, col = j1 + t % nn;
-                double s0 = 0.0, s1 = 0.0;
-                for (int i = 0; i < nb; i += 2) {
-                    s0 = fma(Ys[r * ld + j0 + i], cfs[i * k + col], s0);
-                    if (i + 1 < nb) s1 = fma(Ys[r * ld + j0 + i + 1], cfs[(i + 1) * k + col], s1);
+                double *row = Ys + (size_t)r * ld;
+                double v[QB], cf[QB], x = row[col];
+#pragma unroll
+                for (int i = 0; i < QB; ++i) {
+                    v[i] = i < nb ? row[j0 + i] : 0.0;
+                    cf[i] = i < nb ? cfs[i * k + col] : 0.0;
                 }
-                Ys[r * ld + col] -= s0 + s1;
+#pragma unroll
+                for (int i = 0; i < QB; ++i)
+                    if (i < nb) x = fma(-v[i], cf[i], x);
+                row[col] = x;
             }
             __syncthreads();
         }
         const int ncols = k - j1;
+        // Lanes per column, from what the busiest sub-partition issues: 2 QB multiply-adds per row
+        // of a lane (update and Gram sums) and about log2(P) + 6 instructions to combine lanes;
+        // measured per instruction: ~98 cycles with one warp on the sub-partition, 66 with more.
+        // Rows in the slab come from L2, whose latency wants every warp.
         int P = 1;
-        while (P < 32 && P * 2 * ncols <= (int)blockDim.x) P *= 2;
-        for (int base = 0; base < ncols * P; base += blockDim.x) {
-            const int t = base + tid;
-            const int kk = j1 + t / P, part = t % P;
-            double g[QB];
-#pragma unroll
-            for (int i = 0; i < QB; ++i) g[i] = 0.0;
-            if (t < ncols * P) {
-                const bool upd = nb > 0 && kk >= j1 + nn;
-                for (int r = rs + part; r < nr; r += P) {
-                    double x = Ys[r * ld + kk];
-                    if (upd) {
-                        double s0 = 0.0, s1 = 0.0;
-                        for (int i = 0; i < nb; i += 2) {
-                            s0 = fma(Ys[r * ld + j0 + i], cfs[i * k + kk], s0);
-                            if (i + 1 < nb) s1 = fma(Ys[r * ld + j0 + i + 1], cfs[(i + 1) * k + kk], s1);
-                        }
-                        x -= s0 + s1;
-                        Ys[r * ld + kk] = x;
-                    }
-#pragma unroll
-                    for (int i = 0; i < QB; ++i)
-                        if (i < nn && j1 + i <= kk) g[i] = fma(Ys[r * ld + j1 + i], x, g[i]);
-                    const int rg = r0 + r;
-                    if (rg < j1 + nn) pub[(rg - j1) * k + kk] = x;
-                }
-            }
-#pragma unroll
-            for (int i = 0; i < QB; ++i) {
-                double v = g[i];
-                for (int o = P >> 1; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o, P);
-                if (det) {
-                    // this CTA's slot: every entry of the panel's rows written, zero where
-                    // the CTA has no rows below the panel
-                    if (t < ncols * P && part == 0 && i < nn) acc[i * k + kk] = (nrow > 0 && j1 + i <= kk) ? v : 0.0;
-                } else if (t < ncols * P && part == 0 && nrow > 0 && i < nn && j1 + i <= kk) {
-                    atomicAdd(&acc[i * k + kk], v);
+        if (GY) {
+            while (P < 32 && P * 2 * ncols <= (int)blockDim.x) P *= 2;
+        } else {
+            int best = 1 << 30;
+            for (int lg = 0; lg <= 5 && (ncols << lg) <= 2 * (int)blockDim.x; ++lg) {
+                const int w = ((ncols << lg) + 127) >> 7;
+                const int cost = (w == 1 ? 3 : 2 * w) * (2 * QB * ((nrow + (1 << lg) - 1) >> lg) + (lg ? lg + 6 : 0));
+                if (cost < best) {
+                    best = cost;
+                    P = 1 << lg;
                 }
             }
         }
-    };
-
-    // Reflector of column j from its (downdated) squared norm below the diagonal
-    // and its pivot entry: alpha = -sign(x_0)|x|, v_0 = x_0 - alpha,
-    // tau = 2 / v^T v = 1 / (|x| (|x| + |x_0|)).
-    auto reflector = [&](int j, double nrm2, double x0) {
-        const double nrm = sqrt(nrm2);
-        double tau = 0.0, alpha = x0, v0 = 0.0;
-        if (nrm > 0.0) {
-            alpha = (x0 >= 0.0) ? -nrm : nrm;
-            v0 = x0 - alpha;
-            tau = 1.0 / (nrm * (nrm + fabs(x0)));
-        }
-        taus[j] = tau;
-        v0s[j] = v0;
-        alps[j] = (nrm > 0.0) ? alpha : 0.0;
+        // full panels (all but a restart's and the last one's) take straight-line code
+        if (nb == QB && nn == QB) sweep(j0, QB, j1, QB, rs, P, acc, pub, std::true_type());
+        else sweep(j0, nb, j1, nn, rs, P, acc, pub, std::false_type());
     };
 
     int j0 = 0, nn0 = min(QB, k), blk = 0;
@@ -400,68 +526,200 @@ __global__ void __launch_bounds__(QR_THREADS, 1) qr_kernel(QrArgs a)
             double *z = a.sbuf + (size_t)((blk + 2) % 3) * QB * k;
             for (int t = tid; t < QB * k; t += blockDim.x) z[t] = 0.0;
         }
+        if (tid == 0) pan_stop = -1;
         __syncthreads();
-        if (tid < nn0) g0[tid] = Gs[tid * k + j0 + tid];
-        if (tid == 0) {
-            reflector(j0, Gs[j0], Ps[j0]);
-            stop_sh[0] = -1;
-        }
         // ------------------------------------------------ the panel's reflectors
-        // Per column j two passes.  A: thread kk forms cf = tau v^T a_kk and
-        // R[j][kk] from row i (already downdated), and the thread owning column
-        // j+1 derives reflector j+1 right away from its own entries.  B: the later
-        // panel rows and Gram rows are downdated by H_j.
-        int nb = nn0;
-        for (int i = 0; i < nn0; ++i) {
-            __syncthreads();
-            if (stop_sh[i & 1] >= 0) {
-                nb = i;
-                break;
+        // Warp 0 derives them from the panel's QB x QB blocks of G and P alone, a column after
+        // the other: alpha = -sign(x_0)|x|, v_0 = x_0 - alpha, tau = 1 / (|x| (|x| + |x_0|)),
+        // then cf = tau v^T a and R's entries of the panel's later columns, and both blocks
+        // downdated.  Lane (r, q) holds rows r and r + 4 of column q of each block.  As soon as
+        // a reflector is published (shared memory, named barrier i + 1), the outer warps apply
+        // it to their columns kk >= j0 + nn0 -- cf, R and the downdates of the column's QB
+        // entries of G and P, in registers -- while warp 0 works on the next one.  The chain
+        // per column is one pair of Householder scalars and about eight FP64 instructions; the
+        // two-barrier pass over all columns it replaces took 23k cycles a panel at k = 72.
+        const int warp = tid >> 5, lane = tid & 31;
+        const int jo = j0 + nn0, nout = k - jo;       // outer columns
+        const bool pairs = nout <= 64;                // two lanes per column: one G, one P
+        const int cpw = pairs ? 16 : 32;
+        // outer warps, and behind them the row warps, are the warps off warp 0's sub-partition
+        constexpr int OTHERS = 3 * (QR_THREADS >> 5) / 4;
+        const int rs = max(r0, jo) - r0, nrw = (max(0, nr - rs) + 31) / 32;   // rows below the panel
+        const bool pipe_rows = !GY && nrw <= OTHERS / 2;
+        const int now = min((nout + cpw - 1) / cpw, OTHERS - (pipe_rows ? nrw : 0));
+        const int bar_n = 32 * (now + (pipe_rows ? nrw : 0) + 1);
+        const int wi = (warp & 3) ? warp - 1 - (warp >> 2) : -1;   // index among those warps
+        if (warp == 0) {
+            const int r = lane >> 3, q = lane & 7;
+            double P0 = 0.0, P1 = 0.0, G0 = 0.0, G1 = 0.0;
+            if (q < nn0 && r < nn0) {
+                P0 = Ps[r * k + j0 + q];
+                G0 = Gs[r * k + j0 + q];
             }
-            const int j = j0 + i;
-            const double tau = taus[j], v0 = v0s[j], alpha = alps[j];
-            for (int kk = tid; kk < k; kk += blockDim.x) {
-                double rv = (kk == j) ? alpha : 0.0;
-                if (kk > j) {
-                    const double pik = Ps[i * k + kk];
-                    const double cf = tau * (Gs[i * k + kk] - alpha * pik);
-                    rv = pik - v0 * cf;
-                    cfs[i * k + kk] = cf;
-                    Rj[kk] = rv;
-                    if (kk == j + 1 && i + 1 < nn0) {
-                        const double nrm2 = fma(-rv, rv, Gs[(i + 1) * k + kk]);
-                        const double x0 = fma(-Ps[(i + 1) * k + j], cf, Ps[(i + 1) * k + kk]);
-                        int stop = -1;
-                        if (!(nrm2 >= QR_DOWNDATE_MIN * g0[i + 1])) stop = i + 1;   // cancellation
-                        else reflector(kk, nrm2, x0);
-                        stop_sh[(i + 1) & 1] = stop;
+            if (q < nn0 && r + 4 < nn0) {
+                P1 = Ps[(r + 4) * k + j0 + q];
+                G1 = Gs[(r + 4) * k + j0 + q];
+            }
+            int stop = nn0;
+            // One copy of the loop body: unrolled, its instructions would come from beyond the
+            // instruction cache once per panel (measured: the scalars 910 instead of 590 cycles).
+            // Signs and ranges are tested on the bit patterns: an FP64 compare costs as much as
+            // an FMA.  While rows 0 .. 3 are still wanted, the downdate of rows 4 .. 7 waits until
+            // the next column's scalars are under way (pend).
+            const double fresh = q < nn0 ? Gs[q * k + j0 + q] : 0.0;   // the norms at the panel's start
+            bool pend = false;
+            double cf = 0.0, rv = 0.0, pc1 = 0.0, rr1 = 0.0;
+#pragma unroll 1
+            for (int i = 0; i < nn0; ++i) {
+                const int j = j0 + i, src = ((i & 3) << 3) | i;
+                const double nrm2 = __shfl_sync(0xffffffffu, i < 4 ? G0 : G1, src);
+                const double x0 = __shfl_sync(0xffffffffu, i < 4 ? P0 : P1, src);
+                const long long nb2 = __double_as_longlong(nrm2);
+                // cancellation (or NaN): the panel ends here and the next one starts from fresh sums
+                const long long least = __double_as_longlong(__shfl_sync(0xffffffffu, fresh, i)) - (4LL << 52);
+                if (i > 0 && !(nb2 >= least && nb2 <= 0x7FF0000000000000LL && nb2 > 0)) {
+                    stop = i;
+                    break;
+                }
+                const double gi = __shfl_sync(0xffffffffu, i < 4 ? G0 : G1, ((i & 3) << 3) | q);
+                const double pi = __shfl_sync(0xffffffffu, i < 4 ? P0 : P1, ((i & 3) << 3) | q);
+                double tau = 0.0, alpha = 0.0, v0 = 0.0;
+                if (nb2 > 0) {
+                    const HouseholderScalars h = householder_scalars(nrm2, fabs(x0));
+                    alpha = __hiloint2double(__double2hiint(h.nrm) | (~__double2hiint(x0) & (int)0x80000000),
+                                             __double2loint(h.nrm));
+                    v0 = x0 - alpha;
+                    tau = h.beta;
+                }
+                if (pend) {
+                    G1 = fma(-rr1, rv, G1);
+                    P1 = fma(-pc1, cf, P1);
+                    pend = false;
+                }
+                cf = tau * fma(-alpha, pi, gi);
+                rv = fma(-v0, cf, pi);
+                // every lane stores (equal values meet at equal addresses): no divergent branches
+                pan_sc[i][0] = tau;
+                pan_sc[i][1] = v0;
+                pan_sc[i][2] = alpha;
+                pan_pc[q == i ? i : QB][r] = P0;
+                pan_pc[q == i ? i : QB][r + 4] = P1;
+                pan_rr[i][q] = rv;
+                *(q > i && q < nn0 ? cfs + i * k + j0 + q : &pan_rr[QB][0]) = cf;
+                if (bar_n > 32) {
+                    __syncwarp();
+                    asm volatile("bar.arrive %0, %1;" ::"r"(i + 1), "r"(bar_n) : "memory");
+                }
+                pc1 = __shfl_sync(0xffffffffu, P1, (r << 3) | i);
+                rr1 = __shfl_sync(0xffffffffu, rv, r + 4);
+                if (i < 3) {
+                    const double pc = __shfl_sync(0xffffffffu, P0, (r << 3) | i), rr = __shfl_sync(0xffffffffu, rv, r);
+                    G0 = fma(-rr, rv, G0);
+                    P0 = fma(-pc, cf, P0);
+                    pend = true;
+                } else {
+                    G1 = fma(-rr1, rv, G1);
+                    P1 = fma(-pc1, cf, P1);
+                }
+                if (lane == 0) {
+                    taus[j] = tau;
+                    v0s[j] = v0;
+                    alps[j] = alpha;
+                }
+                if (c == 0) {
+                    for (int kk = lane; kk < j0; kk += 32) a.R[(size_t)j * k + kk] = 0.0;
+                    if (r == 0 && q < nn0) a.R[(size_t)j * k + j0 + q] = q < i ? 0.0 : (q == i ? alpha : rv);
+                }
+            }
+            if (lane == 0) pan_stop = stop;
+            if (stop < nn0 && bar_n > 32) {
+                __syncwarp();
+                asm volatile("bar.arrive %0, %1;" ::"r"(stop + 1), "r"(bar_n) : "memory");
+            }
+        } else if (wi >= now && wi < now + nrw && pipe_rows) {
+            // rows below the panel: v_i's entries take the in-panel updates, one thread per row
+            const int rl = rs + (wi - now) * 32 + lane;
+            double *row = Ys + (size_t)min(rl, nr - 1) * ld + j0;
+            double v[QB];
+#pragma unroll
+            for (int i = 0; i < QB; ++i) v[i] = i < nn0 ? row[i] : 0.0;
+            int done = nn0;
+#pragma unroll
+            for (int i = 0; i < QB; ++i) {
+                if (i >= nn0) break;
+                asm volatile("bar.sync %0, %1;" ::"r"(i + 1), "r"(bar_n) : "memory");
+                if (*(volatile int *)&pan_stop == i) {
+                    done = i;
+                    break;
+                }
+#pragma unroll
+                for (int ip = i + 1; ip < QB; ++ip)
+                    if (ip < nn0) v[ip] = fma(-v[i], cfs[i * k + j0 + ip], v[ip]);
+            }
+            if (rl < nr) {
+#pragma unroll
+                for (int i = 1; i < QB; ++i)
+                    if (i < done) row[i] = v[i];
+            }
+        } else if (wi >= 0 && wi < now) {
+            // columns kk, then (more than the warps hold) a second sweep with nothing to wait for
+            for (int sweep = 0, base = wi * cpw; base < nout; ++sweep, base += now * cpw) {
+                const int kk = jo + base + (pairs ? lane >> 1 : lane);
+                const bool in = kk < k, isg = pairs && (lane & 1);
+                double p[QB], g[QB];   // pairs: p holds this lane's entries (of G or of P)
+#pragma unroll
+                for (int i = 0; i < QB; ++i) {
+                    const bool have = in && i < nn0;
+                    p[i] = have ? (isg ? Gs : Ps)[i * k + kk] : 0.0;
+                    g[i] = have && !pairs ? Gs[i * k + kk] : 0.0;
+                }
+#pragma unroll
+                for (int i = 0; i < QB; ++i) {
+                    if (i >= nn0) break;
+                    if (sweep == 0) asm volatile("bar.sync %0, %1;" ::"r"(i + 1), "r"(bar_n) : "memory");
+                    if (*(volatile int *)&pan_stop == i) break;
+                    const double tau = pan_sc[i][0], v0 = pan_sc[i][1], alpha = pan_sc[i][2];
+                    double pi = p[i], gi = g[i];
+                    if (pairs) {
+                        const double o = __shfl_xor_sync(0xffffffffu, pi, 1);
+                        gi = isg ? pi : o;
+                        pi = isg ? o : pi;
+                    }
+                    const double cf = tau * fma(-alpha, pi, gi);
+                    const double rv = fma(-v0, cf, pi);
+                    if (in && !isg) cfs[i * k + kk] = cf;
+                    if (in && (isg || !pairs) && c == 0) a.R[(size_t)(j0 + i) * k + kk] = rv;
+                    if (pairs) {
+                        const double mul = isg ? rv : cf;
+#pragma unroll
+                        for (int ip = i + 1; ip < QB; ++ip)
+                            p[ip] = fma(-(isg ? pan_rr[i][ip] : pan_pc[i][ip]), mul, p[ip]);
+                    } else {
+#pragma unroll
+                        for (int ip = i + 1; ip < QB; ++ip) {
+                            p[ip] = fma(-pan_pc[i][ip], cf, p[ip]);
+                            g[ip] = fma(-pan_rr[i][ip], rv, g[ip]);
+                        }
                     }
                 }
-                if (c == 0) a.R[(size_t)j * k + kk] = rv;
-            }
-            __syncthreads();
-            const int rest = nn0 - 1 - i;
-            for (int t = tid; t < rest * (k - j - 1); t += blockDim.x) {
-                const int ip = i + 1 + t / (k - j - 1), kk = j + 1 + t % (k - j - 1);
-                Ps[ip * k + kk] = fma(-Ps[ip * k + j], cfs[i * k + kk], Ps[ip * k + kk]);
-                if (kk >= j0 + ip) Gs[ip * k + kk] = fma(-Rj[j0 + ip], Rj[kk], Gs[ip * k + kk]);
             }
         }
+        __syncthreads();
+        const int nb = pan_stop;
         const int j1 = j0 + nb;
-        // reflector entries of the panel's own rows (below the diagonal) come from
-        // the updated panel rows; rows >= j1 get the in-panel updates, one thread
-        // per row, in registers
-        for (int t = tid; t < nb * nb; t += blockDim.x) {
+        // reflector entries of the panel's own rows (below the diagonal) come from the panel
+        // block; the rows below it had the in-panel updates above, or get them here where they
+        // were too many for that (one thread per row, in registers)
+        for (int t = tid; t < nn0 * nb; t += blockDim.x) {
             const int ip = t / nb, i = t % nb;
             const int rg = j0 + ip;
-            if (i < ip && rg >= r0 && rg < r1) Ys[(rg - r0) * ld + j0 + i] = Ps[ip * k + j0 + i];
+            if (i < ip && rg >= r0 && rg < r1) Ys[(size_t)(rg - r0) * ld + j0 + i] = pan_pc[i][ip];
         }
-        {
-            const int rs = max(r0, j1) - r0;
+        if (!pipe_rows)
             for (int r = rs + tid; r < nr; r += blockDim.x) {
                 double v[QB];
 #pragma unroll
-                for (int i = 0; i < QB; ++i) v[i] = (i < nb) ? Ys[r * ld + j0 + i] : 0.0;
+                for (int i = 0; i < QB; ++i) v[i] = (i < nb) ? Ys[(size_t)r * ld + j0 + i] : 0.0;
 #pragma unroll
                 for (int i = 0; i < QB; ++i)
 #pragma unroll
@@ -469,9 +727,8 @@ __global__ void __launch_bounds__(QR_THREADS, 1) qr_kernel(QrArgs a)
                         if (ip < nb) v[ip] = fma(-v[i], cfs[i * k + j0 + ip], v[ip]);
 #pragma unroll
                 for (int i = 1; i < QB; ++i)
-                    if (i < nb) Ys[r * ld + j0 + i] = v[i];
+                    if (i < nb) Ys[(size_t)r * ld + j0 + i] = v[i];
             }
-        }
         __syncthreads();
         const int nn1 = min(QB, k - j1);
         if (j1 < k) gram_pass(j0, nb, j1, nn1, acc_buf(blk + 1), pub_buf(blk + 1));
@@ -503,9 +760,12 @@ __global__ void __launch_bounds__(QR_THREADS, 1) qr_kernel(QrArgs a)
     __syncthreads();
     // S = V^T V (upper triangle): this CTA's rows, two chains per entry, summed over
     // the CTAs with FP64 atomics
-    for (int e = tid; e < k * k; e += blockDim.x) {
-        const int i = e / k, j = e % k;
-        if (j < i) continue;
+    // (rows i and k-1-i of the triangle together have k+1 entries: no lane idles)
+    for (int e = tid; e < (k + 1) / 2 * (k + 1); e += blockDim.x) {
+        const int a0 = e / (k + 1), f = e % (k + 1);
+        const bool first = f < k - a0;
+        const int i = first ? a0 : k - 1 - a0, j = first ? a0 + f : f - 1;
+        if (!first && i == a0) continue;   // the middle row of an odd k is listed once
         const int rs = max(0, j - r0);
         if (rs >= nr) continue;
         double s0 = 0.0, s1 = 0.0;
@@ -515,7 +775,7 @@ __global__ void __launch_bounds__(QR_THREADS, 1) qr_kernel(QrArgs a)
             s1 = fma(Ys[(rl + 1) * ld + i], Ys[(rl + 1) * ld + j], s1);
         }
         if (rl < nr) s0 = fma(Ys[rl * ld + i], Ys[rl * ld + j], s0);
-        if (det) a.spart[(size_t)c * k * k + e] = s0 + s1;
+        if (det) a.spart[(size_t)c * k * k + (size_t)i * k + j] = s0 + s1;
         else atomicAdd(&a.S[(size_t)i * k + j], s0 + s1);
     }
     if (det) {
@@ -541,41 +801,26 @@ __global__ void __launch_bounds__(QR_THREADS, 1) qr_kernel(QrArgs a)
         __syncthreads();
     }
     if (!grid_barrier(a.bar, a.G, ++ep, a.err, a.bar_extra, a.spin_limit)) return;
-    // Q rows of this CTA: (E - V W) with column c negated where alpha_c < 0; a thread
-    // owns one column and up to QR_QROWS rows at a time (W read once per row chunk)
+    // Q rows of this CTA: (E - V W) with column c negated where alpha_c < 0; a thread owns one
+    // column and the same number of rows, known at compile time, in every pass: a predicated-off
+    // FP64 instruction takes the pipe as long as one that runs
     {
         const int grp = blockDim.x / k;
-        const int col = tid % k, g = tid / k;
-        if (g < grp) {
-            const double sgn = alps[col] < 0.0 ? -1.0 : 1.0;
-            for (int rb = g * QR_QROWS; rb < nr; rb += grp * QR_QROWS) {
-                double acc[QR_QROWS];
-#pragma unroll
-                for (int q = 0; q < QR_QROWS; ++q) acc[q] = 0.0;
-                for (int j = 0; j < k; ++j) {
-                    const double w = __ldcg(a.W + (size_t)j * k + col);
-#pragma unroll
-                    for (int q = 0; q < QR_QROWS; ++q)
-                        if (rb + q < nr) acc[q] = fma(Ys[(rb + q) * ld + j], w, acc[q]);
-                }
-#pragma unroll
-                for (int q = 0; q < QR_QROWS; ++q) {
-                    const int rl = rb + q;
-                    if (rl < nr) {
-                        const int rg = r0 + rl;
-                        a.Q[(size_t)rg * k + col] = sgn * ((rg == col ? 1.0 : 0.0) - acc[q]);
-                    }
-                }
-            }
-        }
+        const int share = (nr + grp - 1) / grp;
+        if (share <= 1) q_rows<1>(a, alps, Ys, ld, r0, nr);
+        else if (share <= 2) q_rows<2>(a, alps, Ys, ld, r0, nr);
+        else if (share <= 3) q_rows<3>(a, alps, Ys, ld, r0, nr);
+        else if (share <= 4) q_rows<4>(a, alps, Ys, ld, r0, nr);
+        else if (share <= 6) q_rows<6>(a, alps, Ys, ld, r0, nr);
+        else q_rows<8>(a, alps, Ys, ld, r0, nr);
     }
 }
 
 size_t qr_smem_bytes(int rows_per, int k, bool slab)
 {
-    const size_t panel = 3 * (size_t)QB * k + k;
+    const size_t panel = 3 * (size_t)QB * k;
     const size_t solve = qr_wy_smem_bytes(k) / sizeof(double);
-    return sizeof(double) * ((slab ? 0 : (size_t)rows_per * (k | 1)) + 3 * (size_t)k + QB +
+    return sizeof(double) * ((slab ? 0 : (size_t)rows_per * (k | 1)) + 3 * (size_t)k +
                              (panel > solve ? panel : solve));
 }
 
