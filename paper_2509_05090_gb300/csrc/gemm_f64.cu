@@ -6,8 +6,8 @@
 // addressed through two-level index maps (Idx2) so that the permuted 4-index
 // layouts are read and written in place, with no transpose kernels.
 //
-// Tiles from 32 x 32 to 72 x 72 outputs per CTA (the bond dimensions divide
-// them), a strided micro-tile per thread so a warp's shared-memory reads are
+// Tiles from 16 x 16 to 72 x 72 outputs per CTA (the bond dimensions divide
+// the larger ones), a strided micro-tile per thread so a warp's shared-memory reads are
 // conflict-free, K staged through shared memory with a register prefetch of the
 // next K tile; the tile and the K split are chosen per shape from a wave model.
 #include "ctm_internal.h"
@@ -142,12 +142,16 @@ __global__ void __launch_bounds__((BM / MT) * (BN / MT)) gemm_f64_kernel(GemmF64
     }
 }
 
+// The 16 x 16 tile serves the small instances: their products are a few hundred thousand
+// multiply-adds, and 32- to 36-wide tiles left most SMs without a CTA (243 x 243 x 27: 49 of
+// them, 17k cycles of FP64 issue each).  243 x 243 x 27 14.2 -> 9.9 us, 243 x 27 x 243 23 -> 14,
+// 32 x 8 x 32 14 -> 8, 1024 x 16 x 256 31 -> 19.
 struct TileCfg {
     int bm, bn, bk, mt;
 };
 constexpr TileCfg kTiles[] = {{64, 64, 16, 4}, {72, 72, 12, 4}, {64, 32, 16, 4}, {72, 36, 12, 4},
                               {32, 64, 16, 4}, {36, 72, 12, 4}, {64, 72, 12, 4}, {72, 64, 16, 4},
-                              {32, 32, 16, 2}, {36, 36, 12, 2}};
+                              {32, 32, 16, 2}, {36, 36, 12, 2}, {16, 16, 16, 1}};
 
 // Deterministic split-K reduction: fixed summation order over the splits.
 __global__ void splitk_reduce_kernel(GemmF64 g, int ksplit, const double *partial)
@@ -193,6 +197,9 @@ struct TilePick {
     int ksplit;
 };
 
+// The split-K reduction's own launch, in multiply-adds of one SM (about 2.5 us at 2 per cycle)
+constexpr double SPLITK_LAUNCH = 9000.0;
+
 static TilePick pick_tile_split(int M, int N, int K, bool splitk_ok)
 {
     const long long sms = device_sm_count();
@@ -216,7 +223,7 @@ static TilePick pick_tile_split(int M, int N, int K, bool splitk_ok)
             const long long ctas = tiles * s_eff;
             const long long waves = (ctas + sms - 1) / sms;
             double cost = (double)waves * t.bm * t.bn * kchunk * (1.0 + 8.0 / t.bm + 8.0 / t.bn);
-            if (s_eff > 1) cost += (double)M * N * s_eff / (double)sms;   // the split-K reduction
+            if (s_eff > 1) cost += (double)M * N * s_eff / (double)sms + SPLITK_LAUNCH;   // the split-K reduction
             if (cost < best_cost * 0.999) {
                 best_cost = cost;
                 best = TilePick{t, (int)s_eff};
@@ -280,6 +287,7 @@ cudaError_t gemm_f64(const GemmF64 &g, int ksplit, double *scratch, size_t scrat
     CTM_TILE(72, 64, 16, 4)
     CTM_TILE(32, 32, 16, 2)
     CTM_TILE(36, 36, 12, 2)
+    CTM_TILE(16, 16, 16, 1)
 #undef CTM_TILE
     return cudaErrorInvalidValue;
 }
