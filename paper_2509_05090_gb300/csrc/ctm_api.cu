@@ -70,7 +70,8 @@ struct Shape {
     int M, N, K;
 };
 
-// (M, N, K) of the eleven contractions of one step, in launch order.
+// (M, N, K) of the contractions of one step, in launch order: through X' and H1' (also the
+// energy's and the transfer matrix's), and through TA.
 std::vector<Shape> step_shapes(const ctm_ctx *c)
 {
     const int chi = c->chi, D2 = c->D2, n = (int)c->n;
@@ -325,8 +326,15 @@ cudaError_t run_gemm(ctm_ctx *c, const GemmF64 &g, int hint, int lane)
             o.a_fill = use ? 0 : 1;
             if (!use) fill_slot = slot;
         }
+        if (hint == GEMM_A_FILL_TA || hint == GEMM_A_USE_TA) {
+            o.a_pk = c->sw_e.Apk;
+            o.a_e = c->sw_e.eA;
+            o.a_cap = c->sw_e.a_pack_cap;
+            o.a_fill = hint == GEMM_A_USE_TA && c->ta_packed ? 0 : 1;
+        }
         cudaError_t e = gemm_split(g, T, lw, lst, ev, &o);
         if (fill_slot >= 0) c->ack_valid[fill_slot] = (e == cudaSuccess);
+        if (hint == GEMM_A_FILL_TA || hint == GEMM_A_USE_TA) c->ta_packed = (e == cudaSuccess);
         return e;
     }
     if (ev) {
@@ -344,6 +352,47 @@ cudaError_t run_gemm(ctm_ctx *c, const GemmF64 &g, int hint, int lane)
         cudaError_t _e = (expr);                          \
         if (_e != cudaSuccess) return CTM_ECUDA;          \
     } while (0)
+
+static bool uses_ta(const ctm_ctx *c) { return c->cfg.precision == CTM_FP64; }
+
+// M[(a,y)][(b,x)] = sum_z Y1[(a,b), z] a[z, x, y]; the GEMM column index runs over (y, x)
+// with x fastest, so an output tile covers whole contiguous (b, x) runs of M
+static cudaError_t corner_from_y1(ctm_ctx *c)
+{
+    const int chi = c->chi, D2 = c->D2;
+    const long long n = c->n;
+    GemmF64 g{chi * chi, D2 * D2, D2, c->Y1, idx_lin(D2), idx_lin(1), c->a, idx_lin((long long)D2 * D2),
+              idx_split(D2, 1, D2), c->M, idx_split(chi, (long long)D2 * n, D2), idx_split(D2, n, 1), 1.0, 0.0};
+    return run_gemm(c, g, GEMM_B_IS_A_ZX);
+}
+
+// FP64: the radial dimer's outer site contracted with the row edge first,
+// TA[(a,z)][(g,l)] = sum_u T[a,u,g] a[u,l,z]; CT[b][(g,l)] = sum_h C[g,h] T[b,l,h];
+// Y1[(a,b)][z] = sum_{g,l} TA CT; M as below.  TA depends neither on C nor on Q, and the edge
+// update's H2 = T Q a is TA Q: one n x n intermediate and its pack serve both, where X' = T C T
+// and H1' = T Q are one each (two n x n outputs, two packs and 2 chi^2 D2^3 multiply-adds a step
+// more): 1.44 -> 1.36 ms per step at D = 6, chi = 72.  The split modes keep the order below: their
+// results carry the truncation of its operands.
+static int enqueue_enlarged_corner_ta(ctm_ctx *c)
+{
+    const int chi = c->chi, D2 = c->D2;
+    const long long n = c->n;
+    GemmF64 g;
+    // rows (a, g), columns (z, l) with l fastest: the pack of a is the one M = Y1 a uses
+    g = GemmF64{chi * chi, D2 * D2, D2, c->T, idx_split(chi, (long long)D2 * chi, 1), idx_lin(chi), c->a,
+                idx_lin((long long)D2 * D2), idx_split(D2, 1, D2), c->X, idx_split(chi, (long long)D2 * n, D2),
+                idx_split(D2, n, 1), 1.0, 0.0};
+    c->ta_packed = 0;
+    CK(run_gemm(c, g, GEMM_B_IS_A_ZX));
+    g = GemmF64{(int)n, chi, chi, c->T, idx_lin(chi), idx_lin(1), c->C, idx_lin(1), idx_lin(chi),
+                c->W, idx_split(D2, n, 1), idx_lin(D2), 1.0, 0.0};
+    CK(run_gemm(c, g));
+    g = GemmF64{(int)n, chi, (int)n, c->X, idx_lin(n), idx_lin(1), c->W, idx_lin(1), idx_lin(n),
+                c->Y1, idx_split(D2, (long long)chi * D2, 1), idx_lin(D2), 1.0, 0.0};
+    CK(run_gemm(c, g, GEMM_A_FILL_TA));
+    CK(corner_from_y1(c));
+    return CTM_OK;
+}
 
 // ---------------------------------------------------------------- enlarged corner
 // Fig. 3(c): X'[a][b][u][l] = sum_{g,h} T[a,u,g] C[g,h] T[b,l,h];
@@ -366,11 +415,7 @@ int enqueue_enlarged_corner(ctm_ctx *c)
     g = GemmF64{chi * chi, D2, D2 * D2, c->X, idx_lin((long long)D2 * D2), idx_lin(1), c->a, idx_lin(D2),
                 idx_lin(1), c->Y1, idx_lin(D2), idx_lin(1), 1.0, 0.0};
     CK(run_gemm(c, g, GEMM_B_IS_A_LZ));
-    // M[(a,y)][(b,x)] = Y1[(a,b), z] a[z, x, y]; the GEMM column index runs over (y, x)
-    // with x fastest, so an output tile covers whole contiguous (b, x) runs of M
-    g = GemmF64{chi * chi, D2 * D2, D2, c->Y1, idx_lin(D2), idx_lin(1), c->a, idx_lin((long long)D2 * D2),
-                idx_split(D2, 1, D2), c->M, idx_split(chi, (long long)D2 * n, D2), idx_split(D2, n, 1), 1.0, 0.0};
-    CK(run_gemm(c, g, GEMM_B_IS_A_ZX));
+    CK(corner_from_y1(c));
     return CTM_OK;
 }
 
@@ -426,7 +471,8 @@ int enqueue_corner_from_r(ctm_ctx *c, double *Cout)
     return CTM_OK;
 }
 
-// Fig. 3(b): T'[i,x,j] = sum Q[(a,y),i] T[a,u,g] a[u,w,z] a[z,x,y] Q[(g,w),j], normalised.
+// Fig. 3(b): T'[i,x,j] = sum Q[(a,y),i] T[a,u,g] a[u,w,z] a[z,x,y] Q[(g,w),j], normalised
+// (FP64: from the step's TA = T a).
 // lane 2: with the edge lane's work buffers, concurrent with a corner
 // update on lane2; the last contraction waits for it (it uses the corner's pack of Q^T).
 int enqueue_edge(ctm_ctx *c, const double *Qp, double *Tout, int lane = 0)
@@ -435,14 +481,22 @@ int enqueue_edge(ctm_ctx *c, const double *Qp, double *Tout, int lane = 0)
     const long long n = c->n;
     cudaStream_t st = c->stream;
     GemmF64 g;
-    // H1'[a][j][u][w] = sum_g T[(a,u),g] Q[(g,w),j]; column index (j, w), w fastest
-    g = GemmF64{(int)n, (int)n, chi, c->T, idx_lin(chi), idx_lin(1), Qp, idx_lin(n), idx_split(D2, 1, chi),
-                c->X, idx_split(D2, (long long)chi * D2 * D2, D2), idx_split(D2, (long long)D2 * D2, 1), 1.0, 0.0};
-    CK(run_gemm(c, g, GEMM_A_USE_T, lane));
-    // H2[(a,j)][z] = H1'[(a,j),(u,w)] a[(u,w),z]
-    g = GemmF64{chi * chi, D2, D2 * D2, c->X, idx_lin((long long)D2 * D2), idx_lin(1), c->a, idx_lin(D2),
-                idx_lin(1), c->Y1, idx_lin(D2), idx_lin(1), 1.0, 0.0};
-    CK(run_gemm(c, g, GEMM_B_IS_A_LZ, lane));
+    if (uses_ta(c)) {
+        // H2[(a,j)][z] = sum_{g,w} TA[(a,z)][(g,w)] Q[(g,w),j]
+        g = GemmF64{(int)n, chi, (int)n, c->X, idx_lin(n), idx_lin(1), Qp, idx_lin(chi), idx_lin(1),
+                    c->Y1, idx_split(D2, (long long)chi * D2, 1), idx_lin(D2), 1.0, 0.0};
+        CK(run_gemm(c, g, GEMM_A_USE_TA, lane));
+        c->ta_packed = 0;   // (the next contraction packs H2 over it)
+    } else {
+        // H1'[a][j][u][w] = sum_g T[(a,u),g] Q[(g,w),j]; column index (j, w), w fastest
+        g = GemmF64{(int)n, (int)n, chi, c->T, idx_lin(chi), idx_lin(1), Qp, idx_lin(n), idx_split(D2, 1, chi),
+                    c->X, idx_split(D2, (long long)chi * D2 * D2, D2), idx_split(D2, (long long)D2 * D2, 1), 1.0, 0.0};
+        CK(run_gemm(c, g, GEMM_A_USE_T, lane));
+        // H2[(a,j)][z] = H1'[(a,j),(u,w)] a[(u,w),z]
+        g = GemmF64{chi * chi, D2, D2 * D2, c->X, idx_lin((long long)D2 * D2), idx_lin(1), c->a, idx_lin(D2),
+                    idx_lin(1), c->Y1, idx_lin(D2), idx_lin(1), 1.0, 0.0};
+        CK(run_gemm(c, g, GEMM_B_IS_A_LZ, lane));
+    }
     // H3'[a][y][x][j] = H2[(a,j),z] a[z, x, y]; column index (y, x), x fastest
     g = GemmF64{chi * chi, D2 * D2, D2, c->Y1, idx_lin(D2), idx_lin(1), c->a, idx_lin((long long)D2 * D2),
                 idx_split(D2, 1, D2), c->H, idx_split(chi, (long long)D2 * D2 * chi, 1),
@@ -485,10 +539,11 @@ int enqueue_step(ctm_ctx *c)
     // update runs on lane2 beside the edge update.  This path also writes the new
     // environment in place: C, T and Q are not read after the QR except by their
     // own updates (the warm start and the enlarged corner come before it; the edge
-    // update reads T in its first contraction, before its last one writes T'), so
+    // update reads T in its first contraction, before its last one writes T', or only
+    // the corner's TA), so
     // no hand-over copies are needed.
     const bool lanes = c->steps_done > 0 && c->cfg.corner_mode == 0;
-    if ((rc = enqueue_enlarged_corner(c)) != CTM_OK) return rc;
+    if ((rc = uses_ta(c) ? enqueue_enlarged_corner_ta(c) : enqueue_enlarged_corner(c)) != CTM_OK) return rc;
     if ((rc = enqueue_projector(c, lanes ? c->Q : c->Qn)) != CTM_OK) return rc;
     if (lanes) {
         CK(cudaEventRecord(c->ev_q, st));
@@ -552,7 +607,7 @@ int enqueue_step_profiled(ctm_ctx *c, cudaEvent_t *ev)
     cudaStream_t st = c->stream;
     const long long chi = c->chi, D2 = c->D2, n = c->n;
     CK(cudaEventRecord(ev[0], st));
-    if ((rc = enqueue_enlarged_corner(c)) != CTM_OK) return rc;
+    if ((rc = uses_ta(c) ? enqueue_enlarged_corner_ta(c) : enqueue_enlarged_corner(c)) != CTM_OK) return rc;
     CK(cudaEventRecord(ev[1], st));
     c->ack_valid[1] = 0;   // the QR below writes a new Q
     CK(launch_warm_start((int)n, (int)chi, c->Q, c->C, c->Qs, st));

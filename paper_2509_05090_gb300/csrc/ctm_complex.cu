@@ -61,6 +61,10 @@ struct ctm_complex_ctx {
     double *norm_part;
     double *rho_part, *rho_raw, *hrot, *eout;
     SplitWork sw;
+    // the packed TA = T a of the step (used by Y1 and H2)
+    unsigned char *ta_pk;
+    int *ta_e;
+    size_t ta_cap;
     int steps_done;
     // steps after the first (eager, autotuning) one replay a captured one-step graph
     cudaStream_t own;
@@ -917,6 +921,10 @@ struct ZGemm {
     Idx2 Cm, Cn;
 };
 
+// A operands of the split engine that an earlier product packed: the previous product's
+// (still in the work buffers), or TA's, kept in a buffer of its own for a second use
+enum { ZA_PACK = 0, ZA_REUSE = 1, ZA_FILL_TA = 2, ZA_USE_TA = 3 };
+
 int real_gemm(ctm_complex_ctx *c, const GemmF64 &g, int reuse_a)
 {
     if (c->tf32_T > 0) return gemm_tf32(g, c->tf32_T, c->sw, c->stream, nullptr) == cudaSuccess ? CTM_OK : CTM_ECUDA;
@@ -926,7 +934,13 @@ int real_gemm(ctm_complex_ctx *c, const GemmF64 &g, int reuse_a)
                       : 0;
     if (T > 0) {
         SplitOpts o{};
-        o.reuse_a = reuse_a;
+        o.reuse_a = reuse_a == ZA_REUSE;
+        if (reuse_a >= ZA_FILL_TA) {
+            o.a_pk = c->ta_pk;
+            o.a_e = c->ta_e;
+            o.a_cap = c->ta_cap;
+            o.a_fill = reuse_a == ZA_FILL_TA;
+        }
         return gemm_split(g, T, c->sw, c->stream, nullptr, &o) == cudaSuccess ? CTM_OK : CTM_ECUDA;
     }
     return gemm_f64(g, gemm_f64_pick_split(g.M, g.N, g.K), c->splitk, c->splitk_elems, c->stream) == cudaSuccess
@@ -940,9 +954,8 @@ static Idx2 zkmap(int K, long long P, long long s2)
     return Idx2{K, P, s2};
 }
 
-// reuse_a: the left operand is that of the previous zgemm call, unchanged since (its
-// packed slices are still in the split engine's work buffers)
-int zgemm(ctm_complex_ctx *c, const ZGemm &z, int reuse_a = 0)
+// reuse_a: ZA_REUSE if the left operand is that of the previous zgemm call, unchanged since
+int zgemm(ctm_complex_ctx *c, const ZGemm &z, int reuse_a = ZA_PACK)
 {
     if (z.Ak.s1 != 0 || z.Bk.s1 != 0) return CTM_EINVAL;
     if (z.conjA && !z.a5) return CTM_EINVAL;
@@ -958,7 +971,7 @@ int zgemm(ctm_complex_ctx *c, const ZGemm &z, int reuse_a = 0)
     GemmF64 gi{z.M, z.N, 2 * z.K, Ap, z.Am, Ak2, Bi, Bk2, z.Bn, z.C + (z.c5 ? 3 : 1) * z.PC, z.Cm, z.Cn, 1.0, 0.0};
     int rc = real_gemm(c, gr, reuse_a);
     if (rc != CTM_OK) return rc;
-    return real_gemm(c, gi, 1);
+    return real_gemm(c, gi, reuse_a >= ZA_FILL_TA ? ZA_USE_TA : ZA_REUSE);
 }
 
 int znormalize(ctm_complex_ctx *c, long long count, double *x, ZLay L)
@@ -1115,6 +1128,9 @@ size_t zlayout(ctm_complex_ctx *c, char *base)
         c->sw.partial_cap = pp;
         c->sw.err = c->err;
         c->sw.autotune = 1;
+        c->ta_pk = (unsigned char *)take(ap);
+        c->ta_cap = ap;
+        c->ta_e = (int *)take(sizeof(int) * (size_t)ecap);
     }
     return off;
 }
@@ -1153,6 +1169,41 @@ int zread_status(ctm_complex_ctx *c)
 // Cr and H two planes stacked (k slowest for the next contraction).
 ZLay lay_T(const ctm_complex_ctx *c) { return zlay_rows(c->chi, 5); }
 
+bool zuses_ta(const ctm_complex_ctx *c) { return c->cfg.precision == CTM_FP64; }
+
+// M[(a,y)][(b,x)] = sum_z Y1[(a,b), z] aA[z,x,y]
+int zcorner_from_y1(ctm_complex_ctx *c)
+{
+    const int chi = c->chi, D2 = c->D2;
+    const long long n = c->n, DD = (long long)D2 * D2;
+    const ZGemm z{chi * chi, D2 * D2, D2, c->Y1, D2, 0, idx_lin(2LL * D2), idx_lin(1), 0, c->aA, c->Pa, idx_lin(DD),
+                  idx_split(D2, 1, D2), 0, c->M, n, 0, idx_split(chi, 2LL * D2 * n, D2), idx_split(D2, 2 * n, 1)};
+    return zgemm(c, z);
+}
+
+// FP64: the step's enlarged corner with the outer site contracted with the row edge first (as on
+// the real path, ctm_api.cu): TA[(a,z)][(g,l)] = sum_u T[a,u,g] a[u,l,z]; CT[b][(g,l)] = sum_h C[g,h]
+// conj(T[b,l,h]) (five planes per row b, in Qs, which the warm start rewrites later);
+// Y1[(a,b)][z] = sum_{g,l} TA CT.  TA and its pack serve the edge update's H2 = TA Q too.
+int zenlarged_corner_ta(ctm_complex_ctx *c)
+{
+    const int chi = c->chi, D2 = c->D2;
+    const long long n = c->n, DD = (long long)D2 * D2;
+    int rc;
+    ZGemm z{chi * chi, D2 * D2, D2, c->T, chi, 1, idx_split(chi, 5LL * D2 * chi, 1), idx_lin(5LL * chi), 0, c->a, c->Pa,
+            idx_lin(DD), idx_split(D2, 1, D2), 0, c->X, n, 0, idx_split(chi, 2LL * D2 * n, D2),
+            idx_split(D2, 2 * n, 1)};
+    if ((rc = zgemm(c, z)) != CTM_OK) return rc;
+    z = ZGemm{(int)n, chi, chi, c->T, chi, 1, idx_lin(5LL * chi), idx_lin(1), 1, c->C, c->PC, idx_lin(1), idx_lin(chi),
+              0, c->Qs, n, 1, idx_split(D2, 5 * n, 1), idx_lin(D2)};
+    if ((rc = zgemm(c, z)) != CTM_OK) return rc;
+    ZLAUNCH(zc_complete_kernel, zgrid(n * chi), 256, n * chi, c->Qs, zlay_rows(n, 5));
+    z = ZGemm{(int)n, chi, (int)n, c->X, n, 0, idx_lin(2 * n), idx_lin(1), 0, c->Qs, n, idx_lin(1), idx_lin(5 * n), 0,
+              c->Y1, D2, 0, idx_split(D2, 2LL * chi * D2, 1), idx_lin(2LL * D2)};
+    if ((rc = zgemm(c, z, ZA_FILL_TA)) != CTM_OK) return rc;
+    return zcorner_from_y1(c);
+}
+
 // Fig. 3c: W = T C; X'[a][b][u][l] = sum_h W[(a,u),h] conj(T[(b,l),h]);
 // Y1[(a,b)][z] = sum_{u,l} X' a[u,l,z]; M[(a,y)][(b,x)] = sum_z Y1 aA[z,x,y], with aA the double
 // layer of the apex site (z leg first; equal to a for a C3-symmetric tensor)
@@ -1170,9 +1221,7 @@ int zenlarged_corner(ctm_complex_ctx *c)
     z = ZGemm{chi * chi, D2, D2 * D2, c->X, DD, 0, idx_lin(2 * DD), idx_lin(1), 0, c->a, c->Pa, idx_lin(D2),
               idx_lin(1), 0, c->Y1, D2, 0, idx_lin(2LL * D2), idx_lin(1)};
     if ((rc = zgemm(c, z)) != CTM_OK) return rc;
-    z = ZGemm{chi * chi, D2 * D2, D2, c->Y1, D2, 0, idx_lin(2LL * D2), idx_lin(1), 0, c->aA, c->Pa, idx_lin(DD),
-              idx_split(D2, 1, D2), 0, c->M, n, 0, idx_split(chi, 2LL * D2 * n, D2), idx_split(D2, 2 * n, 1)};
-    return zgemm(c, z);
+    return zcorner_from_y1(c);
 }
 
 // Fig. 3d: Y = M Q diag(sgn Re C_jj); Y = Q R through the real QR of the embedding
@@ -1201,7 +1250,7 @@ int zcorner(ctm_complex_ctx *c, double *Cout)
     // the previous contraction was Y = M Qs (only the QR in between): M is packed already
     ZGemm z{(int)n, chi, (int)n, c->M, n, 0, idx_lin(2 * n), idx_lin(1), 0, c->Qn, c->PQ, idx_lin(chi), idx_lin(1), 0,
             c->MQ, c->PY, 0, idx_lin(chi), idx_lin(1)};
-    if ((rc = zgemm(c, z, 1)) != CTM_OK) return rc;
+    if ((rc = zgemm(c, z, ZA_REUSE)) != CTM_OK) return rc;
     z = ZGemm{chi, chi, (int)n, c->MQ, c->PY, 0, idx_lin(1), idx_lin(chi), 0, c->Qn, c->PQ, idx_lin(chi), idx_lin(1), 1,
               c->Cr, c->PC, 0, idx_lin(1), idx_lin(chi)};
     if ((rc = zgemm(c, z)) != CTM_OK) return rc;
@@ -1225,8 +1274,15 @@ int zedge(ctm_complex_ctx *c)
     const int chi = c->chi, D2 = c->D2;
     const long long n = c->n, DD = (long long)D2 * D2;
     int rc;
+    ZGemm z;
+    if (zuses_ta(c)) {
+        // H2[(a,j)][z] = sum_{g,w} TA[(a,z)][(g,w)] Q[(g,w),j]
+        z = ZGemm{(int)n, chi, (int)n, c->X, n, 0, idx_lin(2 * n), idx_lin(1), 0, c->Qn, c->PQ, idx_lin(chi), idx_lin(1), 0,
+                  c->Y1, D2, 0, idx_split(D2, 2LL * chi * D2, 1), idx_lin(2LL * D2)};
+        if ((rc = zgemm(c, z, ZA_USE_TA)) != CTM_OK) return rc;
+    } else {
     // H1'[a][j][u][w] = sum_g T[(a,u),g] Q[(g,w),j]   (into X, laid out as X')
-    ZGemm z{(int)n, (int)n, chi, c->T, chi, 1, idx_lin(5LL * chi), idx_lin(1), 0, c->Qn, c->PQ, idx_lin(n),
+    z = ZGemm{(int)n, (int)n, chi, c->T, chi, 1, idx_lin(5LL * chi), idx_lin(1), 0, c->Qn, c->PQ, idx_lin(n),
             idx_split(D2, 1, chi), 0, c->X, DD, 0, idx_split(D2, (long long)chi * 2 * DD, D2),
             idx_split(D2, 2 * DD, 1)};
     if ((rc = zgemm(c, z)) != CTM_OK) return rc;
@@ -1234,6 +1290,7 @@ int zedge(ctm_complex_ctx *c)
     z = ZGemm{chi * chi, D2, D2 * D2, c->X, DD, 0, idx_lin(2 * DD), idx_lin(1), 0, c->a, c->Pa, idx_lin(D2),
               idx_lin(1), 0, c->Y1, D2, 0, idx_lin(2LL * D2), idx_lin(1)};
     if ((rc = zgemm(c, z)) != CTM_OK) return rc;
+    }
     // H3'[a][y][x][j] = H2[(a,j),z] a[z,x,y]
     z = ZGemm{chi * chi, D2 * D2, D2, c->Y1, D2, 0, idx_lin(2LL * D2), idx_lin(1), 0, c->aA, c->Pa, idx_lin(DD),
               idx_split(D2, 1, D2), 0, c->H, c->PM, 0, idx_split(chi, DD * chi, 1),
@@ -1309,7 +1366,7 @@ int zstep(ctm_complex_ctx *c, int join_now)
         if ((rc = zspectrum(c, c->C, c->side, c->delta_head)) != CTM_OK) return rc;
         c->side_pending = 1;
     }
-    if ((rc = zenlarged_corner(c)) != CTM_OK) return rc;
+    if ((rc = zuses_ta(c) ? zenlarged_corner_ta(c) : zenlarged_corner(c)) != CTM_OK) return rc;
     if ((rc = zprojector(c)) != CTM_OK) return rc;
     if (c->side_pending) {
         ZK(cudaStreamWaitEvent(c->stream, c->ev_join, 0));

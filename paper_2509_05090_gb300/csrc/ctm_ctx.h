@@ -54,6 +54,7 @@ struct ctm_ctx {
     int *ace[2];
     size_t ack_cap[2];
     int ack_valid[2];
+    int ta_packed;            // FP64: the packed TA = T a of the step is in the edge lane's A buffer
     double *qr_sbuf, *qr_rowbuf, *qr_wy;
     double *qr_gpart, *qr_spart;   // deterministic mode: per-CTA partial sums (else null)
     double *qr_slab;               // the QR's row blocks where they do not fit shared memory (else null)
@@ -136,7 +137,9 @@ enum {
     GEMM_A_FILL_T = 4,
     GEMM_A_USE_T = 5,
     GEMM_A_FILL_Q = 6,
-    GEMM_A_USE_Q = 7
+    GEMM_A_USE_Q = 7,
+    GEMM_A_FILL_TA = 8,
+    GEMM_A_USE_TA = 9
 };
 // lane 0: the step's stream and work buffers; 1: the corner lane; 2: the edge lane
 cudaError_t run_gemm(ctm_ctx *c, const GemmF64 &g, int hint = GEMM_PLAIN, int lane = 0);

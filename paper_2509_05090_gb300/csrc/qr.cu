@@ -62,7 +62,7 @@ namespace {
 constexpr int QR_THREADS = 512;
 constexpr int QR_DET_GMAX = 320;   // deterministic mode: partial-sum slots (CTAs) provided for
 constexpr int QB = 8;                     // panel width (columns per grid barrier)
-constexpr double QR_DOWNDATE_MIN = 1.0 / 16.0;   // smallest kept ratio of downdated / fresh norm^2
+constexpr int QR_DOWNDATE_LOG2 = 4;               // smallest kept ratio of downdated / fresh norm^2: 2^-4
 constexpr long long QR_SPIN_LIMIT = 20000000LL;   // x ~64 ns sleep: ~1.3 s
 
 // Grid barrier number `epoch` (1, 2, ...): every CTA adds 1 to a monotonic
@@ -576,7 +576,7 @@ __global__ void __launch_bounds__(QR_THREADS, 1) qr_kernel(QrArgs a)
                 const double x0 = __shfl_sync(0xffffffffu, i < 4 ? P0 : P1, src);
                 const long long nb2 = __double_as_longlong(nrm2);
                 // cancellation (or NaN): the panel ends here and the next one starts from fresh sums
-                const long long least = __double_as_longlong(__shfl_sync(0xffffffffu, fresh, i)) - (4LL << 52);
+                const long long least = __double_as_longlong(__shfl_sync(0xffffffffu, fresh, i)) - ((long long)QR_DOWNDATE_LOG2 << 52);
                 if (i > 0 && !(nb2 >= least && nb2 <= 0x7FF0000000000000LL && nb2 > 0)) {
                     stop = i;
                     break;
