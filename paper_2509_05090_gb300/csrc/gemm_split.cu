@@ -31,23 +31,35 @@
 // K 2^-53 sum |a b|.  Measured against 128-bit sums (2-norm over the output): 3e-17 to 6e-17
 // at every shape and for normal, uniform, graded and constant operands, the FP64 GEMM 1e-16
 // to 2e-15.  Rows and columns with infinities or NaNs have no grid; their outputs are the
-// plain FP64 sums.  Against the FP64 pipe's GEMM: 8192 x 8192 x 128 14.07 -> 1.11 ms,
-// 8192 x 128 x 8192 14.28 -> 0.95 ms, 2592 x 2592 x 72 848 -> 146 us, 2592 x 72 x 2592
-// 934 -> 141 us, 900 x 900 x 36 72 -> 34 us; below MNK = 8e6 (512 x 512 x 32: 27 against
-// 28 us, 243 x 243 x 27: 14 against 29) the two packs and three launches cost more than
-// the FP64 GEMM, which keeps those shapes (split_f64_pays).
+// plain FP64 sums.  Against the FP64 pipe's GEMM: 8192 x 8192 x 128 14.09 -> 0.89 ms,
+// 8192 x 128 x 8192 14.30 -> 0.96 ms, 2592 x 2592 x 72 849 -> 111 us, 2592 x 72 x 2592
+// 935 -> 141 us, 900 x 900 x 36 72 -> 29 us; below MNK = 8e6 (512 x 512 x 32: 28 against
+// 26 us, 512 x 32 x 512: 33 against 38, 243 x 243 x 27: 11 against 26) the two packs and three
+// launches cost more than the FP64 GEMM, which keeps those shapes (split_f64_pays).
 //
-// Kernel.  Tile 128 x NT (NT = 64 or 96), K staged 64 at a time; one MMA covers up to
+// Kernel.  Tile 128 x NT (NT = 32 to 96), K staged 64 at a time; one MMA covers up to
 // 256 / NT slice pairs (N = up to 256), since narrow MMAs run far below the tensor peak.  The slicing
 // pre-pass writes each operand tile in the exact shared-memory image the MMA
 // expects (K-major, 128-byte swizzle: row r of a 128-byte-wide tile at
 // (r/8)*1024 + (r%8)*128, 16-byte chunk c at (c ^ (r%8))*16), so one bulk
 // asynchronous copy (cp.async.bulk, the TMA engine) moves a whole tile.
 // Warp 0 issues the copies, warp 1 the tcgen05.mma instructions (one thread),
-// warps 2..17 drain TMEM with tcgen05.ld (four per TMEM sub-partition, a
-// quarter of the tile's columns each) and write the tile out through shared
+// the others (8 or 16) drain TMEM with tcgen05.ld (two or four per TMEM sub-partition, each
+// its share of the tile's columns) and write the tile out through shared
 // memory.  All waits are bounded; on expiry the
 // kernel raises an error flag, stops issuing work, frees its TMEM and returns.
+//
+// What bounds it: at small K (the outer-product shapes) a CTA is one chain -- set-up, first
+// copies (~1k cycles of latency), MMAs, drain, write-out -- of ~20k cycles, two of them in
+// flight per SM; stamps in each stage gave the order of attack.  The first copies leave before
+// the first CTA barrier and a single-K-tile CTA has all its slices in flight; the drain adds
+// exact FP32 integers with one magic addition where they fit 22 bits; the write-out reads each
+// row's and column's address and scale once, converts before it stores and scales by an integer
+// add, since every FP64 instruction, conversions and compares included, holds its
+// sub-partition's FP64 pipe for 64 cycles.  T = 5: 2592 x 2592 x 72 58.9 -> 49.9 us, 5184 x 1296 x 36
+// 52.7 -> 42.7, 512 x 512 x 32 15.0 -> 11.8; T = 8: 2592 x 2592 x 72 131 -> 90, 8192 x 8192 x 128
+// 1077 -> 889.  At large K the MMAs bound it (2592 x 72 x 2592, T = 8: 100 us, 98 % of the
+// CTA's time in the K loop).
 #include <cuda_bf16.h>
 
 #include <vector>
@@ -77,6 +89,14 @@ __host__ __device__ constexpr bool sp_wide(int T) { return T > 5; }
 constexpr int sp_aslots(int nt, int T)
 {
     return T == 8 ? (nt == 32 ? 2 : 6) : nt == 96 ? 6 : (nt == 64 ? 8 : 3);
+}
+// A CTA with a single K tile needs one B slot: the other one's space holds more A slices, so
+// that all T of them are in flight at once.
+constexpr int sp_aslots_one(int nt, int T)
+{
+    const int extra = T * nt * 64 * 2 / (128 * 64 * 2) + (nt == 48 && T == 5 ? 1 : 0);   // (2 KB more, see split_smem_bytes)
+    const int n = sp_aslots(nt, T) + extra;
+    return n > T ? (sp_aslots(nt, T) > T ? sp_aslots(nt, T) : T) : n;
 }
 template <int NT>
 struct SpCfg {
@@ -528,6 +548,41 @@ __device__ __forceinline__ double scaled_int_to_double(long long S, int scale)
     return __hiloint2double((hi & ~0x7FF00000) | (be << 20), lo);
 }
 
+// int64 -> double (rounded half up on the magnitude) times 2^scale, |scale| <= 900, with integer
+// instructions only and no branch.  The write-out mixes this with the conversion instruction: that
+// one holds its sub-partition's FP64 pipe for 64 cycles, these ~25 instructions the integer pipes
+// for about as long, and the two run side by side.
+__device__ __forceinline__ double scaled_int_to_double_i(long long S, int scale)
+{
+    const int sg = (int)(S >> 63);
+    const unsigned long long a = (unsigned long long)((S ^ (long long)sg) - (long long)sg);
+    const uint32_t ah = (uint32_t)(a >> 32), al = (uint32_t)a;
+    const uint32_t h = ah != 0 ? ah : al, l = ah != 0 ? al : 0u;
+    const int lz = __clz((int)h);
+    const uint32_t nh = __funnelshift_l(l, h, lz), nl = l << (lz & 31);
+    // 53 bits (the leading one included: the exponent field is one less) plus the next bit; a carry
+    // moves the exponent up
+    const uint32_t hi = ((uint32_t)((ah != 0 ? 1085 : 1053) + scale - lz) << 20) + (nh >> 11);
+    const unsigned long long r = (((unsigned long long)hi << 32) | __funnelshift_r(nl, nh, 11)) + ((nl >> 10) & 1u);
+    const unsigned long long sgn = (unsigned long long)(uint32_t)(sg & (int)0x80000000) << 32;
+    return __longlong_as_double((long long)(h == 0 ? 0ull : (r | sgn)));
+}
+
+// One row's or column's output offset and exponent scale, in the epilogue's shared memory
+struct __align__(16) SpLine {
+    long long off;
+    int sc, pad;
+};
+
+// Largest magnitude a level-t accumulator can reach over K products: t + 1 digit pairs of at
+// most 2^14 each (FP64 slices: the top digit is at most 2^6, so level 0 has 2^12 and level t
+// two pairs of 2^13 among its t + 1)
+template <int T>
+__host__ __device__ constexpr long long level_max(int t, int K)
+{
+    return (long long)K * (sp_wide(T) ? (t == 0 ? 1 << 12 : t << 14) : (t + 1) << 14);
+}
+
 struct SplitArgs {
     int M, N, K, T;
     int mTiles, nTiles, kTiles;
@@ -542,6 +597,7 @@ struct SplitArgs {
     // FP64 slices (T = 8) only: C = alpha A B + beta C, and the operands, for rows and
     // columns that hold an infinity or a NaN
     double alpha, beta;
+    int plain;                       // alpha = 1 and beta = 0 (an FP64 compare per element would cost an FMA's time)
     const double *A, *B;
     Idx2 Am, Ak, Bk, Bn;
 };
@@ -566,9 +622,31 @@ __device__ __noinline__ double plain_dot(const SplitArgs &a, int m, int n)
 __device__ __forceinline__ void store_wide(const SplitArgs &a, double d, int scale, int m, int n, long long off)
 {
     double v = scale > SP_NONFINITE / 2 ? plain_dot(a, m, n) : scale_exponent(d, scale);
-    if (a.alpha != 1.0) v *= a.alpha;
-    if (a.beta != 0.0) v = fma(a.beta, a.C[off], v);
+    if (!a.plain) {
+        v *= a.alpha;
+        if (a.beta != 0.0) v = fma(a.beta, a.C[off], v);
+    }
     a.C[off] = v;
+}
+
+// Output elements: v is the int64 sum, or (FP64 slices) the unscaled double.  Within +-900 the
+// scale cannot leave the exponent range (a sum has at most 95 bits), so it is one integer add on
+// the high word, without a branch; beyond, for rows and columns without a grid, and with alpha or
+// beta, the general functions.
+__device__ __forceinline__ bool scale_in_range(int sc) { return (unsigned)(sc + 900) <= 1800u; }
+template <bool WIDE>
+__device__ __forceinline__ double out_value(long long v, int sc, bool by_int)
+{
+    if (!WIDE && by_int) return scaled_int_to_double_i(v, sc);
+    const double d = WIDE ? __longlong_as_double(v) : __ll2double_rn(v);
+    const int hi = __double2hiint(d);
+    return __hiloint2double(hi == 0 ? 0 : hi + (sc << 20), __double2loint(d));
+}
+template <bool WIDE>
+__device__ __noinline__ void store_general(const SplitArgs &a, long long v, int sc, int m, int n, long long off)
+{
+    if (WIDE) store_wide(a, __longlong_as_double(v), sc, m, n, off);
+    else a.C[off] = scaled_int_to_double(v, sc);
 }
 
 template <int NT, int T, bool DEEP = false>
@@ -586,32 +664,48 @@ gemm_split_kernel(SplitArgs a)
     constexpr int UNIT = 2 * sp_top_bits(T) + 8 * (T - 1);   // the sums' unit is 2^(E_A + E_B - UNIT)
     constexpr int TMEM_COLS = SpCfg<NT>::TMEM_COLS;
     extern __shared__ unsigned char smem_raw[];
-    __shared__ uint64_t bars[SP_ASLOTS * 2 + SP_BSLOTS * 2 + 3];
+    constexpr int ONE_ASLOTS = DEEP ? 0 : sp_aslots_one(NT, T);           // A slots of a CTA with one K tile
+    constexpr int MAX_ASLOTS = SP_ASLOTS > ONE_ASLOTS ? SP_ASLOTS : ONE_ASLOTS;
+    __shared__ uint64_t bars[MAX_ASLOTS * 2 + SP_BSLOTS * 2 + 3];
     __shared__ uint32_t tmem_base_sh;
     __shared__ int abort_sh;
 
     unsigned char *sm = (unsigned char *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
-    unsigned char *Asm = sm;                                   // SP_ASLOTS x A_TILE
-    unsigned char *Bsm = sm + SP_ASLOTS * A_TILE;              // SP_BSLOTS x (T x B_TILE)
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const uint32_t bar0 = smem_u32(bars);
-    auto A_full = [&](int s) { return bar0 + 8u * s; };
-    auto A_empty = [&](int s) { return bar0 + 8u * (SP_ASLOTS + s); };
-    auto B_full = [&](int s) { return bar0 + 8u * (2 * SP_ASLOTS + s); };
-    auto B_empty = [&](int s) { return bar0 + 8u * (2 * SP_ASLOTS + SP_BSLOTS + s); };
-    const uint32_t ACC_FULL = bar0 + 8u * (2 * SP_ASLOTS + 2 * SP_BSLOTS);
-    const uint32_t ACC_EMPTY = ACC_FULL + 8u;
-    const uint32_t DRAIN = ACC_FULL + 16u;
-
     const int nt = blockIdx.x, mt = blockIdx.y, ks = blockIdx.z;
     const int total_chunks = (a.kTiles + SP_KT_PER_CHUNK - 1) / SP_KT_PER_CHUNK;
     const int c_beg = ks * a.chunks_per_split;
     const int c_end = min(total_chunks, c_beg + a.chunks_per_split);
+    const int kt_beg = c_beg * SP_KT_PER_CHUNK, nkt = min(a.kTiles, c_end * SP_KT_PER_CHUNK) - kt_beg;
+    const int aslots = nkt == 1 && !DEEP ? ONE_ASLOTS : SP_ASLOTS;
+    unsigned char *Asm = sm;                                   // aslots x A_TILE
+    unsigned char *Bsm = sm + aslots * A_TILE;                 // SP_BSLOTS (one K tile: 1) x (T x B_TILE)
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const uint32_t bar0 = smem_u32(bars);
+    auto A_full = [&](int s) { return bar0 + 8u * s; };
+    auto A_empty = [&](int s) { return bar0 + 8u * (MAX_ASLOTS + s); };
+    auto B_full = [&](int s) { return bar0 + 8u * (2 * MAX_ASLOTS + s); };
+    auto B_empty = [&](int s) { return bar0 + 8u * (2 * MAX_ASLOTS + SP_BSLOTS + s); };
+    const uint32_t ACC_FULL = bar0 + 8u * (2 * MAX_ASLOTS + 2 * SP_BSLOTS);
+    const uint32_t ACC_EMPTY = ACC_FULL + 8u;
+    const uint32_t DRAIN = ACC_FULL + 16u;
+
     volatile int *abort_flag = &abort_sh;
+
+    // Copy u of the A stream (slice u % T of K tile u / T) and b of the B stream into their slots
+    auto a_slot = [&](int u) { return nkt == 1 && !DEEP ? u % (ONE_ASLOTS > 0 ? ONE_ASLOTS : 1) : u % SP_ASLOTS; };
+    auto a_round = [&](int u) { return nkt == 1 && !DEEP ? u / (ONE_ASLOTS > 0 ? ONE_ASLOTS : 1) : u / SP_ASLOTS; };
+    auto copy = [&](uint32_t bar, uint32_t dst, const unsigned char *src, uint32_t bytes) {
+        mbar_expect_tx(bar, bytes);
+        bulk_g2s(dst, src, bytes, bar);
+    };
+    auto a_src = [&](int u) { return a.Apk + (((long long)mt * a.kTiles + kt_beg) * T + u) * A_TILE; };
+    auto b_src = [&](int b) { return a.Bpk + ((long long)nt * a.kTiles + kt_beg + b) * (T * B_TILE); };
+    // copies that need no empty slot: issued below, before the CTA's first barrier
+    const int b_first = min(nkt, nkt == 1 ? 1 : SP_BSLOTS), a_first = min(nkt * T, aslots);
 
     if (threadIdx.x == 0) {
         abort_sh = 0;
-        for (int s = 0; s < SP_ASLOTS; ++s) {
+        for (int s = 0; s < MAX_ASLOTS; ++s) {
             mbar_init(A_full(s), 1);
             mbar_init(A_empty(s), 1);
         }
@@ -625,6 +719,18 @@ gemm_split_kernel(SplitArgs a)
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (warp == 0) {
+        // the first copies start while warp 1 allocates TMEM and the others arrive: lane 0 the B
+        // tiles, lane 1 the A slices, side by side in the same instructions
+        if (lane == 0) asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        __syncwarp();
+        for (int q = 0; q < MAX_ASLOTS; ++q) {
+            const bool isb = lane == 0;
+            if (lane < 2 && q < (isb ? b_first : a_first))
+                copy(isb ? B_full(q) : A_full(q), smem_u32(isb ? Bsm + q * (T * B_TILE) : Asm + q * A_TILE),
+                     isb ? b_src(q) : a_src(q), isb ? (uint32_t)(T * B_TILE) : (uint32_t)A_TILE);
+        }
+        __syncwarp();
+    } else if (warp == 1) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base_sh)),
                      "r"(TMEM_COLS)
                      : "memory");
@@ -641,30 +747,16 @@ gemm_split_kernel(SplitArgs a)
         // A slices; each blocks only on its own ring, so the A stream runs ahead of a
         // full B ring instead of queueing behind it
         if (lane == 0) {
-            int b = 0;
-            for (int c = c_beg; c < c_end && !*abort_flag; ++c) {
-                const int kt0 = c * SP_KT_PER_CHUNK, kt1 = min(a.kTiles, kt0 + SP_KT_PER_CHUNK);
-                for (int kt = kt0; kt < kt1; ++kt, ++b) {
-                    const int sb = b % SP_BSLOTS;
-                    if (!mbar_wait(B_empty(sb), ((b / SP_BSLOTS) & 1) ^ 1, abort_flag)) break;
-                    mbar_expect_tx(B_full(sb), (uint32_t)(T * B_TILE));
-                    bulk_g2s(smem_u32(Bsm + sb * T * B_TILE),
-                             a.Bpk + ((long long)nt * a.kTiles + kt) * (T * B_TILE), T * B_TILE, B_full(sb));
-                }
+            for (int b = b_first; b < nkt && !*abort_flag; ++b) {
+                const int sb = b % SP_BSLOTS;
+                if (!mbar_wait(B_empty(sb), ((b / SP_BSLOTS) & 1) ^ 1, abort_flag)) break;
+                copy(B_full(sb), smem_u32(Bsm + sb * (T * B_TILE)), b_src(b), (uint32_t)(T * B_TILE));
             }
         } else if (lane == 1) {
-            int u = 0;
-            for (int c = c_beg; c < c_end && !*abort_flag; ++c) {
-                const int kt0 = c * SP_KT_PER_CHUNK, kt1 = min(a.kTiles, kt0 + SP_KT_PER_CHUNK);
-                for (int kt = kt0; kt < kt1 && !*abort_flag; ++kt) {
-                    for (int i = 0; i < T; ++i, ++u) {
-                        const int sa = u % SP_ASLOTS;
-                        if (!mbar_wait(A_empty(sa), ((u / SP_ASLOTS) & 1) ^ 1, abort_flag)) break;
-                        mbar_expect_tx(A_full(sa), (uint32_t)A_TILE);
-                        const unsigned char *src = a.Apk + (((long long)mt * a.kTiles + kt) * T + i) * A_TILE;
-                        bulk_g2s(smem_u32(Asm + sa * A_TILE), src, A_TILE, A_full(sa));
-                    }
-                }
+            for (int u = a_first; u < nkt * T && !*abort_flag; ++u) {
+                const int sa = a_slot(u);
+                if (!mbar_wait(A_empty(sa), (a_round(u) & 1) ^ 1, abort_flag)) break;
+                copy(A_full(sa), smem_u32(Asm + sa * A_TILE), a_src(u), (uint32_t)A_TILE);
             }
         }
     } else if (warp == 1) {
@@ -695,8 +787,8 @@ gemm_split_kernel(SplitArgs a)
                     const uint64_t bdb = bd0 + (uint64_t)((sb * T * B_TILE) >> 4);
 #pragma unroll
                     for (int i = 0; i < T; ++i) {
-                        const int sa = u % SP_ASLOTS;
-                        if (!mbar_wait(A_full(sa), (u / SP_ASLOTS) & 1, abort_flag)) break;
+                        const int sa = a_slot(u);
+                        if (!mbar_wait(A_full(sa), a_round(u) & 1, abort_flag)) break;
                         tc_fence_after();
                         const uint64_t ad = ad0 + (uint64_t)((sa * A_TILE) >> 4);
 #pragma unroll
@@ -736,6 +828,20 @@ gemm_split_kernel(SplitArgs a)
         const int sub = warp & 3;              // TMEM sub-partition this warp may read
         const int part = (warp - 2) >> 2;      // which slice of the NT columns
         const uint32_t lane_base = (uint32_t)(32 * sub) << 16;
+        // this thread's output row (or column): offset and exponent scale, fetched while the
+        // operands are on their way and put into shared memory with the sums
+        const int et = threadIdx.x - 64;   // epilogue thread index
+        const int m0 = mt * SP_BM, n0 = nt * NT;
+        const int rows = min(SP_BM, a.M - m0), cols = min(NT, a.N - n0);
+        const bool fin = a.ksplit == 1;   // FP64 output here, else int64 sums to the split-K buffer
+        SpLine line{0, 0, 0};
+        if (et < rows) {
+            line.off = fin ? off2(a.Cm, m0 + et) : (long long)(m0 + et) * a.N;
+            line.sc = fin ? operand_scale<T>(__ldg(a.eA + m0 + et)) - UNIT : 0;
+        } else if (et >= SP_BM && et < SP_BM + cols) {
+            line.off = fin ? off2(a.Cn, n0 + et - SP_BM) : (long long)(n0 + et - SP_BM);
+            line.sc = fin ? operand_scale<T>(__ldg(a.eB + n0 + et - SP_BM)) : 0;
+        }
         long long acc[QW], acl[WIDE ? QW : 1];   // acl: levels 4 .. 7 of the FP64 slices
 #pragma unroll
         for (int q = 0; q < QW; ++q) acc[q] = 0;
@@ -762,9 +868,15 @@ gemm_split_kernel(SplitArgs a)
                 tmem_wait_ld();
 #pragma unroll
                 for (int q = 0; q < QW; ++q) {
-                    const int v = __float2int_rn(__uint_as_float(r[q]));
-                    if (WIDE && t >= 4) acl[WIDE ? q : 0] += (long long)v * (1 << sh);
-                    else if (WIDE) acc[q] += (long long)v * (1 << sh);
+                    // Integer of the level sum.  Up to 2^22 in magnitude, adding 1.5 2^23 leaves it in
+                    // the low bits (one FP32 addition at full rate); above, the conversion
+                    // instruction (a quarter of a warp per cycle and SM).
+                    const bool low = level_max<T>(t, SP_KT_PER_CHUNK * SP_BK) <= (1 << 22) ||
+                                     (level_max<T>(t, SP_BK) <= (1 << 22) && nkt == 1);
+                    const float f = __uint_as_float(r[q]);
+                    const int v = low ? __float_as_int(f + 12582912.0f) - 0x4B400000 : __float2int_rn(f);
+                    if (WIDE && t >= 4) acl[WIDE ? q : 0] += (long long)v * (1 << (sh & 31));
+                    else if (sh < 31) acc[q] += (long long)v * (1 << (sh & 31));
                     else acc[q] += (long long)v << sh;
                 }
             }
@@ -780,14 +892,9 @@ gemm_split_kernel(SplitArgs a)
         constexpr int PITCH = NT + 1;
         long long *stage = reinterpret_cast<long long *>(sm);
         long long *stage_lo = stage + SP_BM * PITCH;   // FP64 slices with split-K: the second accumulator
-        long long *row_off = stage + (WIDE ? 2 : 1) * SP_BM * PITCH;
-        long long *col_off = row_off + SP_BM;
-        int *row_sc = reinterpret_cast<int *>(col_off + NT);   // exponent scales of the output
-        int *col_sc = row_sc + SP_BM;
-        const int ew = warp - 2, et = threadIdx.x - 64;   // epilogue warp / thread index
-        const int m0 = mt * SP_BM, n0 = nt * NT;
-        const int rows = min(SP_BM, a.M - m0), cols = min(NT, a.N - n0);
-        const bool fin = a.ksplit == 1;   // FP64 output here, else int64 sums to the split-K buffer
+        // offsets of the output maps and exponent scales
+        SpLine *rowl = reinterpret_cast<SpLine *>(stage + (((WIDE ? 2 : 1) * SP_BM * PITCH + 1) & ~1));
+        SpLine *coll = rowl + SP_BM;
         if (!*abort_flag) {
             // the raw sums go to shared memory; they are converted in the write-out,
             // where the accumulator registers are free and a batch of values converts
@@ -796,10 +903,6 @@ gemm_split_kernel(SplitArgs a)
             const int r = 32 * sub + lane;
             const int m = m0 + r;
             if (m < a.M) {
-                if (part == 0) {
-                    row_off[r] = fin ? off2(a.Cm, m) : (long long)m * a.N;
-                    row_sc[r] = fin ? operand_scale<T>(__ldg(a.eA + m)) - UNIT : 0;
-                }
 #pragma unroll
                 for (int q = 0; q < QW; ++q) {
                     const int c = part * QW + q;
@@ -812,95 +915,116 @@ gemm_split_kernel(SplitArgs a)
                     }
                 }
             }
-            for (int c = et; c < cols; c += SP_EPI_THREADS) {
-                col_off[c] = fin ? off2(a.Cn, n0 + c) : (long long)(n0 + c);
-                col_sc[c] = fin ? operand_scale<T>(__ldg(a.eB + n0 + c)) : 0;
-            }
+            if (et < rows) rowl[et] = line;
+            else if (et >= SP_BM && et < SP_BM + cols) coll[et - SP_BM] = line;
         }
         asm volatile("bar.sync 1, %0;" ::"n"(SP_EPI_THREADS) : "memory");
         if (!*abort_flag) {
-            // Write-out in groups of WU rows (columns): the staged values, offsets and
-            // scales of a group are read from shared memory before its stores.
-            constexpr int WU = 4;
+            // Write-out with the lanes along whichever output index is contiguous.  Along columns a
+            // group of RG rows is a whole number of warp instructions (two rows of a 48-wide tile
+            // are three), so a lane's columns are the same in every group: offsets and scales of its
+            // columns stay in registers, those of the row come as one shared-memory word.
+            const int ew = warp - 2;
             const bool along_n = (a.ksplit > 1) || a.Cn.s2 == 1 || a.Cm.s2 != 1;
             if (along_n) {
-                constexpr int NCH = (NT + 31) / 32;   // 32-column chunks of a row
-                long long co[NCH];
-                int cs[NCH];
+                constexpr int RG = NT % 32 ? 2 : 1, NI = RG * NT / 32;
+                int cr[NI], cc[NI], cs[NI];
+                long long co[NI];
 #pragma unroll
-                for (int j = 0; j < NCH; ++j) {
-                    const bool in = lane + 32 * j < cols;
-                    co[j] = in ? col_off[lane + 32 * j] : 0;
-                    cs[j] = in ? col_sc[lane + 32 * j] : 0;
+                for (int q = 0; q < NI; ++q) {
+                    const int e = lane + 32 * q;
+                    cr[q] = e / NT;
+                    cc[q] = e % NT;
+                    const SpLine cl = coll[min(cc[q], cols - 1)];
+                    co[q] = cl.off;
+                    cs[q] = cl.sc;
                 }
-                for (int rb = ew; rb < rows; rb += WU * SP_EPI_WARPS) {
-                    long long ro[WU], v[WU][NCH];
-                    int rsc[WU];
+                constexpr int GP = NI >= 3 ? 2 : 4;   // row groups whose reads precede their stores
+                for (int g0 = ew * RG; g0 < rows; g0 += GP * SP_EPI_WARPS * RG) {
+                    long long v[GP][NI], ro[GP][NI];
+                    int sc[GP][NI];
 #pragma unroll
-                    for (int w = 0; w < WU; ++w) {
-                        const int r = rb + w * SP_EPI_WARPS;
-                        ro[w] = r < rows ? row_off[r] : 0;
-                        rsc[w] = r < rows ? row_sc[r] : 0;
+                    for (int u = 0; u < GP; ++u)
 #pragma unroll
-                        for (int j = 0; j < NCH; ++j)
-                            v[w][j] = (r < rows && lane + 32 * j < cols) ? stage[r * PITCH + lane + 32 * j] : 0;
-                    }
-#pragma unroll
-                    for (int w = 0; w < WU; ++w) {
-                        if (rb + w * SP_EPI_WARPS >= rows) break;
-#pragma unroll
-                        for (int j = 0; j < NCH; ++j) {
-                            if (lane + 32 * j >= cols) continue;
-                            if (WIDE && fin) {
-                                store_wide(a, __longlong_as_double(v[w][j]), rsc[w] + cs[j],
-                                           m0 + rb + w * SP_EPI_WARPS, n0 + lane + 32 * j, ro[w] + co[j]);
-                            } else if (fin) {
-                                a.C[ro[w] + co[j]] = scaled_int_to_double(v[w][j], rsc[w] + cs[j]);
-                            } else {
-                                atomicAdd(&a.partial[ro[w] + co[j]], (unsigned long long)v[w][j]);
-                                if (WIDE)
-                                    atomicAdd(&a.partial[(long long)a.M * a.N + ro[w] + co[j]],
-                                              (unsigned long long)stage_lo[(rb + w * SP_EPI_WARPS) * PITCH + lane + 32 * j]);
-                            }
+                        for (int q = 0; q < NI; ++q) {
+                            const int r = min(g0 + u * SP_EPI_WARPS * RG + cr[q], rows - 1);
+                            const SpLine rl = rowl[r];
+                            ro[u][q] = rl.off + co[q];
+                            sc[u][q] = rl.sc + cs[q];
+                            v[u][q] = stage[r * PITCH + cc[q]];
                         }
+                    if (!fin) {
+#pragma unroll
+                        for (int u = 0; u < GP; ++u)
+#pragma unroll
+                            for (int q = 0; q < NI; ++q) {
+                                const int r = g0 + u * SP_EPI_WARPS * RG + cr[q];
+                                if (r >= rows || cc[q] >= cols) continue;
+                                atomicAdd(&a.partial[ro[u][q]], (unsigned long long)v[u][q]);
+                                if (WIDE)
+                                    atomicAdd(&a.partial[(long long)a.M * a.N + ro[u][q]],
+                                              (unsigned long long)stage_lo[r * PITCH + cc[q]]);
+                            }
+                        continue;
                     }
+                    // every third conversion on the integer pipes (see scaled_int_to_double_i); all
+                    // of them before the first store
+                    bool ok = !WIDE || a.plain;
+                    double d[GP][NI];
+#pragma unroll
+                    for (int u = 0; u < GP; ++u)
+#pragma unroll
+                        for (int q = 0; q < NI; ++q) {
+                            ok = ok && scale_in_range(sc[u][q]);
+                            d[u][q] = out_value<WIDE>(v[u][q], sc[u][q], NI >= 3 && q == NI - 1);
+                        }
+#pragma unroll
+                    for (int u = 0; u < GP; ++u)
+#pragma unroll
+                        for (int q = 0; q < NI; ++q) {
+                            const int r = g0 + u * SP_EPI_WARPS * RG + cr[q];
+                            if (ok && r < rows && cc[q] < cols) a.C[ro[u][q]] = d[u][q];
+                        }
+                    if (!ok)
+#pragma unroll 1
+                        for (int e = 0; e < GP * NI; ++e) {
+                            const int ee = lane + 32 * (e % NI);
+                            const int r = g0 + (e / NI) * SP_EPI_WARPS * RG + ee / NT, c = ee % NT;
+                            if (r < rows && c < cols)
+                                store_general<WIDE>(a, stage[r * PITCH + c], rowl[r].sc + coll[c].sc, m0 + r, n0 + c,
+                                                    rowl[r].off + coll[c].off);
+                        }
                 }
             } else {
                 constexpr int NRC = SP_BM / 32;   // 32-row chunks of a column
                 long long ro[NRC];
                 int rsc[NRC];
 #pragma unroll
-                for (int j = 0; j < NRC; ++j) {
-                    const bool in = lane + 32 * j < rows;
-                    ro[j] = in ? row_off[lane + 32 * j] : 0;
-                    rsc[j] = in ? row_sc[lane + 32 * j] : 0;
+                for (int q = 0; q < NRC; ++q) {
+                    const SpLine rl = rowl[min(lane + 32 * q, rows - 1)];
+                    ro[q] = rl.off;
+                    rsc[q] = rl.sc;
                 }
-                for (int cb = ew; cb < cols; cb += WU * SP_EPI_WARPS) {
-                    long long co[WU], v[WU][NRC];
-                    int cs[WU];
+                for (int c = ew; c < cols; c += SP_EPI_WARPS) {
+                    const SpLine cl = coll[c];
+                    long long v[NRC];
 #pragma unroll
-                    for (int w = 0; w < WU; ++w) {
-                        const int c = cb + w * SP_EPI_WARPS;
-                        co[w] = c < cols ? col_off[c] : 0;
-                        cs[w] = c < cols ? col_sc[c] : 0;
+                    for (int q = 0; q < NRC; ++q) v[q] = stage[min(lane + 32 * q, rows - 1) * PITCH + c];
+                    bool ok = !WIDE || a.plain;
+                    double d[NRC];
 #pragma unroll
-                        for (int j = 0; j < NRC; ++j)
-                            v[w][j] = (c < cols && lane + 32 * j < rows) ? stage[(lane + 32 * j) * PITCH + c] : 0;
+                    for (int q = 0; q < NRC; ++q) {
+                        ok = ok && scale_in_range(rsc[q] + cl.sc);
+                        d[q] = out_value<WIDE>(v[q], rsc[q] + cl.sc, q == NRC - 1);
                     }
 #pragma unroll
-                    for (int w = 0; w < WU; ++w) {
-                        if (cb + w * SP_EPI_WARPS >= cols) break;
-#pragma unroll
-                        for (int j = 0; j < NRC; ++j)
-                        {
-                            if (lane + 32 * j >= rows) continue;
-                            if (WIDE)
-                                store_wide(a, __longlong_as_double(v[w][j]), rsc[j] + cs[w], m0 + lane + 32 * j,
-                                           n0 + cb + w * SP_EPI_WARPS, ro[j] + co[w]);
-                            else
-                                a.C[ro[j] + co[w]] = scaled_int_to_double(v[w][j], rsc[j] + cs[w]);
-                        }
-                    }
+                    for (int q = 0; q < NRC; ++q)
+                        if (ok && lane + 32 * q < rows) a.C[ro[q] + cl.off] = d[q];
+                    if (!ok)
+#pragma unroll 1
+                        for (int r = lane; r < rows; r += 32)
+                            store_general<WIDE>(a, stage[r * PITCH + c], rowl[r].sc + cl.sc, m0 + r, n0 + c,
+                                                rowl[r].off + cl.off);
                 }
             }
         }
@@ -910,7 +1034,7 @@ gemm_split_kernel(SplitArgs a)
     if (abort_sh && threadIdx.x == 0)
         for (int i = 0; i < 2000; ++i) __nanosleep(100);   // let bulk copies still in flight land
     __syncthreads();
-    if (warp == 0) {
+    if (warp == 1) {
         __syncwarp();
         tc_fence_after();
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(TMEM_COLS) : "memory");
@@ -959,8 +1083,11 @@ size_t split_smem_bytes(int T)
     const int aslots = DEEP ? (T == 2 ? SpDeep<2>::A : T == 3 ? SpDeep<3>::A : T == 4 ? SpDeep<4>::A : SpDeep<5>::A)
                             : sp_aslots(NT, T);
     size_t b = 1024 + (size_t)aslots * SP_BM * SP_BK * 2 + (size_t)SP_BSLOTS * T * NT * SP_BK * 2;
+    // one K tile: more A slots, one B slot (NT = 48, T = 5: 113664 bytes, still two CTAs per SM)
+    const size_t one = 1024 + (size_t)(DEEP ? 0 : sp_aslots_one(NT, T)) * SP_BM * SP_BK * 2 + (size_t)T * NT * SP_BK * 2;
+    if (b < one) b = one;
     const size_t out_stage =
-        1024 + (size_t)SP_BM * (NT + 1) * (sp_wide(T) ? 16 : 8) + (size_t)(SP_BM + NT) * 12;   // epilogue reuse
+        1024 + (size_t)SP_BM * (NT + 1) * (sp_wide(T) ? 16 : 8) + (size_t)(SP_BM + NT) * 16;   // epilogue reuse
     if (b < out_stage) b = out_stage;
     if ((DEEP || SpCfg<NT>::MIN_BLOCKS == 1) && b < 120 * 1024) b = 120 * 1024;
     return b;
@@ -1029,8 +1156,8 @@ SplitPlan split_plan_caps(int M, int N, int K, int T)
     return c;
 }
 
-// Both sides measured on either side of this line: MNK = 8.4e6 27 (FP64 pipe) against 28 us and
-// 51 against 38; 4.2e6 31 against 37 and 16 against 27; 2.5e7 86 against 43.
+// Both sides measured on either side of this line (us, FP64 pipe against slices): MNK = 8.4e6
+// 28 : 26, 33 : 38 and 33 : 34; 4.2e6 19 : 36 and 16 : 24; 1.3e7 33 : 30; 2.5e7 85 : 43.
 bool split_f64_pays(int M, int N, int K) { return (double)M * N * K >= 8e6; }
 
 bool split_fits(int M, int N, int K, int T, const SplitWork &w)
@@ -1313,6 +1440,7 @@ static cudaError_t gemm_split_run(const GemmF64 &g, int T, SplitWork w, cudaStre
                 w.err,
                 g.alpha,
                 g.beta,
+                g.alpha == 1.0 && g.beta == 0.0,
                 g.A,
                 g.B,
                 g.Am,
