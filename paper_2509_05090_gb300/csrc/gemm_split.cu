@@ -32,8 +32,8 @@
 // at every shape and for normal, uniform, graded and constant operands, the FP64 GEMM 1e-16
 // to 2e-15.  Rows and columns with infinities or NaNs have no grid; their outputs are the
 // plain FP64 sums.  Against the FP64 pipe's GEMM: 8192 x 8192 x 128 14.09 -> 0.89 ms,
-// 8192 x 128 x 8192 14.30 -> 0.96 ms, 2592 x 2592 x 72 849 -> 111 us, 2592 x 72 x 2592
-// 935 -> 141 us, 900 x 900 x 36 72 -> 29 us; below MNK = 8e6 (512 x 512 x 32: 28 against
+// 8192 x 128 x 8192 14.30 -> 0.96 ms, 2592 x 2592 x 72 849 -> 107 us, 2592 x 72 x 2592
+// 935 -> 135 us, 900 x 900 x 36 72 -> 29 us; below MNK = 8e6 (512 x 512 x 32: 28 against
 // 26 us, 512 x 32 x 512: 33 against 38, 243 x 243 x 27: 11 against 26) the two packs and three
 // launches cost more than the FP64 GEMM, which keeps those shapes (split_f64_pays).
 //
@@ -57,9 +57,8 @@
 // row's and column's address and scale once, converts before it stores and scales by an integer
 // add, since every FP64 instruction, conversions and compares included, holds its
 // sub-partition's FP64 pipe for 64 cycles.  T = 5: 2592 x 2592 x 72 58.9 -> 49.9 us, 5184 x 1296 x 36
-// 52.7 -> 42.7, 512 x 512 x 32 15.0 -> 11.8; T = 8: 2592 x 2592 x 72 131 -> 90, 8192 x 8192 x 128
-// 1077 -> 889.  At large K the MMAs bound it (2592 x 72 x 2592, T = 8: 100 us, 98 % of the
-// CTA's time in the K loop).
+// 52.7 -> 42.7, 512 x 512 x 32 15.0 -> 11.8; T = 8: 2592 x 2592 x 72 131 -> 86, 8192 x 8192 x 128
+// 1077 -> 889.  At large K the K loop is all (2592 x 72 x 2592, T = 8: 88 % of a CTA's time).
 #include <cuda_bf16.h>
 
 #include <vector>
@@ -88,13 +87,18 @@ __host__ __device__ constexpr bool sp_wide(int T) { return T > 5; }
 // T = 8 takes NT = 32 (256 TMEM columns, 97 KB, two CTAs per SM) or NT = 64.
 constexpr int sp_aslots(int nt, int T)
 {
-    return T == 8 ? (nt == 32 ? 2 : 6) : nt == 96 ? 6 : (nt == 64 ? 8 : 3);
+    return T == 8 ? (nt == 32 ? 4 : 6) : nt == 96 ? 6 : (nt == 64 ? 8 : 3);
 }
+// B slots: all T slices of a K tile each.  At T = 8, NT = 32 two of them (64 KB) left a CTA two A
+// slots, and a copy's latency (~1.3k cycles) bounded the K loop; with one B slot and four A slots
+// the other CTA of the SM covers the wait for the next K tile's B: 2592 x 72 x 2592 100 -> 80 us,
+// 2592 x 2592 x 72 90 -> 86.
+constexpr int sp_bslots(int nt, int T) { return T == 8 && nt == 32 ? 1 : SP_BSLOTS; }
 // A CTA with a single K tile needs one B slot: the other one's space holds more A slices, so
 // that all T of them are in flight at once.
 constexpr int sp_aslots_one(int nt, int T)
 {
-    const int extra = T * nt * 64 * 2 / (128 * 64 * 2) + (nt == 48 && T == 5 ? 1 : 0);   // (2 KB more, see split_smem_bytes)
+    const int extra = (sp_bslots(nt, T) - 1) * T * nt * 64 * 2 / (128 * 64 * 2) + (nt == 48 && T == 5 ? 1 : 0);   // (2 KB more, see split_smem_bytes)
     const int n = sp_aslots(nt, T) + extra;
     return n > T ? (sp_aslots(nt, T) > T ? sp_aslots(nt, T) : T) : n;
 }
@@ -657,6 +661,7 @@ gemm_split_kernel(SplitArgs a)
     constexpr int B_TILE = NT * SP_BK * 2;
     constexpr int QW = NT / (SpCfg<NT>::EPI_WARPS / 4);   // columns per epilogue warp
     constexpr int SP_ASLOTS = DEEP ? SpDeep<T>::A : sp_aslots(NT, T);
+    constexpr int BSLOTS = sp_bslots(NT, T);
     constexpr int SP_EPI_WARPS = SpCfg<NT>::EPI_WARPS;
     constexpr int SP_EPI_THREADS = SpCfg<NT>::EPI_THREADS;
     constexpr int SP_KT_PER_CHUNK = sp_chunk_kt(T);
@@ -666,7 +671,7 @@ gemm_split_kernel(SplitArgs a)
     extern __shared__ unsigned char smem_raw[];
     constexpr int ONE_ASLOTS = DEEP ? 0 : sp_aslots_one(NT, T);           // A slots of a CTA with one K tile
     constexpr int MAX_ASLOTS = SP_ASLOTS > ONE_ASLOTS ? SP_ASLOTS : ONE_ASLOTS;
-    __shared__ uint64_t bars[MAX_ASLOTS * 2 + SP_BSLOTS * 2 + 3];
+    __shared__ uint64_t bars[MAX_ASLOTS * 2 + BSLOTS * 2 + 3];
     __shared__ uint32_t tmem_base_sh;
     __shared__ int abort_sh;
 
@@ -678,14 +683,14 @@ gemm_split_kernel(SplitArgs a)
     const int kt_beg = c_beg * SP_KT_PER_CHUNK, nkt = min(a.kTiles, c_end * SP_KT_PER_CHUNK) - kt_beg;
     const int aslots = nkt == 1 && !DEEP ? ONE_ASLOTS : SP_ASLOTS;
     unsigned char *Asm = sm;                                   // aslots x A_TILE
-    unsigned char *Bsm = sm + aslots * A_TILE;                 // SP_BSLOTS (one K tile: 1) x (T x B_TILE)
+    unsigned char *Bsm = sm + aslots * A_TILE;                 // BSLOTS (one K tile: 1) x (T x B_TILE)
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t bar0 = smem_u32(bars);
     auto A_full = [&](int s) { return bar0 + 8u * s; };
     auto A_empty = [&](int s) { return bar0 + 8u * (MAX_ASLOTS + s); };
     auto B_full = [&](int s) { return bar0 + 8u * (2 * MAX_ASLOTS + s); };
-    auto B_empty = [&](int s) { return bar0 + 8u * (2 * MAX_ASLOTS + SP_BSLOTS + s); };
-    const uint32_t ACC_FULL = bar0 + 8u * (2 * MAX_ASLOTS + 2 * SP_BSLOTS);
+    auto B_empty = [&](int s) { return bar0 + 8u * (2 * MAX_ASLOTS + BSLOTS + s); };
+    const uint32_t ACC_FULL = bar0 + 8u * (2 * MAX_ASLOTS + 2 * BSLOTS);
     const uint32_t ACC_EMPTY = ACC_FULL + 8u;
     const uint32_t DRAIN = ACC_FULL + 16u;
 
@@ -701,7 +706,7 @@ gemm_split_kernel(SplitArgs a)
     auto a_src = [&](int u) { return a.Apk + (((long long)mt * a.kTiles + kt_beg) * T + u) * A_TILE; };
     auto b_src = [&](int b) { return a.Bpk + ((long long)nt * a.kTiles + kt_beg + b) * (T * B_TILE); };
     // copies that need no empty slot: issued below, before the CTA's first barrier
-    const int b_first = min(nkt, nkt == 1 ? 1 : SP_BSLOTS), a_first = min(nkt * T, aslots);
+    const int b_first = min(nkt, nkt == 1 ? 1 : BSLOTS), a_first = min(nkt * T, aslots);
 
     if (threadIdx.x == 0) {
         abort_sh = 0;
@@ -709,7 +714,7 @@ gemm_split_kernel(SplitArgs a)
             mbar_init(A_full(s), 1);
             mbar_init(A_empty(s), 1);
         }
-        for (int s = 0; s < SP_BSLOTS; ++s) {
+        for (int s = 0; s < BSLOTS; ++s) {
             mbar_init(B_full(s), 1);
             mbar_init(B_empty(s), 1);
         }
@@ -748,8 +753,8 @@ gemm_split_kernel(SplitArgs a)
         // full B ring instead of queueing behind it
         if (lane == 0) {
             for (int b = b_first; b < nkt && !*abort_flag; ++b) {
-                const int sb = b % SP_BSLOTS;
-                if (!mbar_wait(B_empty(sb), ((b / SP_BSLOTS) & 1) ^ 1, abort_flag)) break;
+                const int sb = b % BSLOTS;
+                if (!mbar_wait(B_empty(sb), ((b / BSLOTS) & 1) ^ 1, abort_flag)) break;
                 copy(B_full(sb), smem_u32(Bsm + sb * (T * B_TILE)), b_src(b), (uint32_t)(T * B_TILE));
             }
         } else if (lane == 1) {
@@ -777,8 +782,8 @@ gemm_split_kernel(SplitArgs a)
                 tc_fence_after();
                 const int kt0 = c * SP_KT_PER_CHUNK, kt1 = min(a.kTiles, kt0 + SP_KT_PER_CHUNK);
                 for (int kt = kt0; kt < kt1; ++kt) {
-                    const int sb = b % SP_BSLOTS;
-                    if (!mbar_wait(B_full(sb), (b / SP_BSLOTS) & 1, abort_flag)) break;
+                    const int sb = b % BSLOTS;
+                    if (!mbar_wait(B_full(sb), (b / BSLOTS) & 1, abort_flag)) break;
                     tc_fence_after();
                     const int kvalid = min(SP_BK, a.K - kt * SP_BK);
                     const int ksteps = (kvalid + 15) / 16;
@@ -1082,7 +1087,7 @@ size_t split_smem_bytes(int T)
 {
     const int aslots = DEEP ? (T == 2 ? SpDeep<2>::A : T == 3 ? SpDeep<3>::A : T == 4 ? SpDeep<4>::A : SpDeep<5>::A)
                             : sp_aslots(NT, T);
-    size_t b = 1024 + (size_t)aslots * SP_BM * SP_BK * 2 + (size_t)SP_BSLOTS * T * NT * SP_BK * 2;
+    size_t b = 1024 + (size_t)aslots * SP_BM * SP_BK * 2 + (size_t)sp_bslots(NT, T) * T * NT * SP_BK * 2;
     // one K tile: more A slots, one B slot (NT = 48, T = 5: 113664 bytes, still two CTAs per SM)
     const size_t one = 1024 + (size_t)(DEEP ? 0 : sp_aslots_one(NT, T)) * SP_BM * SP_BK * 2 + (size_t)T * NT * SP_BK * 2;
     if (b < one) b = one;
