@@ -87,6 +87,9 @@ constexpr int SPLIT_F64_T = 8;
 // whether its packs fit the work buffers.
 bool split_f64_pays(int M, int N, int K);
 bool split_fits(int M, int N, int K, int T, const SplitWork &w);
+// B's pack alone (N x K, tiles NT wide): rewrites a kept pack whose operand changed.
+cudaError_t split_pack_b(int N, int K, const double *B, Idx2 Bn, Idx2 Bk, int T, int NT, int *e, unsigned char *pk,
+                         cudaStream_t st);
 cudaError_t split_prepare();
 // ev (may be null): three events, recorded around the contraction kernel (ev[0] before,
 // ev[1] after) and before its operand pre-pass (ev[2]).

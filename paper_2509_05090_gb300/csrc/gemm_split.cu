@@ -1386,6 +1386,13 @@ static cudaError_t split_prepass(int R, int K, const double *X, Idx2 rmap, Idx2 
     }
 }
 
+cudaError_t split_pack_b(int N, int K, const double *B, Idx2 Bn, Idx2 Bk, int T, int NT, int *e, unsigned char *pk,
+                         cudaStream_t st)
+{
+    const SplitPlan p = split_plan(SP_BM, N, K, T, NT);
+    return split_prepass(N, K, B, Bn, Bk, p.NT, p.nTiles, p.kTiles, T, e, pk, st);
+}
+
 static cudaError_t gemm_split_run(const GemmF64 &g, int T, SplitWork w, cudaStream_t st, cudaEvent_t *ev,
                                   SplitPlan p, const SplitOpts *opt = nullptr)
 {
