@@ -455,8 +455,7 @@ int enqueue_projector(ctm_ctx *c, double *Qout)
         CK(run_gemm(c, g));
         c->m_packed = 1;
     }
-    QrScratch qs = qr_scratch(c);
-    CK(qr_householder((int)n, chi, c->Y, Qout, c->R, qs, st));
+    CK(qr_householder((int)n, chi, c->Y, Qout, c->R, step_qr_scratch(c), st));
     return CTM_OK;
 }
 
@@ -637,8 +636,7 @@ int enqueue_step_profiled(ctm_ctx *c, cudaEvent_t *ev)
     }
     CK(cudaEventRecord(ev[2], st));
     {
-        QrScratch qs = qr_scratch(c);
-        CK(qr_householder((int)n, (int)chi, c->Y, c->Qn, c->R, qs, st));
+        CK(qr_householder((int)n, (int)chi, c->Y, c->Qn, c->R, step_qr_scratch(c), st));
     }
     CK(cudaEventRecord(ev[3], st));
     if ((rc = c->cfg.corner_mode ? enqueue_corner_from_r(c, c->Cn) : enqueue_corner(c, c->Qn, c->Cn)) != CTM_OK)

@@ -127,6 +127,16 @@ inline QrScratch qr_scratch(ctm_ctx *c)
     q.yslab = c->qr_slab;
     q.yslab_elems = c->qr_slab_elems;
     q.force_slab = c->qr_force_slab;
+    q.blocked = nullptr;
+    q.blocked_bytes = 0;
+    return q;
+}
+// ... of a step, whose H (n x n) is written only after the QR
+inline QrScratch step_qr_scratch(ctm_ctx *c)
+{
+    QrScratch q = qr_scratch(c);
+    q.blocked = c->H;
+    q.blocked_bytes = sizeof(double) * (size_t)c->n * c->n;
     return q;
 }
 enum {

@@ -151,6 +151,9 @@ struct QrScratch {
     // row blocks too tall for shared memory (qr_slab_doubles(n, k) > 0): a global slab
     double *yslab;
     size_t yslab_elems;
+    // workspace of the blocked factorisation (many columns): free while the QR runs; null: none
+    void *blocked;
+    size_t blocked_bytes;
     bool force_slab;   // the slab for every shape (CTM_QR_SLAB=1 at init: a check of that path)
 };
 size_t qr_wy_doubles(int n, int k);   // V + S + W + ta + split-K scratch

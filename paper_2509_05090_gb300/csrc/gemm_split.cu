@@ -601,7 +601,8 @@ struct SplitArgs {
     // FP64 slices (T = 8) only: C = alpha A B + beta C, and the operands, for rows and
     // columns that hold an infinity or a NaN
     double alpha, beta;
-    int plain;                       // alpha = 1 and beta = 0 (an FP64 compare per element would cost an FMA's time)
+    int plain;                       // 1: alpha = 1, beta = 0; 2: alpha = beta = 1 (an FP64 compare per element
+                                     // would cost an FMA's time)
     const double *A, *B;
     Idx2 Am, Ak, Bk, Bn;
 };
@@ -626,7 +627,7 @@ __device__ __noinline__ double plain_dot(const SplitArgs &a, int m, int n)
 __device__ __forceinline__ void store_wide(const SplitArgs &a, double d, int scale, int m, int n, long long off)
 {
     double v = scale > SP_NONFINITE / 2 ? plain_dot(a, m, n) : scale_exponent(d, scale);
-    if (!a.plain) {
+    if (a.plain != 1) {
         v *= a.alpha;
         if (a.beta != 0.0) v = fma(a.beta, a.C[off], v);
     }
@@ -988,7 +989,10 @@ gemm_split_kernel(SplitArgs a)
 #pragma unroll
                         for (int q = 0; q < NI; ++q) {
                             const int r = g0 + u * SP_EPI_WARPS * RG + cr[q];
-                            if (ok && r < rows && cc[q] < cols) a.C[ro[u][q]] = d[u][q];
+                            if (ok && r < rows && cc[q] < cols) {
+                                double *o = a.C + ro[u][q];
+                                *o = WIDE && a.plain == 2 ? *o + d[u][q] : d[u][q];
+                            }
                         }
                     if (!ok)
 #pragma unroll 1
@@ -1024,7 +1028,10 @@ gemm_split_kernel(SplitArgs a)
                     }
 #pragma unroll
                     for (int q = 0; q < NRC; ++q)
-                        if (ok && lane + 32 * q < rows) a.C[ro[q] + cl.off] = d[q];
+                        if (ok && lane + 32 * q < rows) {
+                            double *o = a.C + ro[q] + cl.off;
+                            *o = WIDE && a.plain == 2 ? *o + d[q] : d[q];
+                        }
                     if (!ok)
 #pragma unroll 1
                         for (int r = lane; r < rows; r += 32)
@@ -1452,7 +1459,7 @@ static cudaError_t gemm_split_run(const GemmF64 &g, int T, SplitWork w, cudaStre
                 w.err,
                 g.alpha,
                 g.beta,
-                g.alpha == 1.0 && g.beta == 0.0,
+                g.alpha != 1.0 ? 0 : g.beta == 0.0 ? 1 : g.beta == 1.0 ? 2 : 0,
                 g.A,
                 g.B,
                 g.Am,

@@ -42,7 +42,8 @@
 // from that cost; partial sums are combined by halving; nothing FP64 sits under a predicate.
 // n x k: 512 x 32 119 -> 66 us, 2592 x 72 307 -> 214 (panels 23k -> 13k cycles each, update and
 // Gram passes 17k -> 8k), 8192 x 128 1027 -> 833, 5184 x 144 987 -> 802, 12000 x 240
-// 2350 -> 1960.
+// 2350 -> 1960.  Many columns (4 n k^2 of them with Q formed) go to the blocked form near the end
+// of this file, which leaves that pipe the 64-column panels only: 12000 x 480 12.9 -> 4.3 ms.
 //
 // The grid barrier is one monotonic counter in global memory; its spin is
 // bounded (about a second) and on expiry sets an error flag that the host
@@ -127,10 +128,14 @@ struct QrArgs {
     double *spart;    // G x k x k: partial V^T V
     // row blocks too tall for shared memory: CTA c's block at yslab + c * rows_per * (k | 1)
     double *yslab;
+    // one panel of the blocked factorisation (qr_kernel's FACT): row pitch of Y, R and V (n x k
+    // here, all rows), and per column tau and the sign of R's diagonal
+    int pitch;
+    double *taus, *sgn;
 };
 
 // W = U^{-1} V_top^T with U = striu(S) + diag(S)/2 (unit diagonal where tau = 0).
-// The k right-hand sides are independent: CTA b of the QR grid solves columns
+// (V null: U^{-1} itself.)  The k right-hand sides are independent: CTA b of the QR grid solves columns
 // [4b, 4b + 4) after the grid barrier that completes S.
 // Rows are blocked by QR_WB = 8 from the bottom; every CTA first inverts the
 // diagonal 8 x 8 blocks of U (all blocks at once, one thread per block column),
@@ -186,7 +191,7 @@ __device__ void wy_solve_cta(int k, int cblk, const double *S, const double *V, 
         }
     for (int t = tid; t < k * QR_WC; t += blockDim.x) {
         const int i = t / QR_WC, cc = t % QR_WC;
-        Wc[t] = (cc < ncol) ? __ldcg(V + (size_t)(c0 + cc) * k + i) : 0.0;
+        Wc[t] = V ? ((cc < ncol) ? __ldcg(V + (size_t)(c0 + cc) * k + i) : 0.0) : (i == c0 + cc ? 1.0 : 0.0);
     }
     __syncthreads();
     for (int i = tid; i < k; i += blockDim.x) rd[i] = 1.0 / uval(i, i);
@@ -300,7 +305,9 @@ __device__ void q_rows(const QrArgs &a, const double *alps, const double *Ys, in
 
 // GY: the CTA's row block lives in a global slab (L2) instead of shared memory, for
 // blocks too tall for it (large k or n); the algorithm and the access order are the same.
-template <bool GY>
+// FACT: one panel of the blocked factorisation below, columns of a wider matrix: R's block, the
+// reflectors (each scaled by a power of two to v_0 in [1, 2)) and T = U^{-1} instead of Q.
+template <bool GY, bool FACT = false>
 __global__ void __launch_bounds__(QR_THREADS, 1) qr_kernel(QrArgs a)
 {
     extern __shared__ double sm[];
@@ -330,7 +337,9 @@ __global__ void __launch_bounds__(QR_THREADS, 1) qr_kernel(QrArgs a)
     };
     auto pub_buf = [&](int blk) { return a.rowbuf + (size_t)(blk & 1) * QB * k; };
 
-    for (int t = tid; t < nr * k; t += blockDim.x) Ys[(t / k) * ld + t % k] = a.Y[(size_t)r0 * k + t];
+    const int pitch = FACT ? a.pitch : k;
+    for (int t = tid; t < nr * k; t += blockDim.x)
+        Ys[(t / k) * ld + t % k] = FACT ? a.Y[(size_t)(r0 + t / k) * pitch + t % k] : a.Y[(size_t)r0 * k + t];
     __syncthreads();
 
     // The sweep of gram_pass below over the columns kk >= j1: P lanes per column share its rows
@@ -627,8 +636,8 @@ __global__ void __launch_bounds__(QR_THREADS, 1) qr_kernel(QrArgs a)
                     alps[j] = alpha;
                 }
                 if (c == 0) {
-                    for (int kk = lane; kk < j0; kk += 32) a.R[(size_t)j * k + kk] = 0.0;
-                    if (r == 0 && q < nn0) a.R[(size_t)j * k + j0 + q] = q < i ? 0.0 : (q == i ? alpha : rv);
+                    for (int kk = lane; kk < j0; kk += 32) a.R[(size_t)j * pitch + kk] = 0.0;
+                    if (r == 0 && q < nn0) a.R[(size_t)j * pitch + j0 + q] = q < i ? 0.0 : (q == i ? alpha : rv);
                 }
             }
             if (lane == 0) pan_stop = stop;
@@ -688,7 +697,7 @@ __global__ void __launch_bounds__(QR_THREADS, 1) qr_kernel(QrArgs a)
                     const double cf = tau * fma(-alpha, pi, gi);
                     const double rv = fma(-v0, cf, pi);
                     if (in && !isg) cfs[i * k + kk] = cf;
-                    if (in && (isg || !pairs) && c == 0) a.R[(size_t)(j0 + i) * k + kk] = rv;
+                    if (in && (isg || !pairs) && c == 0) a.R[(size_t)(j0 + i) * pitch + kk] = rv;
                     if (pairs) {
                         const double mul = isg ? rv : cf;
 #pragma unroll
@@ -747,10 +756,22 @@ __global__ void __launch_bounds__(QR_THREADS, 1) qr_kernel(QrArgs a)
         if (rg == j) v = v0s[j];
         else if (rg > j) v = Ys[rl * ld + j];
         if (taus[j] == 0.0) v = 0.0;
+        if (FACT) {
+            // 2^-exponent(v_0), v_0 being the column's largest entry: the reflector is the same, and
+            // the trailing update's row grids see columns of one size
+            const int e = (__double2hiint(v0s[j]) >> 20) & 0x7FF;
+            v = e > 0 && e < 2046 ? v * __hiloint2double((2046 - e) << 20, 0) : v;
+            a.V[(size_t)rg * pitch + j] = v;
+        }
         Ys[rl * ld + j] = v;
-        if (rg < k) a.V[(size_t)rg * k + j] = v;
+        if (!FACT && rg < k) a.V[(size_t)rg * k + j] = v;
     }
-    if (c == 0) {
+    if (FACT && c == 0)
+        for (int j = tid; j < k; j += blockDim.x) {
+            a.taus[j] = taus[j];
+            a.sgn[j] = alps[j] < 0.0 ? -1.0 : 1.0;
+        }
+    if (!FACT && c == 0) {
         __syncthreads();
         for (int t = tid; t < k * k; t += blockDim.x) {
             int rr = t / k;
@@ -796,10 +817,12 @@ __global__ void __launch_bounds__(QR_THREADS, 1) qr_kernel(QrArgs a)
     }
     if (!grid_barrier(a.bar, a.G, ++ep, a.err, a.bar_extra, a.spin_limit)) return;
     for (int cb = c; cb < (k + QR_WC - 1) / QR_WC; cb += a.G) {   // a small grid solves several blocks
-        if (wy_packed(k)) wy_solve_cta<true>(k, cb, a.S, a.V, taus, a.W, Gs);
-        else wy_solve_cta<false>(k, cb, a.S, a.V, taus, a.W, Gs);
+        const double *V = FACT ? nullptr : a.V;
+        if (wy_packed(k)) wy_solve_cta<true>(k, cb, a.S, V, taus, a.W, Gs);
+        else wy_solve_cta<false>(k, cb, a.S, V, taus, a.W, Gs);
         __syncthreads();
     }
+    if (FACT) return;
     if (!grid_barrier(a.bar, a.G, ++ep, a.err, a.bar_extra, a.spin_limit)) return;
     // Q rows of this CTA: (E - V W) with column c negated where alpha_c < 0; a thread owns one
     // column and the same number of rows, known at compile time, in every pass: a predicated-off
@@ -887,15 +910,16 @@ size_t qr_sk_doubles(int n, int k)
 
 size_t qr_wy_doubles(int n, int k) { return (size_t)k * k + 3 * (size_t)k * k + 2 * (size_t)k; }
 
+// pitch > 0: one panel of the blocked factorisation (Q unused; V, R in the wider matrices)
 static cudaError_t qr_factor_launch(int n, int k, int rows_per, const double *Y, double *Q, double *R, QrScratch s,
-                                    cudaStream_t st)
+                                    cudaStream_t st, int pitch = 0, double *taus = nullptr, double *sgn = nullptr)
 {
     const int G = (n + rows_per - 1) / rows_per;
-    const bool slab = s.force_slab || qr_smem_bytes(rows_per, k, false) > QR_SMEM_MAX;
+    const bool slab = pitch == 0 && (s.force_slab || qr_smem_bytes(rows_per, k, false) > QR_SMEM_MAX);
     if (slab && (!s.yslab || s.yslab_elems < (size_t)G * rows_per * (k | 1))) return cudaErrorInvalidValue;
     const size_t smem = qr_smem_bytes(rows_per, k, slab);
     if (smem > QR_SMEM_MAX) return cudaErrorInvalidValue;
-    void (*kern)(QrArgs) = slab ? qr_kernel<true> : qr_kernel<false>;
+    void (*kern)(QrArgs) = pitch > 0 ? qr_kernel<false, true> : slab ? qr_kernel<true> : qr_kernel<false>;
     int per_sm = 0;
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, QR_THREADS, smem);
     if (per_sm * device_sm_count() < G) return cudaErrorCooperativeLaunchTooLarge;
@@ -907,7 +931,8 @@ static cudaError_t qr_factor_launch(int n, int k, int rows_per, const double *Y,
     if (e != cudaSuccess) return e;
     if (s.gpart && (!s.spart || G > s.gmax)) return cudaErrorInvalidValue;
     QrArgs a{n, k, G, rows_per, Y, R, Q, s.V, s.S, s.W, s.sbuf, s.rowbuf, s.bar, s.err, s.bar_extra,
-             s.spin_limit > 0 ? s.spin_limit : QR_SPIN_LIMIT, s.gpart, s.spart, slab ? s.yslab : nullptr};
+             s.spin_limit > 0 ? s.spin_limit : QR_SPIN_LIMIT, s.gpart, s.spart, slab ? s.yslab : nullptr, pitch, taus,
+             sgn};
     void *args[] = {&a};
     CTM_COUNT_LAUNCH(1);
     return cudaLaunchCooperativeKernel((void *)kern, dim3(G), dim3(QR_THREADS), args, smem, st);
@@ -993,10 +1018,164 @@ static int qr_pick_rows(int n, int k, const double *Y, double *Q, double *R, QrS
     return best;
 }
 
+// ---------------------------------------------------------------- blocked, for many columns
+// At k = 480 the one-launch factorisation is bound by the FP64 pipe: 4 n k^2 multiply-adds with Q
+// formed, 13 ms at n = 12000.  Here panels of QR_NB columns are factored by that kernel (FACT),
+// and what is a contraction runs on the tensor cores as FP64 slices (gemm_split.cu, T = 8, whose
+// error is below the FP64 sums'): the trailing update A -= V (A^T V T)^T of each panel, and, once
+// all reflectors are known, S = V^T V and Q = E - V W with W = U^{-1} V_top^T as above.  The
+// reflectors are scaled to one size (a power of two each) because the update's grids are per row
+// of V.  A = Y is copied to Q's buffer and factored there, rows above the panel becoming R's.
+constexpr int QR_NB = 64;   // an engine tile's K and N (48: 12000 x 480 4.52 ms against 4.31)
+
+struct QrBlockedWork {
+    double *V, *Z, *X, *taus, *sgn;
+    SplitWork sw;
+    size_t bytes;
+};
+static QrBlockedWork qr_blocked_work(int n, int k, void *base_)
+{
+    QrBlockedWork w{};
+    char *base = (char *)base_;
+    size_t off = 0;
+    auto take = [&](size_t bytes) {
+        char *p = base ? base + off : nullptr;
+        off += (bytes + 255) & ~(size_t)255;
+        return p;
+    };
+    w.V = (double *)take(sizeof(double) * (size_t)n * k);
+    w.Z = (double *)take(sizeof(double) * (size_t)k * QR_NB);
+    w.X = (double *)take(sizeof(double) * (size_t)k * QR_NB);
+    w.taus = (double *)take(sizeof(double) * k);
+    w.sgn = (double *)take(sizeof(double) * k);
+    // A^T V and V X^T of the first panel, V^T V, V W: the largest of each operand
+    const int shapes[4][3] = {{k, QR_NB, n}, {n, k, QR_NB}, {k, k, n}, {n, k, k}};
+    for (auto &m : shapes) {
+        const SplitPlan p = split_plan_caps(m[0], m[1], m[2], SPLIT_F64_T);
+        if (p.a_pack_bytes > w.sw.a_pack_cap) w.sw.a_pack_cap = p.a_pack_bytes;
+        if (p.b_pack_bytes > w.sw.b_pack_cap) w.sw.b_pack_cap = p.b_pack_bytes;
+        if (p.partial_bytes > w.sw.partial_cap) w.sw.partial_cap = p.partial_bytes;
+    }
+    w.sw.e_cap = n;
+    w.sw.Apk = (unsigned char *)take(w.sw.a_pack_cap);
+    w.sw.Bpk = (unsigned char *)take(w.sw.b_pack_cap);
+    w.sw.partial = take(w.sw.partial_cap + 8);
+    w.sw.eA = (int *)take(sizeof(int) * (size_t)n);
+    w.sw.eB = (int *)take(sizeof(int) * (size_t)n);
+    w.bytes = off;
+    return w;
+}
+
+// Columns 4b .. 4b + 3 of W = -U^{-1} V_top^T diag(sgn), so that Q = E diag(sgn) + V W has the gauge
+__global__ void __launch_bounds__(QR_THREADS) qr_blocked_w_kernel(int k, const double *S, const double *V,
+                                                                  const double *taus, const double *sgn, double *W)
+{
+    extern __shared__ double sm[];
+    if (wy_packed(k)) wy_solve_cta<true>(k, blockIdx.x, S, V, taus, W, sm);
+    else wy_solve_cta<false>(k, blockIdx.x, S, V, taus, W, sm);
+    __syncthreads();
+    for (int t = threadIdx.x; t < k * QR_WC; t += blockDim.x) {
+        const int j = blockIdx.x * QR_WC + t % QR_WC;
+        if (j < k) W[(size_t)(t / QR_WC) * k + j] *= -sgn[j];
+    }
+}
+// R from the panels' blocks (in R) and the updated rows above them (in A), with the gauge
+__global__ void qr_blocked_r_kernel(int k, const double *A, const double *sgn, double *R)
+{
+    const int i = blockIdx.x;
+    for (int j = threadIdx.x; j < k; j += blockDim.x) {
+        const size_t o = (size_t)i * k + j;
+        R[o] = j < i ? 0.0 : sgn[i] * (j / QR_NB == i / QR_NB ? R[o] : A[o]);
+    }
+}
+__global__ void qr_blocked_diag_kernel(int k, const double *sgn, double *Q)
+{
+    const int j = blockIdx.x * blockDim.x + threadIdx.x;
+    if (j < k) Q[(size_t)j * k + j] += sgn[j];
+}
+
+// Rows per CTA of a panel: one CTA per SM, two SMs left free as for the slab
+static int qr_panel_rows(int n, int rows_min)
+{
+    const int sms = device_sm_count(), g = sms > 4 ? sms - 2 : sms, base = (n + g - 1) / g;
+    return base > rows_min ? base : rows_min;
+}
+
+// Where the blocked form pays (us, one launch : blocked): below this line 1728 x 192 668 : 849 and
+// 3072 x 192 956 : 930; above it 4800 x 192 1156 : 1006, 4096 x 256 1756 : 1330, 8000 x 320
+// 4346 : 2033, 4608 x 512 6589 : 2885, 12000 x 480 12928 : 4306.  |Y - QR| / |Y| and |Q^T Q - 1| at
+// those sizes 4e-16 to 6e-16 and 1.4e-14 to 3.5e-14, one launch 2e-16 to 9e-16 and 2.8e-14 to 5.5e-14.
+constexpr int QR_BLOCKED_MIN = 192;
+constexpr double QR_BLOCKED_NK2 = 1.2e8;
+static bool qr_blocked_ok(int n, int k, const QrScratch &s)
+{
+    if (k < QR_BLOCKED_MIN || (double)n * k * k < QR_BLOCKED_NK2 || !s.blocked || s.force_slab) return false;
+    const int rows = qr_panel_rows(n, s.rows_min);
+    if (qr_smem_bytes(rows, QR_NB, false) > QR_SMEM_MAX) return false;
+    if (s.gpart && (n + rows - 1) / rows > s.gmax) return false;
+    return qr_blocked_work(n, k, nullptr).bytes <= s.blocked_bytes;
+}
+
+static cudaError_t qr_blocked(int n, int k, const double *Y, double *Q, double *R, QrScratch s, cudaStream_t st)
+{
+    QrBlockedWork w = qr_blocked_work(n, k, s.blocked);
+    w.sw.err = s.err;
+    double *A = Q;
+    cudaError_t e = cudaMemcpyAsync(A, Y, sizeof(double) * (size_t)n * k, cudaMemcpyDeviceToDevice, st);
+    if (e == cudaSuccess) e = cudaMemsetAsync(w.V, 0, sizeof(double) * (size_t)n * k, st);
+    for (int j0 = 0; j0 < k && e == cudaSuccess; j0 += QR_NB) {
+        const int nb = k - j0 < QR_NB ? k - j0 : QR_NB, m = n - j0, j1 = j0 + nb, rem = k - j1;
+        double *Vp = w.V + (size_t)j0 * k + j0;
+        QrScratch sp = s;
+        sp.V = Vp;
+        e = qr_factor_launch(m, nb, qr_panel_rows(m, s.rows_min), A + (size_t)j0 * k + j0, nullptr,
+                             R + (size_t)j0 * k + j0, sp, st, k, w.taus + j0, w.sgn + j0);
+        if (e != cudaSuccess || rem == 0) continue;
+        double *At = A + (size_t)j0 * k + j1;
+        // Z = A^T V, X = -Z T, A += V X^T
+        e = gemm_split(GemmF64{rem, nb, m, At, idx_lin(1), idx_lin(k), Vp, idx_lin(k), idx_lin(1), w.Z, idx_lin(QR_NB),
+                               idx_lin(1), 1.0, 0.0},
+                       SPLIT_F64_T, w.sw, st, nullptr);
+        if (e == cudaSuccess)
+            e = gemm_f64(GemmF64{rem, nb, nb, w.Z, idx_lin(QR_NB), idx_lin(1), s.W, idx_lin(nb), idx_lin(1), w.X,
+                                 idx_lin(QR_NB), idx_lin(1), -1.0, 0.0},
+                         1, nullptr, 0, st);
+        if (e == cudaSuccess)
+            e = gemm_split(GemmF64{m, rem, nb, Vp, idx_lin(k), idx_lin(1), w.X, idx_lin(1), idx_lin(QR_NB), At,
+                                   idx_lin(k), idx_lin(1), 1.0, 1.0},
+                           SPLIT_F64_T, w.sw, st, nullptr);
+    }
+    if (e != cudaSuccess) return e;
+    CTM_COUNT_LAUNCH(3);
+    qr_blocked_r_kernel<<<k, 128, 0, st>>>(k, A, w.sgn, R);
+    // S in two parts: the engine's error is in units of the columns' largest entries, which are the
+    // v_0 of order 1 in the first k rows and ~1 / sqrt(n) below (in one part: |Q^T Q - 1| 1.0e-13
+    // at n = 12000, k = 480)
+    const double *Vb = w.V + (size_t)k * k;
+    if (n > k)
+        e = gemm_split(GemmF64{k, k, n - k, Vb, idx_lin(1), idx_lin(k), Vb, idx_lin(k), idx_lin(1), s.S, idx_lin(k),
+                               idx_lin(1), 1.0, 0.0},
+                       SPLIT_F64_T, w.sw, st, nullptr);
+    if (e == cudaSuccess)
+        e = gemm_split(GemmF64{k, k, k, w.V, idx_lin(1), idx_lin(k), w.V, idx_lin(k), idx_lin(1), s.S, idx_lin(k),
+                               idx_lin(1), 1.0, n > k ? 1.0 : 0.0},
+                       SPLIT_F64_T, w.sw, st, nullptr);
+    if (e != cudaSuccess) return e;
+    qr_blocked_w_kernel<<<(k + QR_WC - 1) / QR_WC, QR_THREADS, qr_wy_smem_bytes(k), st>>>(k, s.S, w.V, w.taus, w.sgn,
+                                                                                          s.W);
+    e = gemm_split(GemmF64{n, k, k, w.V, idx_lin(k), idx_lin(1), s.W, idx_lin(k), idx_lin(1), Q, idx_lin(k), idx_lin(1),
+                           1.0, 0.0},
+                   SPLIT_F64_T, w.sw, st, nullptr);
+    if (e != cudaSuccess) return e;
+    qr_blocked_diag_kernel<<<(k + 127) / 128, 128, 0, st>>>(k, w.sgn, Q);
+    return cudaGetLastError();
+}
+
 cudaError_t qr_householder(int n, int k, const double *Y, double *Q, double *R, QrScratch s, cudaStream_t st)
 {
     int G, rp;
     if (!qr_supported(n, k) || !s.V) return cudaErrorInvalidValue;
+    if (qr_blocked_ok(n, k, s)) return qr_blocked(n, k, Y, Q, R, s, st);
     if (!qr_layout(n, k, s.rows_min > 0 ? s.rows_min : 1, &G, &rp, nullptr, s.force_slab) &&
         !qr_layout(n, k, 1, &G, &rp, nullptr, s.force_slab))
         return cudaErrorInvalidValue;
@@ -1008,5 +1187,10 @@ cudaError_t qr_prepare()
 {
     cudaError_t e = cudaFuncSetAttribute(qr_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, QR_SMEM_MAX);
     if (e != cudaSuccess) return e;
-    return cudaFuncSetAttribute(qr_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, QR_SMEM_MAX);
+    e = cudaFuncSetAttribute(qr_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, QR_SMEM_MAX);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(qr_kernel<false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, QR_SMEM_MAX);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(qr_blocked_w_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, QR_SMEM_MAX);
+    return e;
 }
