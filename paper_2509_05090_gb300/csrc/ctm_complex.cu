@@ -1235,7 +1235,10 @@ int zprojector(ctm_complex_ctx *c)
             c->Y, c->PY, 0, idx_lin(chi), idx_lin(1)};
     if ((rc = zgemm(c, z)) != CTM_OK) return rc;
     ZLAUNCH(zc_embed_kernel, zgrid(n * chi), 256, n, chi, c->Y, c->PY, c->Yemb);
-    ZK(qr_householder((int)(2 * n), 2 * chi, c->Yemb, c->Qemb, c->Remb, zqr_scratch(c), c->stream));
+    QrScratch qs = zqr_scratch(c);
+    qs.blocked = c->H;   // written by the edge update only, after the QR
+    qs.blocked_bytes = sizeof(double) * 2 * c->PM;
+    ZK(qr_householder((int)(2 * n), 2 * chi, c->Yemb, c->Qemb, c->Remb, qs, c->stream));
     ZLAUNCH(zc_extract_kernel, zgrid(n * chi), 256, n, chi, c->Qemb, c->Qn, c->PQ, 5);
     ZLAUNCH(zc_extract_kernel, zgrid((long long)chi * chi), 256, (long long)chi, chi, c->Remb, c->R, c->PC, 2);
     return CTM_OK;

@@ -42,8 +42,9 @@
 // from that cost; partial sums are combined by halving; nothing FP64 sits under a predicate.
 // n x k: 512 x 32 119 -> 66 us, 2592 x 72 307 -> 214 (panels 23k -> 13k cycles each, update and
 // Gram passes 17k -> 8k), 8192 x 128 1027 -> 833, 5184 x 144 987 -> 802, 12000 x 240
-// 2350 -> 1960.  Many columns (4 n k^2 of them with Q formed) go to the blocked form near the end
-// of this file, which leaves that pipe the 64-column panels only: 12000 x 480 12.9 -> 4.3 ms.
+// 2350 -> 1960.  From n k^2 = 5e7 on, S, W and Q, and
+// with many columns the trailing update too, leave that pipe for the tensor cores (the blocked
+// form near the end of this file): 8192 x 128 845 -> 643 us, 12000 x 480 12.9 -> 4.3 ms.
 //
 // The grid barrier is one monotonic counter in global memory; its spin is
 // bounded (about a second) and on expiry sets an error flag that the host
@@ -771,6 +772,7 @@ __global__ void __launch_bounds__(QR_THREADS, 1) qr_kernel(QrArgs a)
             a.taus[j] = taus[j];
             a.sgn[j] = alps[j] < 0.0 ? -1.0 : 1.0;
         }
+    if (FACT && !a.S) return;   // a lone panel: its S and W are the whole matrix's
     if (!FACT && c == 0) {
         __syncthreads();
         for (int t = tid; t < k * k; t += blockDim.x) {
@@ -927,7 +929,7 @@ static cudaError_t qr_factor_launch(int n, int k, int rows_per, const double *Y,
     if (e != cudaSuccess) return e;
     e = cudaMemsetAsync(s.bar, 0, sizeof(unsigned) * 2, st);
     if (e != cudaSuccess) return e;
-    e = cudaMemsetAsync(s.S, 0, sizeof(double) * (size_t)k * k, st);
+    if (s.S) e = cudaMemsetAsync(s.S, 0, sizeof(double) * (size_t)k * k, st);
     if (e != cudaSuccess) return e;
     if (s.gpart && (!s.spart || G > s.gmax)) return cudaErrorInvalidValue;
     QrArgs a{n, k, G, rows_per, Y, R, Q, s.V, s.S, s.W, s.sbuf, s.rowbuf, s.bar, s.err, s.bar_extra,
@@ -1020,12 +1022,12 @@ static int qr_pick_rows(int n, int k, const double *Y, double *Q, double *R, QrS
 
 // ---------------------------------------------------------------- blocked, for many columns
 // At k = 480 the one-launch factorisation is bound by the FP64 pipe: 4 n k^2 multiply-adds with Q
-// formed, 13 ms at n = 12000.  Here panels of QR_NB columns are factored by that kernel (FACT),
+// formed, 13 ms at n = 12000.  Here panels of QR_NB columns (or all k in one) are factored by that kernel (FACT),
 // and what is a contraction runs on the tensor cores as FP64 slices (gemm_split.cu, T = 8, whose
 // error is below the FP64 sums'): the trailing update A -= V (A^T V T)^T of each panel, and, once
 // all reflectors are known, S = V^T V and Q = E - V W with W = U^{-1} V_top^T as above.  The
 // reflectors are scaled to one size (a power of two each) because the update's grids are per row
-// of V.  A = Y is copied to Q's buffer and factored there, rows above the panel becoming R's.
+// of V.  With several panels A = Y is copied to Q's buffer and factored there, rows above the panel becoming R's.
 constexpr int QR_NB = 64;   // an engine tile's K and N (48: 12000 x 480 4.52 ms against 4.31)
 
 struct QrBlockedWork {
@@ -1033,7 +1035,7 @@ struct QrBlockedWork {
     SplitWork sw;
     size_t bytes;
 };
-static QrBlockedWork qr_blocked_work(int n, int k, void *base_)
+static QrBlockedWork qr_blocked_work(int n, int k, int width, void *base_)
 {
     QrBlockedWork w{};
     char *base = (char *)base_;
@@ -1044,12 +1046,12 @@ static QrBlockedWork qr_blocked_work(int n, int k, void *base_)
         return p;
     };
     w.V = (double *)take(sizeof(double) * (size_t)n * k);
-    w.Z = (double *)take(sizeof(double) * (size_t)k * QR_NB);
-    w.X = (double *)take(sizeof(double) * (size_t)k * QR_NB);
+    w.Z = (double *)take(sizeof(double) * (size_t)k * width);
+    w.X = (double *)take(sizeof(double) * (size_t)k * width);
     w.taus = (double *)take(sizeof(double) * k);
     w.sgn = (double *)take(sizeof(double) * k);
     // A^T V and V X^T of the first panel, V^T V, V W: the largest of each operand
-    const int shapes[4][3] = {{k, QR_NB, n}, {n, k, QR_NB}, {k, k, n}, {n, k, k}};
+    const int shapes[4][3] = {{k, width, n}, {n, k, width}, {k, k, n}, {n, k, k}};
     for (auto &m : shapes) {
         const SplitPlan p = split_plan_caps(m[0], m[1], m[2], SPLIT_F64_T);
         if (p.a_pack_bytes > w.sw.a_pack_cap) w.sw.a_pack_cap = p.a_pack_bytes;
@@ -1080,12 +1082,12 @@ __global__ void __launch_bounds__(QR_THREADS) qr_blocked_w_kernel(int k, const d
     }
 }
 // R from the panels' blocks (in R) and the updated rows above them (in A), with the gauge
-__global__ void qr_blocked_r_kernel(int k, const double *A, const double *sgn, double *R)
+__global__ void qr_blocked_r_kernel(int k, int width, const double *A, const double *sgn, double *R)
 {
     const int i = blockIdx.x;
     for (int j = threadIdx.x; j < k; j += blockDim.x) {
         const size_t o = (size_t)i * k + j;
-        R[o] = j < i ? 0.0 : sgn[i] * (j / QR_NB == i / QR_NB ? R[o] : A[o]);
+        R[o] = j < i ? 0.0 : sgn[i] * (j / width == i / width ? R[o] : A[o]);
     }
 }
 __global__ void qr_blocked_diag_kernel(int k, const double *sgn, double *Q)
@@ -1101,53 +1103,65 @@ static int qr_panel_rows(int n, int rows_min)
     return base > rows_min ? base : rows_min;
 }
 
-// Where the blocked form pays (us, one launch : blocked): below this line 1728 x 192 668 : 849 and
-// 3072 x 192 956 : 930; above it 4800 x 192 1156 : 1006, 4096 x 256 1756 : 1330, 8000 x 320
-// 4346 : 2033, 4608 x 512 6589 : 2885, 12000 x 480 12928 : 4306.  |Y - QR| / |Y| and |Q^T Q - 1| at
-// those sizes 4e-16 to 6e-16 and 1.4e-14 to 3.5e-14, one launch 2e-16 to 9e-16 and 2.8e-14 to 5.5e-14.
-constexpr int QR_BLOCKED_MIN = 192;
-constexpr double QR_BLOCKED_NK2 = 1.2e8;
-static bool qr_blocked_ok(int n, int k, const QrScratch &s)
+// Where each form pays, by n k^2 (us: the kernel alone : one panel : 64-column panels).  Below
+// 5e7 the kernel alone: 2592 x 72 225 : 318, 2048 x 128 434 : 462, 3000 x 120 449 : 447.  Then one
+// panel, for S and Q by the engine: 6144 x 96 498 : 455, 4608 x 128 600 : 549, 8192 x 128
+// 845 : 643, 1728 x 192 668 : 635 : 849, 4800 x 192 1153 : 870 : 1006, 6000 x 240 1969 : 1303 : 1348.
+// From 3.9e8 panels: 6400 x 256 1492 (one panel) : 1433, 5120 x 320 1933 : 1766, 8000 x 320
+// 4346 (kernel) : 2019, 4608 x 512 6589 : 2895, 12000 x 480 12928 : 4289.  |Y - QR| / |Y| there is
+// 2e-16 to 6e-16 and |Q^T Q - 1| 8e-15 to 3.5e-14, by the kernel alone 4e-16 to 9e-16 and
+// 1.4e-14 to 5.5e-14.
+constexpr int QR_ONE_PANEL_MIN = 96;
+constexpr double QR_ONE_PANEL_NK2 = 5e7, QR_PANELS_NK2 = 3.9e8;
+// Panel width of the blocked form (k: one panel), or 0 for the one-launch kernel
+static int qr_blocked_width(int n, int k, const QrScratch &s)
 {
-    if (k < QR_BLOCKED_MIN || (double)n * k * k < QR_BLOCKED_NK2 || !s.blocked || s.force_slab) return false;
+    if (!s.blocked || s.force_slab) return 0;
+    const double nk2 = (double)n * k * k;
+    if (k < QR_ONE_PANEL_MIN || nk2 < QR_ONE_PANEL_NK2) return 0;
+    const int width = nk2 >= QR_PANELS_NK2 ? QR_NB : k;
     const int rows = qr_panel_rows(n, s.rows_min);
-    if (qr_smem_bytes(rows, QR_NB, false) > QR_SMEM_MAX) return false;
-    if (s.gpart && (n + rows - 1) / rows > s.gmax) return false;
-    return qr_blocked_work(n, k, nullptr).bytes <= s.blocked_bytes;
+    if (qr_smem_bytes(rows, width, false) > QR_SMEM_MAX) return 0;
+    if (s.gpart && (n + rows - 1) / rows > s.gmax) return 0;
+    return qr_blocked_work(n, k, width, nullptr).bytes <= s.blocked_bytes ? width : 0;
 }
 
-static cudaError_t qr_blocked(int n, int k, const double *Y, double *Q, double *R, QrScratch s, cudaStream_t st)
+static cudaError_t qr_blocked(int n, int k, int width, const double *Y, double *Q, double *R, QrScratch s,
+                              cudaStream_t st)
 {
-    QrBlockedWork w = qr_blocked_work(n, k, s.blocked);
+    QrBlockedWork w = qr_blocked_work(n, k, width, s.blocked);
     w.sw.err = s.err;
+    const bool lone = width >= k;   // one panel, read from Y itself
     double *A = Q;
-    cudaError_t e = cudaMemcpyAsync(A, Y, sizeof(double) * (size_t)n * k, cudaMemcpyDeviceToDevice, st);
-    if (e == cudaSuccess) e = cudaMemsetAsync(w.V, 0, sizeof(double) * (size_t)n * k, st);
-    for (int j0 = 0; j0 < k && e == cudaSuccess; j0 += QR_NB) {
-        const int nb = k - j0 < QR_NB ? k - j0 : QR_NB, m = n - j0, j1 = j0 + nb, rem = k - j1;
+    cudaError_t e = cudaSuccess;
+    if (!lone) e = cudaMemcpyAsync(A, Y, sizeof(double) * (size_t)n * k, cudaMemcpyDeviceToDevice, st);
+    if (!lone && e == cudaSuccess) e = cudaMemsetAsync(w.V, 0, sizeof(double) * (size_t)n * k, st);
+    for (int j0 = 0; j0 < k && e == cudaSuccess; j0 += width) {
+        const int nb = k - j0 < width ? k - j0 : width, m = n - j0, j1 = j0 + nb, rem = k - j1;
         double *Vp = w.V + (size_t)j0 * k + j0;
         QrScratch sp = s;
         sp.V = Vp;
-        e = qr_factor_launch(m, nb, qr_panel_rows(m, s.rows_min), A + (size_t)j0 * k + j0, nullptr,
+        if (lone) sp.S = nullptr;
+        e = qr_factor_launch(m, nb, qr_panel_rows(m, s.rows_min), lone ? Y : A + (size_t)j0 * k + j0, nullptr,
                              R + (size_t)j0 * k + j0, sp, st, k, w.taus + j0, w.sgn + j0);
         if (e != cudaSuccess || rem == 0) continue;
         double *At = A + (size_t)j0 * k + j1;
         // Z = A^T V, X = -Z T, A += V X^T
-        e = gemm_split(GemmF64{rem, nb, m, At, idx_lin(1), idx_lin(k), Vp, idx_lin(k), idx_lin(1), w.Z, idx_lin(QR_NB),
+        e = gemm_split(GemmF64{rem, nb, m, At, idx_lin(1), idx_lin(k), Vp, idx_lin(k), idx_lin(1), w.Z, idx_lin(width),
                                idx_lin(1), 1.0, 0.0},
                        SPLIT_F64_T, w.sw, st, nullptr);
         if (e == cudaSuccess)
-            e = gemm_f64(GemmF64{rem, nb, nb, w.Z, idx_lin(QR_NB), idx_lin(1), s.W, idx_lin(nb), idx_lin(1), w.X,
-                                 idx_lin(QR_NB), idx_lin(1), -1.0, 0.0},
+            e = gemm_f64(GemmF64{rem, nb, nb, w.Z, idx_lin(width), idx_lin(1), s.W, idx_lin(nb), idx_lin(1), w.X,
+                                 idx_lin(width), idx_lin(1), -1.0, 0.0},
                          1, nullptr, 0, st);
         if (e == cudaSuccess)
-            e = gemm_split(GemmF64{m, rem, nb, Vp, idx_lin(k), idx_lin(1), w.X, idx_lin(1), idx_lin(QR_NB), At,
+            e = gemm_split(GemmF64{m, rem, nb, Vp, idx_lin(k), idx_lin(1), w.X, idx_lin(1), idx_lin(width), At,
                                    idx_lin(k), idx_lin(1), 1.0, 1.0},
                            SPLIT_F64_T, w.sw, st, nullptr);
     }
     if (e != cudaSuccess) return e;
     CTM_COUNT_LAUNCH(3);
-    qr_blocked_r_kernel<<<k, 128, 0, st>>>(k, A, w.sgn, R);
+    qr_blocked_r_kernel<<<k, 128, 0, st>>>(k, width, A, w.sgn, R);
     // S in two parts: the engine's error is in units of the columns' largest entries, which are the
     // v_0 of order 1 in the first k rows and ~1 / sqrt(n) below (in one part: |Q^T Q - 1| 1.0e-13
     // at n = 12000, k = 480)
@@ -1175,7 +1189,8 @@ cudaError_t qr_householder(int n, int k, const double *Y, double *Q, double *R, 
 {
     int G, rp;
     if (!qr_supported(n, k) || !s.V) return cudaErrorInvalidValue;
-    if (qr_blocked_ok(n, k, s)) return qr_blocked(n, k, Y, Q, R, s, st);
+    const int width = qr_blocked_width(n, k, s);
+    if (width) return qr_blocked(n, k, width, Y, Q, R, s, st);
     if (!qr_layout(n, k, s.rows_min > 0 ? s.rows_min : 1, &G, &rp, nullptr, s.force_slab) &&
         !qr_layout(n, k, 1, &G, &rp, nullptr, s.force_slab))
         return cudaErrorInvalidValue;

@@ -1,5 +1,5 @@
-"""The blocked Householder QR of many columns (csrc/qr.cu: 64-column panels, the rest as FP64 slices on
-the tensor cores): Y = Q R of a step at panel edges, and with zero and dependent columns."""
+"""The blocked Householder QR (csrc/qr.cu: one panel or 64-column panels, the rest as FP64 slices on the
+tensor cores): Y = Q R of a step at panel edges, and with zero and dependent columns."""
 import numpy as np
 import pytest
 import torch
@@ -21,7 +21,7 @@ def _check(g, chi):
 
 
 @pytest.mark.parametrize("deterministic", [False, True])
-@pytest.mark.parametrize("D,chi", [(4, 200), (5, 193), (3, 256), (3, 257), (5, 320), (3, 512)])
+@pytest.mark.parametrize("D,chi", [(8, 97), (4, 200), (5, 193), (3, 256), (3, 257), (4, 321), (5, 320), (3, 512)])
 def test_panels(ctm_lib, D, chi, deterministic):
     from paper_2509_05090_gb300 import binding
     g = binding.CTM(I.random_site_tensor(2, D, 50 + chi), chi, precision="split_bf16", n_split=3,
@@ -33,10 +33,10 @@ def test_panels(ctm_lib, D, chi, deterministic):
     g.close()
 
 
-def test_zero_and_dependent_columns(ctm_lib):
+@pytest.mark.parametrize("D,chi", [(3, 260), (5, 320)])
+def test_zero_and_dependent_columns(ctm_lib, D, chi):
     from paper_2509_05090_gb300 import binding
-    chi = 260
-    g = binding.CTM(I.random_site_tensor(2, 3, 77), chi, precision="split_bf16", n_split=3)
+    g = binding.CTM(I.random_site_tensor(2, D, 77), chi, precision="split_bf16", n_split=3)
     g.ctm_step(2)
     C, T, Q = g.ctm_get_env()
     for c in (0, 63, 64, 130, chi - 1):
@@ -47,4 +47,16 @@ def test_zero_and_dependent_columns(ctm_lib):
     g.ctm_step(1)
     _check(g, chi)
     assert np.isfinite(g.ctm_get_intermediate("R").cpu().numpy()).all()
+    g.close()
+
+
+def test_complex_embedding(ctm_lib):
+    """The complex step's QR of the real 2n x 2chi embedding: Q stays an isometry."""
+    from paper_2509_05090_gb300 import binding
+    chi = 72
+    g = binding.CTMComplex(I.random_complex_site_tensor(2, 6, 3), chi, precision="split_bf16", n_split=5)
+    g.ctm_complex_step(3)
+    Q = g.ctm_complex_get_env()[2].reshape(-1, chi)
+    eye = torch.eye(chi, dtype=Q.dtype, device=Q.device)
+    assert float((Q.conj().T @ Q - eye).abs().pow(2).sum().sqrt()) <= 4 * (2 * chi) ** 1.5 * 2.0 ** -53
     g.close()
