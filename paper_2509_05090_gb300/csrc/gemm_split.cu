@@ -342,13 +342,16 @@ __global__ void __launch_bounds__(256) split_rowpack_kernel(int R, int K, int ro
 // Packing of a contiguous-K operand read once, held in registers: a group of
 // WPR warps owns one row; at step j warp w of the group loads the 64-wide K
 // tile kt = j WPR + w as one double2 per lane (512 contiguous bytes per warp
-// instruction), the group reduces the exponent word through shared memory, and
+// instruction; two 8-byte loads where PAIR does not hold: an odd K or rows off 16 bytes),
+// the group reduces the exponent word through shared memory, and
 // each lane writes its two digits of every slice as one 32-bit word, so one
 // store instruction fills the tile's whole 128-byte swizzled row of that
-// slice.  Needs K even, 16-byte aligned rows and NV WPR >= kTiles; rows from R
+// slice.  Needs NV WPR >= kTiles; rows from R
 // up to rowsTotal and columns from K up to the tile edge get zero digits.
-template <int NV, int T>
-__global__ void __launch_bounds__(512, 1) split_rowpack_reg_kernel(int R, int K, int rowsT, int rowsTotal, int kTiles,
+// Bound by memory; a warp with more of a row has more loads in flight and fewer partners to
+// wait for, see the rule in split_prepass_t.
+template <int NV, int T, bool PAIR>
+__global__ void __launch_bounds__(512, NV > 8 ? 1 : 2) split_rowpack_reg_kernel(int R, int K, int rowsT, int rowsTotal, int kTiles,
                                                                 int WPR, const double *X, Idx2 rmap, int *e,
                                                                 unsigned char *out)
 {
@@ -364,7 +367,12 @@ __global__ void __launch_bounds__(512, 1) split_rowpack_reg_kernel(int R, int K,
     for (int j = 0; j < NV; ++j) {
         const int k = ((j * WPR + w) << 6) + 2 * lane;
         v[j] = make_double2(0.0, 0.0);
-        if (live && k < K) v[j] = *reinterpret_cast<const double2 *>(x + k);
+        if (PAIR) {
+            if (live && k < K) v[j] = *reinterpret_cast<const double2 *>(x + k);
+        } else {
+            if (live && k < K) v[j].x = x[k];
+            if (live && k + 1 < K) v[j].y = x[k + 1];
+        }
     }
 #pragma unroll
     for (int j = 0; j < NV; ++j) m = max(m, max(abs_hi_word(v[j].x), abs_hi_word(v[j].y)));
@@ -1352,18 +1360,33 @@ static cudaError_t split_prepass_t(int R, int K, const double *X, Idx2 rmap, Idx
         const int rows = rowTiles * rowsT;
         CTM_COUNT_LAUNCH(1);
         const bool pairs = ((uintptr_t)X & 15) == 0 && (K & 1) == 0 && (rmap.s1 & 1) == 0 && (rmap.s2 & 1) == 0;
-        if (pairs && kTiles <= 128) {
-            int nv = 1;
-            while (nv < 8 && (kTiles + nv - 1) / nv > 8) nv *= 2;
+        if (kTiles <= 256) {
+            // Tiles per warp: up to 8 (16 where a row is longer than 16 warps of 8), halved while
+            // that leaves fewer than 16 warps per SM.  us by tiles per warp, T = 5: 5184 x 1296
+            // 36.6 (2) 30.6 (4) 25.5 (8); 12000 x 480 38.2 (1) 28.1 (2) 24.1 (4) 21.9 (8); 512 x 512
+            // the same for all.  One row per block from two warps on (5184 x 1296 25.5 against
+            // 28.3 with two), four below (5184 x 36 8.2 with one, 6.3).
+            const int cap = 16 * device_sm_count();
+            int nv = kTiles > 128 ? 16 : 8;
+            while (nv > 1 && nv <= 8 &&
+                   (nv / 2 >= kTiles || (long long)rows * ((kTiles + nv - 1) / nv) < cap) &&
+                   (kTiles + nv / 2 - 1) / (nv / 2) <= 16)
+                nv /= 2;
             const int wpr = (kTiles + nv - 1) / nv;        // <= 16 warps per row
-            const int rpb = wpr >= 8 ? 1 : 8 / wpr;         // rows per block
+            const int rpb = wpr >= 2 ? 1 : 4;               // rows per block
             const int blocks = (rows + rpb - 1) / rpb, threads = 32 * wpr * rpb;
-#define CTM_ROWPACK(NVV)                                                                                              \
-    split_rowpack_reg_kernel<NVV, T><<<blocks, threads, 0, st>>>(R, K, rowsT, rows, kTiles, wpr, X, rmap, e, pk)
-            if (nv == 1) CTM_ROWPACK(1);
-            else if (nv == 2) CTM_ROWPACK(2);
-            else if (nv == 4) CTM_ROWPACK(4);
-            else CTM_ROWPACK(8);
+#define CTM_ROWPACK(NVV)                                                                                               \
+    if (nv == NVV && pairs)                                                                                            \
+        split_rowpack_reg_kernel<NVV, T, true><<<blocks, threads, 0, st>>>(R, K, rowsT, rows, kTiles, wpr, X, rmap, e, \
+                                                                           pk);                                        \
+    if (nv == NVV && !pairs)                                                                                           \
+        split_rowpack_reg_kernel<NVV, T, false><<<blocks, threads, 0, st>>>(R, K, rowsT, rows, kTiles, wpr, X, rmap,   \
+                                                                            e, pk);
+            CTM_ROWPACK(1)
+            CTM_ROWPACK(2)
+            CTM_ROWPACK(4)
+            CTM_ROWPACK(8)
+            CTM_ROWPACK(16)
 #undef CTM_ROWPACK
             return cudaGetLastError();
         }
