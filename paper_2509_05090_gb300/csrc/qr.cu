@@ -912,6 +912,16 @@ size_t qr_sk_doubles(int n, int k)
 
 size_t qr_wy_doubles(int n, int k) { return (size_t)k * k + 3 * (size_t)k * k + 2 * (size_t)k; }
 
+// The accumulators and the barrier count before a factorisation: one launch for all three (three
+// memset nodes and the gaps between them took 3 to 6 us more of a step)
+__global__ void qr_zero_kernel(int nsbuf, double *sbuf, int ns, double *S, unsigned *bar)
+{
+    const int t0 = blockIdx.x * blockDim.x + threadIdx.x, nt = gridDim.x * blockDim.x;
+    for (int t = t0; t < nsbuf; t += nt) sbuf[t] = 0.0;
+    for (int t = t0; t < ns; t += nt) S[t] = 0.0;
+    if (t0 < 2) bar[t0] = 0;
+}
+
 // pitch > 0: one panel of the blocked factorisation (Q unused; V, R in the wider matrices)
 static cudaError_t qr_factor_launch(int n, int k, int rows_per, const double *Y, double *Q, double *R, QrScratch s,
                                     cudaStream_t st, int pitch = 0, double *taus = nullptr, double *sgn = nullptr)
@@ -925,13 +935,13 @@ static cudaError_t qr_factor_launch(int n, int k, int rows_per, const double *Y,
     int per_sm = 0;
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, QR_THREADS, smem);
     if (per_sm * device_sm_count() < G) return cudaErrorCooperativeLaunchTooLarge;
-    cudaError_t e = cudaMemsetAsync(s.sbuf, 0, sizeof(double) * 3 * QB * k, st);
-    if (e != cudaSuccess) return e;
-    e = cudaMemsetAsync(s.bar, 0, sizeof(unsigned) * 2, st);
-    if (e != cudaSuccess) return e;
-    if (s.S) e = cudaMemsetAsync(s.S, 0, sizeof(double) * (size_t)k * k, st);
-    if (e != cudaSuccess) return e;
     if (s.gpart && (!s.spart || G > s.gmax)) return cudaErrorInvalidValue;
+    const int zb = (k * k + 1023) / 1024;
+    CTM_COUNT_LAUNCH(1);
+    qr_zero_kernel<<<zb < device_sm_count() ? zb : device_sm_count(), 256, 0, st>>>(3 * QB * k, s.sbuf, s.S ? k * k : 0,
+                                                                                 s.S, s.bar);
+    cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
     QrArgs a{n, k, G, rows_per, Y, R, Q, s.V, s.S, s.W, s.sbuf, s.rowbuf, s.bar, s.err, s.bar_extra,
              s.spin_limit > 0 ? s.spin_limit : QR_SPIN_LIMIT, s.gpart, s.spart, slab ? s.yslab : nullptr, pitch, taus,
              sgn};
