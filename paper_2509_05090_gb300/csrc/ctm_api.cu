@@ -235,15 +235,16 @@ size_t layout(ctm_ctx *c, char *base)
         c->sw.eA = (int *)take(sizeof(int) * (size_t)ecap);
         c->sw.eB = (int *)take(sizeof(int) * (size_t)ecap);
         c->sw.e_cap = (int)ecap;
-        c->sw.partial = (void *)take(pp + 8);
+        c->sw.partial = (void *)take(2 * align_up(pp));   // and the corner lane's, zeroed in ctm_init
         c->sw.partial_cap = pp;
         c->sw.err = c->err;
+        c->sw.partial_zero = pp > 0;
         c->sw.autotune = 1;   // the first eager call of each contraction shape times its plans
         // the two lanes of the corner / edge updates (see enqueue_step)
         c->sw_c = c->sw;
         c->sw_c.Bpk = (unsigned char *)take(bp);
         c->sw_c.eB = (int *)take(sizeof(int) * (size_t)ecap);
-        c->sw_c.partial = (void *)take(pp + 8);
+        c->sw_c.partial = (char *)c->sw.partial + align_up(pp);
         c->sw_e = c->sw;
         c->sw_e.Apk = (unsigned char *)take(ap);
         c->sw_e.eA = (int *)take(sizeof(int) * (size_t)ecap);
@@ -1016,6 +1017,11 @@ int ctm_init(const ctm_config *cfg, const double *A_dev, void *workspace, size_t
             break;
         }
         if (cudaMemsetAsync(c->err, 0, sizeof(int), st) != cudaSuccess) { rc = CTM_ECUDA; break; }
+        if (c->sw.partial_zero &&
+            cudaMemsetAsync(c->sw.partial, 0, 2 * align_up(c->sw.partial_cap), st) != cudaSuccess) {
+            rc = CTM_ECUDA;
+            break;
+        }
         if (cudaMemcpyAsync(c->Araw, A_dev, sizeof(double) * c->d * c->D * c->D * c->D, cudaMemcpyDeviceToDevice,
                             st) != cudaSuccess) {
             rc = CTM_ECUDA;
@@ -1393,7 +1399,7 @@ int ctm_gemm(int M, int N, int K, const double *A, const double *B, double *C, i
         const int tT = tf32_slices(precision);
         SplitPlan p = tT > 0 ? tf32_plan_caps(M, N, K, tT) : split_plan(M, N, K, n_split);
         int ec = M > N ? M : N;
-        SplitWork w;
+        SplitWork w{};
         w.Apk = (unsigned char *)(base + off);
         off += align_up(p.a_pack_bytes);
         w.a_pack_cap = p.a_pack_bytes;

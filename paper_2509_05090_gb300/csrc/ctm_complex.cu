@@ -1128,6 +1128,7 @@ size_t zlayout(ctm_complex_ctx *c, char *base)
         c->sw.partial_cap = pp;
         c->sw.err = c->err;
         c->sw.autotune = 1;
+        c->sw.partial_zero = pp > 0;   // (zeroed at init)
         c->ta_pk = (unsigned char *)take(ap);
         c->ta_cap = ap;
         c->ta_e = (int *)take(sizeof(int) * (size_t)ecap);
@@ -1560,6 +1561,11 @@ int ctm_complex_init(const ctm_config *cfg, int irrep, const double *A_dev, void
         }
         const long long cnt = c->PA;
         if (cudaMemsetAsync(c->err, 0, sizeof(int), c->stream) != cudaSuccess) { rc = CTM_ECUDA; break; }
+        if (c->sw.partial_zero &&
+            cudaMemsetAsync(c->sw.partial, 0, c->sw.partial_cap, c->stream) != cudaSuccess) {
+            rc = CTM_ECUDA;
+            break;
+        }
         CTM_COUNT_LAUNCH(5);
         zc_load_kernel<<<zgrid(cnt), 256, 0, c->stream>>>(cnt, A_dev, c->Ain, zlay_stacked(cnt, 2));
         zc_project_kernel<<<zgrid(cnt), 256, 0, c->stream>>>(c->d, c->D, c->Ain, cnt, grp, cfg->symmetrize ? 1 : 0,

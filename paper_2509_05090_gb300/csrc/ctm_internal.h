@@ -54,6 +54,7 @@ struct SplitWork {
     int e_cap;
     void *partial;
     size_t partial_cap;
+    int partial_zero;  // the BF16 engine finds the split-K sums zero and leaves them so (zeroed at init)
     int *err;
     int autotune;      // time the candidate tile shapes / K-splits of a new shape once (eager only)
 };
