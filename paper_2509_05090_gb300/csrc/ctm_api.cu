@@ -235,16 +235,17 @@ size_t layout(ctm_ctx *c, char *base)
         c->sw.eA = (int *)take(sizeof(int) * (size_t)ecap);
         c->sw.eB = (int *)take(sizeof(int) * (size_t)ecap);
         c->sw.e_cap = (int)ecap;
-        c->sw.partial = (void *)take(2 * align_up(pp));   // and the corner lane's, zeroed in ctm_init
+        c->sw.partial = (void *)take(pp + 8);
         c->sw.partial_cap = pp;
         c->sw.err = c->err;
-        c->sw.partial_zero = pp > 0;
+        c->sw.zeroed = &c->sw_zeroed[0];
         c->sw.autotune = 1;   // the first eager call of each contraction shape times its plans
         // the two lanes of the corner / edge updates (see enqueue_step)
         c->sw_c = c->sw;
         c->sw_c.Bpk = (unsigned char *)take(bp);
         c->sw_c.eB = (int *)take(sizeof(int) * (size_t)ecap);
-        c->sw_c.partial = (char *)c->sw.partial + align_up(pp);
+        c->sw_c.partial = (void *)take(pp + 8);
+        c->sw_c.zeroed = &c->sw_zeroed[1];
         c->sw_e = c->sw;
         c->sw_e.Apk = (unsigned char *)take(ap);
         c->sw_e.eA = (int *)take(sizeof(int) * (size_t)ecap);
@@ -750,8 +751,7 @@ int graph_launch(ctm_ctx *c, int nsteps)
     return CTM_OK;
 }
 
-// Forget every captured graph (they hold launch arguments and the packed operand
-// state of the moment they were captured); the next calls capture again.
+// Forget every captured graph (they hold launch arguments); the next calls capture again.
 void drop_graphs(ctm_ctx *c)
 {
     if (c->graph) cudaGraphExecDestroy(c->graph);
@@ -1017,11 +1017,6 @@ int ctm_init(const ctm_config *cfg, const double *A_dev, void *workspace, size_t
             break;
         }
         if (cudaMemsetAsync(c->err, 0, sizeof(int), st) != cudaSuccess) { rc = CTM_ECUDA; break; }
-        if (c->sw.partial_zero &&
-            cudaMemsetAsync(c->sw.partial, 0, 2 * align_up(c->sw.partial_cap), st) != cudaSuccess) {
-            rc = CTM_ECUDA;
-            break;
-        }
         if (cudaMemcpyAsync(c->Araw, A_dev, sizeof(double) * c->d * c->D * c->D * c->D, cudaMemcpyDeviceToDevice,
                             st) != cudaSuccess) {
             rc = CTM_ECUDA;

@@ -61,6 +61,7 @@ struct ctm_complex_ctx {
     double *norm_part;
     double *rho_part, *rho_raw, *hrot, *eout;
     SplitWork sw;
+    size_t sw_zeroed;   // see SplitWork
     // the packed TA = T a of the step (used by Y1 and H2)
     unsigned char *ta_pk;
     int *ta_e;
@@ -1128,7 +1129,7 @@ size_t zlayout(ctm_complex_ctx *c, char *base)
         c->sw.partial_cap = pp;
         c->sw.err = c->err;
         c->sw.autotune = 1;
-        c->sw.partial_zero = pp > 0;   // (zeroed at init)
+        c->sw.zeroed = &c->sw_zeroed;
         c->ta_pk = (unsigned char *)take(ap);
         c->ta_cap = ap;
         c->ta_e = (int *)take(sizeof(int) * (size_t)ecap);
@@ -1561,11 +1562,6 @@ int ctm_complex_init(const ctm_config *cfg, int irrep, const double *A_dev, void
         }
         const long long cnt = c->PA;
         if (cudaMemsetAsync(c->err, 0, sizeof(int), c->stream) != cudaSuccess) { rc = CTM_ECUDA; break; }
-        if (c->sw.partial_zero &&
-            cudaMemsetAsync(c->sw.partial, 0, c->sw.partial_cap, c->stream) != cudaSuccess) {
-            rc = CTM_ECUDA;
-            break;
-        }
         CTM_COUNT_LAUNCH(5);
         zc_load_kernel<<<zgrid(cnt), 256, 0, c->stream>>>(cnt, A_dev, c->Ain, zlay_stacked(cnt, 2));
         zc_project_kernel<<<zgrid(cnt), 256, 0, c->stream>>>(c->d, c->D, c->Ain, cnt, grp, cfg->symmetrize ? 1 : 0,

@@ -41,6 +41,7 @@ struct ctm_ctx {
     SplitWork sw;
     SplitWork sw_c;           // corner lane: M's pack read from sw; own B pack, exponents, split-K buffer
     SplitWork sw_e;           // edge lane: own A pack and exponents; B pack and split-K buffer of sw
+    size_t sw_zeroed[2];      // bytes of the split-K sums of sw / sw_e and of sw_c known to be zero (see SplitWork)
     // the double layer a is a constant B operand of four contractions per step:
     // its packed digit slices are kept (slot 0: a as [(u,l)][z], slot 1: a as [z][(x,y)])
     unsigned char *apk[2];
@@ -157,6 +158,6 @@ int enqueue_enlarged_corner(ctm_ctx *c);
 int enqueue_step(ctm_ctx *c);
 int join_side(ctm_ctx *c);
 int read_status(ctm_ctx *c);
-void drop_graphs(ctm_ctx *c);   // forget captured graphs (launch arguments or packed state changed)
+void drop_graphs(ctm_ctx *c);   // forget captured graphs (launch arguments changed)
 cudaError_t rho_reduce(ctm_ctx *c);   // raw[pB][pA] = sum Y1o G2 (energy contraction)
 }  // namespace ctmi

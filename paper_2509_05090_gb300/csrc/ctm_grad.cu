@@ -368,7 +368,7 @@ size_t grad_layout(const ctm_ctx *c, int k, GradBufs *g, char *base)
     b.sw.e_cap = (int)ecap;
     b.sw.partial = bytes(pp);
     b.sw.partial_cap = pp;
-    b.sw.partial_zero = 0;
+    b.sw.zeroed = nullptr;
     b.sw.err = c->err;
     b.sw.autotune = 1;
     if (g) *g = b;

@@ -54,7 +54,7 @@ struct SplitWork {
     int e_cap;
     void *partial;
     size_t partial_cap;
-    int partial_zero;  // the BF16 engine finds the split-K sums zero and leaves them so (zeroed at init)
+    size_t *zeroed;    // the BF16 engine keeps the first *zeroed bytes of partial zero between calls; null: it does not
     int *err;
     int autotune;      // time the candidate tile shapes / K-splits of a new shape once (eager only)
 };

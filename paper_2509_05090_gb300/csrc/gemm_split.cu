@@ -1460,9 +1460,14 @@ static cudaError_t gemm_split_run(const GemmF64 &g, int T, SplitWork w, cudaStre
         if (e != cudaSuccess) return e;
         if (opt && opt->b_pk) *opt->b_state = p.NT;
     }
-    if (p.ksplit > 1 && !w.partial_zero) {
+    const int clear = w.zeroed != nullptr;
+    if (p.ksplit > 1 && (!clear || *w.zeroed < p.partial_bytes)) {
         e = cudaMemsetAsync(w.partial, 0, p.partial_bytes, st);
         if (e != cudaSuccess) return e;
+        // (a captured memset has not run yet: its graph repeats it)
+        cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+        if (clear && cudaStreamIsCapturing(st, &cs) == cudaSuccess && cs == cudaStreamCaptureStatusNone)
+            *w.zeroed = p.partial_bytes;
     }
     SplitArgs a{g.M,
                 g.N,
@@ -1525,9 +1530,9 @@ static cudaError_t gemm_split_run(const GemmF64 &g, int T, SplitWork w, cudaStre
         long long blocks = (total + 255) / 256, cap = 16LL * device_sm_count();
         if (blocks > cap) blocks = cap;
         CTM_COUNT_LAUNCH(1);
-        if (sp_wide(T)) split_finalize_wide_kernel<<<(int)blocks, 256, 0, st>>>(a, w.partial_zero);
+        if (sp_wide(T)) split_finalize_wide_kernel<<<(int)blocks, 256, 0, st>>>(a, clear);
         else
-            split_finalize_kernel<<<(int)blocks, 256, 0, st>>>(g.M, g.N, T, (unsigned long long *)w.partial, w.partial_zero,
+            split_finalize_kernel<<<(int)blocks, 256, 0, st>>>(g.M, g.N, T, (unsigned long long *)w.partial, clear,
                                                                   w.eA, w.eB, g.C, g.Cm, g.Cn);
         e = cudaGetLastError();
     }
