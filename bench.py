@@ -32,7 +32,7 @@ L2_FLUSH_BYTES = 256 << 20
 # workload (--metrics dram__bytes_read.sum,dram__bytes_write.sum on the launches
 # of one step, plans replayed from the plain run's autotune cache).  Set back to
 # absent whenever the contraction kernel changes.
-NCU_TRAFFIC = {("kh_D6_chi72", "split_bf16", 5): 400.4e6}
+NCU_TRAFFIC = {}
 
 
 def _peaks():
@@ -388,7 +388,8 @@ def time_to_converged(w, precision, n_split, max_steps, corner="qmq", spectrum=F
 
 
 def fp64_step_record(w, steps, fp64_peak):
-    """FP64 steps of workload w (one captured graph of `steps` steps), CUDA-event timed."""
+    """FP64 steps of workload w (one captured graph of `steps` steps), CUDA-event timed.  The fractions of
+    the FP64 pipe exceed 1: the contractions run as BF16 digit slices on the tensor cores."""
     import torch
     from paper_2509_05090_gb300 import binding
     c = binding.CTM(w.site_tensor(), w.chi, precision="fp64")
@@ -567,11 +568,11 @@ def run_complex(args, w):
     peaks, src = _peaks()
     flops = 4.0 * step_gemm_flops(w.chi, w.D2)
     if args.precision == "fp64":
-        fp64_peak = binding.ctm_probe_fp64_peak()
-        ach = flops / (ms / 1e3) / 1e12
-        roofline = {"bound": "alu", "achieved": ach, "peak": fp64_peak, "unit": "TFLOP/s", "frac": ach / fp64_peak,
-                    "traffic": None, "peak_source": "measured live: DFMA throughput probe",
-                    "scope": "whole step (contractions, embedded QR, corner spectrum) against the FP64 pipe"}
+        ach = 36 * (flops - 8.0 * w.chi ** 2 * w.D2 ** 3) / (ms / 1e3) / 1e12
+        roofline = {"bound": "tensor", "achieved": ach, "peak": peaks["bf16_tflops"], "unit": "TFLOP/s",
+                    "frac": ach / peaks["bf16_tflops"], "traffic": None, "peak_source": f"{src} bf16 burst",
+                    "fp64_equivalent_tflops": flops / (ms / 1e3) / 1e12,
+                    "scope": "36 BF16 slice products per FP64 product over the whole step time"}
     else:
         pairs = args.n_split * (args.n_split + 1) // 2
         ach = pairs * flops / (ms / 1e3) / 1e12
@@ -772,12 +773,17 @@ def main():
     prepass_ms = phases["prepass"] / nprof
     flops = step_gemm_flops(w.chi, w.D2)
     if args.precision == "fp64":
-        achieved = flops / (kern_ms / 1e3) / 1e12
-        roofline = {"bound": "alu", "achieved": achieved, "peak": fp64_peak, "unit": "TFLOP/s",
-                    "frac": achieved / fp64_peak, "traffic": None,
-                    "kernel": "gemm_f64_kernel (+ split-K reduce): the step's 11 FP64 contractions",
-                    "peak_source": "measured live: DFMA throughput probe (ctm_probe_fp64_peak); GB300 has no "
-                                   "FP64 tcgen05 kind, so the DFMA pipe is the FP64 ceiling"}
+        # 36 slice products per FP64 product; the FP64 step shares T a between the corner and the
+        # edge, one product of chi^2 D2^3 less than the algorithm's count
+        achieved = 36 * (flops - 2.0 * w.chi ** 2 * w.D2 ** 3) / (kern_ms / 1e3) / 1e12
+        peak = peaks["bf16_tflops"]
+        roofline = {"bound": "tensor", "achieved": achieved, "peak": peak, "unit": "TFLOP/s", "frac": achieved / peak,
+                    "traffic": None,
+                    "kernel": "gemm_split_kernel: 36 BF16 slice products (T=8, 62-bit grids) per FP64 contraction, "
+                              "tcgen05 kind::f16 into TMEM (below 8e6 multiply-adds: gemm_f64_kernel)",
+                    "peak_source": f"{src} bf16 burst",
+                    "fp64_equivalent_tflops": flops / (kern_ms / 1e3) / 1e12,
+                    "fp64_equivalent_over_fp64_pipe": flops / (kern_ms / 1e3) / 1e12 / fp64_peak}
     elif args.precision in ("split_tf32", "fp32_tf32"):
         # TF32 products on the tensor pipe: 3 (A_hi B_hi + A_hi B_lo + A_lo B_hi) or 1 per
         # contraction; the TF32 peak is the measured BF16 burst times the nominal dense ratio

@@ -55,7 +55,9 @@ typedef enum {
 } ctm_status;
 
 typedef enum {
-    CTM_FP64 = 0,            /* every contraction in FP64 */
+    CTM_FP64 = 0,            /* every contraction to FP64 accuracy: as exact products of eight
+                                BF16 digit slices on tcgen05 (62-bit grids, one rounding of the
+                                result) where the shape gains from it, else on the FP64 pipe */
     CTM_SPLIT_BF16 = 1,      /* contractions as split-BF16 tcgen05 products (FP32 accumulate,
                                 FP64 recombination); QR, normalisation and the
                                 convergence test stay FP64 */
@@ -209,8 +211,8 @@ int ctm_transfer_spectrum(ctm_ctx *ctx, int nev, int max_iter, double tol, void 
  * normalised under the context's symmetrize setting and its double layer formed;
  * the environment is kept as the warm start of the next steps (reset_env = 0) or
  * reset to the initial environment of ctm_init (reset_env != 0).  Captured step
- * graphs are dropped and captured again on the next call.  CTM_ENONFINITE if the
- * tensor holds NaN/Inf.  Synchronous. */
+ * graphs stay valid (kept packs of the double layer are rewritten in place).
+ * CTM_ENONFINITE if the tensor holds NaN/Inf.  Synchronous. */
 int ctm_set_site(ctm_ctx *ctx, const double *A_dev, int reset_env);
 
 /* Copy the current environment out / in (device pointers; parity checks and
@@ -237,11 +239,11 @@ int ctm_get_intermediate(const ctm_ctx *ctx, int which, double *dst_dev, size_t 
  * summed time of the contraction-engine kernels alone (events around each
  * launch: the FP64 GEMM with its split-K reduction, or the tcgen05 kernel
  * without its operand pre-pass), and (nphase >= 10) [9] the summed time of the
- * split engine's operand pre-pass (exponents and digit packing; 0 in FP64). */
+ * split engine's operand pre-pass (exponents and digit packing). */
 int ctm_step_profiled(ctm_ctx *ctx, double *phase_ms, int nphase);
 
-/* Measured FP64 peak of the device (no counterpart in the paper; the roofline
- * denominator of the FP64 contractions): a grid of 4 CTAs per SM, each thread
+/* Measured FP64 peak of the device (no counterpart in the paper; what the QR, the
+ * corner spectrum and the small FP64 contractions run against): a grid of 4 CTAs per SM, each thread
  * running 16 independent chains of dependent DFMAs, timed with CUDA events after a
  * warm-up launch.  *tflops_host receives 2 x DFMAs / second / 1e12.  Synchronous
  * on `stream`. */
