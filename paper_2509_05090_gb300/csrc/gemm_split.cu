@@ -31,9 +31,9 @@
 // K 2^-53 sum |a b|.  Measured against 128-bit sums (2-norm over the output): 3e-17 to 6e-17
 // at every shape and for normal, uniform, graded and constant operands, the FP64 GEMM 1e-16
 // to 2e-15.  Rows and columns with infinities or NaNs have no grid; their outputs are the
-// plain FP64 sums.  Against the FP64 pipe's GEMM: 8192 x 8192 x 128 14.09 -> 0.89 ms,
-// 8192 x 128 x 8192 14.30 -> 0.96 ms, 2592 x 2592 x 72 849 -> 107 us, 2592 x 72 x 2592
-// 935 -> 135 us, 900 x 900 x 36 72 -> 29 us; below MNK = 8e6 (512 x 512 x 32: 28 against
+// plain FP64 sums.  Against the FP64 pipe's GEMM (kernels; the packs take 5 to
+// 320 us more): 8192 x 8192 x 128 14.09 -> 0.82 ms, 8192 x 128 x 8192 14.30 -> 0.56 ms, 2592 x 2592 x 72
+// 849 -> 86 us, 2592 x 72 x 2592 935 -> 80 us, 900 x 900 x 36 72 -> 18 us; below MNK = 8e6 (512 x 512 x 32: 28 against
 // 26 us, 512 x 32 x 512: 33 against 38, 243 x 243 x 27: 11 against 26) the two packs and three
 // launches cost more than the FP64 GEMM, which keeps those shapes (split_f64_pays).
 //
@@ -58,7 +58,7 @@
 // add, since every FP64 instruction, conversions and compares included, holds its
 // sub-partition's FP64 pipe for 64 cycles.  T = 5: 2592 x 2592 x 72 58.9 -> 49.9 us, 5184 x 1296 x 36
 // 52.7 -> 42.7, 512 x 512 x 32 15.0 -> 11.8; T = 8: 2592 x 2592 x 72 131 -> 86, 8192 x 8192 x 128
-// 1077 -> 889.  At large K the K loop is all (2592 x 72 x 2592, T = 8: 88 % of a CTA's time).
+// 1077 -> 821.  At large K the K loop is all (2592 x 72 x 2592, T = 8: 88 % of a CTA's time).
 #include <cuda_bf16.h>
 
 #include <vector>

@@ -751,7 +751,7 @@ __global__ void bisect_kernel(int chi, const double *work, double *lam)
         hi = (double)fhi + 0x1p-19;
     }
     const double width = BISECT_WIDTH * sc * sqrt(f2);
-    bool ends = true;       // this round checks the bracket's own ends
+    bool ends = true;       // this pass checks the bracket's own ends
     bool even = true;       // evenly spaced points
     double r = 0.0;         // secant estimate, when !even
     for (int round = 0; round < 40 && hi - lo > width; ++round) {
